@@ -133,12 +133,11 @@ kc_status kc_lower_bounds(kc_ctx *ctx, const void *lo, const void *hi, int32_t B
  * nothing).  If a CUDA error is already pending in the calling thread the
  * call returns KC_ECUDA at once, launches nothing and leaves that error in
  * place for its owner.
- * Scratch is one fixed array in the library (512 partial results for each of
- * 256 nodes, 1 MiB, kept by every GPU that loads the library until the
- * process exits); nodes are processed 256 at a time and B may be at most
- * 4096 (larger B returns KC_EINVAL).  The first call on a device looks up the
- * array's device address with that device current and keeps it for the
- * process; make that first call before any stream capture, and do not call
+ * Scratch is one fixed array in the library (the best value of each of 4096
+ * nodes, 32 KiB, kept by every GPU that loads the library until the process
+ * exits); B may be at most 4096 (larger B returns KC_EINVAL).  The first call on
+ * a device looks up the array's device address with that device current and
+ * keeps it for the process; make that first call before any stream capture, and do not call
  * the entry point on a device after cudaDeviceReset (the kept address would
  * be stale).  Every call reuses the same array, so calls that can overlap on
  * the GPU (different streams, no ordering between them) race and must not be
@@ -151,7 +150,7 @@ kc_status kc_lower_bounds_noalloc(const float *X, int64_t N, int64_t ld, int32_t
 
 /*
  * kc_autotune -- picks the launch shape of the float lower-bound kernel
- * (samples per thread, nodes per launch: occupancy against extra passes over
+ * (samples per thread, nodes per CTA: occupancy against extra passes over
  * the samples) by timing each candidate with CUDA events on the given batch
  * of B nodes (lo, hi as in kc_lower_bounds), and keeps the fastest for later
  * kc_lower_bounds calls on this context.  Outputs (host, each may be NULL):

@@ -114,7 +114,7 @@ void kc_destroy(kc_ctx *ctx)
 {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->stream);
-    for (DevBuf *b : {&ctx->part, &ctx->stage_in, &ctx->stage_out, &ctx->work})
+    for (DevBuf *b : {&ctx->part, &ctx->keys, &ctx->stage_in, &ctx->stage_out, &ctx->work, &ctx->vs.buf, &ctx->vs.jbuf})
         if (b->p) cudaFree(b->p);
     if (ctx->X) cudaFree(ctx->X);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);

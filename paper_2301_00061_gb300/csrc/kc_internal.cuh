@@ -54,6 +54,7 @@ struct kc_ctx {
     void *X = nullptr;           // [D][ldx] owned device copy
     // scratch
     kc::DevBuf part;             // per-CTA partial results
+    kc::DevBuf keys;             // best key per node of the float bound, zero between calls
     kc::DevBuf stage_in;         // staged host inputs
     kc::DevBuf stage_out;        // device-side outputs destined for host
     kc::DevBuf work;             // per-call work arrays
@@ -64,8 +65,8 @@ struct kc_ctx {
     int64_t launches = 0;
     std::string err;
     // launch shape of the float lower-bound kernel, set by kc_autotune (kc_lb.cu)
-    int lb_st = 0;               // samples per thread of the float lower-bound kernel
-    int lb_chunk = 0;            // node chunk of the float lower-bound kernel (0: largest that fits)
+    int lb_st = 0;               // samples per thread of the float lower-bound kernel, 4 or 2 (0: by size)
+    int lb_chunk = 0;            // nodes per CTA of the float lower-bound kernel (0: as many as fit)
 };
 
 namespace kc {

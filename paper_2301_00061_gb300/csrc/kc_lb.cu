@@ -1,225 +1,23 @@
 // kc_lb.cu -- node lower bound beta(M) = max_s min_k beta_s^k(M^k)
 // (Section 3.1, Eqs. 9-11 with the closed-form minimiser mid{lo, x, hi}).
 //
-// One persistent launch evaluates a batch of B nodes: the node boxes are staged
-// once per CTA in shared memory, every sample is read from HBM once per batch
-// (coalesced 64/128-bit loads of the attribute-major copy), and each thread
-// keeps ST samples in registers while it sweeps all B nodes.  The max over
-// samples is tracked per warp in shared memory as a packed (value, position)
-// key; a warp only reduces with shuffles when one of its lanes beats the
-// warp's running best.  One partial per CTA and node goes to global scratch
-// and a second small kernel reduces them (deterministic: the largest value,
-// the smallest position on ties).
+// Float data: batches of nodes take the pruning kernel (kc_prune.cuh), few
+// nodes the streaming kernel (kc_stream.cu); both raise one (value, position)
+// key per node with 64-bit atomics (the largest value, the smallest position
+// on ties), which a small second kernel turns into the outputs.  Double data:
+// every thread sweeps the batch's nodes for one sample in the serial order of
+// operations, and per-CTA partials are reduced by a second kernel.
 #include <cuda_runtime.h>
 
 #include <atomic>
 
 #include "kc_device.cuh"
 #include "kc_internal.cuh"
+#include "kc_prune.cuh"
 
 namespace kc {
 
 namespace {
-
-template <int ST>
-__device__ __forceinline__ void load_row(const float *__restrict__ p, float (&v)[ST])
-{
-    if constexpr (ST == 4) {
-        const float4 q = __ldg(reinterpret_cast<const float4 *>(p));
-        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
-    } else if constexpr (ST == 2) {
-        const float2 q = __ldg(reinterpret_cast<const float2 *>(p));
-        v[0] = q.x; v[1] = q.y;
-    } else {
-        v[0] = __ldg(p);
-    }
-}
-
-// D packed (lo, -hi) pairs of one box from shared memory into registers.
-template <int D>
-__device__ __forceinline__ void load_box(const uint64_t *p, uint64_t (&bx)[D])
-{
-    if constexpr ((D % 2) == 0) {
-#pragma unroll
-        for (int a = 0; a < D; a += 2) {
-            const ulonglong2 q = *reinterpret_cast<const ulonglong2 *>(p + a);
-            bx[a] = q.x;
-            bx[a + 1] = q.y;
-        }
-    } else {
-#pragma unroll
-        for (int a = 0; a < D; ++a) bx[a] = p[a];
-    }
-}
-
-// Every node's running maximum over one thread's ST samples px (packed
-// (x, -x) per attribute; when not `full`, samples s0 + j >= n are ignored),
-// merged into the warp's keys mine[b] (value bits, ~position): a warp
-// reduces with shuffles only when one of its lanes may beat the warp's best.
-template <int D, int K, int ST>
-__device__ __forceinline__ void eval_nodes(const uint64_t (&px)[ST][D], bool full, int64_t s0, int64_t n,
-                                           const uint64_t *sbox, int B, unsigned long long *mine, int lane)
-{
-    constexpr int KD = K * D;
-    for (int b = 0; b < B; ++b) {
-        const uint64_t *bb = sbox + (size_t)b * KD;
-        float best[ST];
-#pragma unroll
-        for (int j = 0; j < ST; ++j) best[j] = __int_as_float(0x7f800000);
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            uint64_t bx[D];
-            load_box<D>(bb + k * D, bx);
-#pragma unroll
-            for (int j = 0; j < ST; ++j) best[j] = fminf(best[j], box_dist_f32<D>(px[j], bx));
-        }
-        if (!full) {
-#pragma unroll
-            for (int j = 0; j < ST; ++j)
-                if (s0 + j >= n) best[j] = -1.f;
-        }
-        float m = best[0];
-#pragma unroll
-        for (int j = 1; j < ST; ++j) m = fmaxf(m, best[j]);
-        const unsigned long long cur = mine[b];
-        const bool maybe = m >= key_val(cur);
-        if (__any_sync(0xffffffffu, maybe)) {
-            unsigned long long key = 0ull;
-            if (maybe) {
-                int jm = 0;
-#pragma unroll
-                for (int j = ST - 1; j >= 0; --j)
-                    if (best[j] == m) jm = j;
-                key = key_max(m, (uint32_t)(s0 + jm));
-            }
-            key = warp_max_u64(key);
-            if (lane == 0 && key > cur) mine[b] = key;
-            __syncwarp();
-        }
-    }
-}
-
-// Float lower bound, compile-time D and K.  Shared memory: B*K*D packed
-// boxes + (warps x B) running-best keys.
-template <int D, int K, int ST>
-__global__ void __launch_bounds__(kThreads, 2)
-lb_f32_fast(const float *__restrict__ X, int64_t ld, int64_t n, const float *__restrict__ lo,
-            const float *__restrict__ hi, int B, unsigned long long *__restrict__ part)
-{
-    constexpr int KD = K * D;
-    constexpr int NW = kThreads / 32;
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sbox = reinterpret_cast<uint64_t *>(smem);
-    unsigned long long *wbest = reinterpret_cast<unsigned long long *>(sbox + (size_t)B * KD);
-    for (int i = threadIdx.x; i < B * KD; i += kThreads) sbox[i] = pk(lo[i], -hi[i]);
-    for (int i = threadIdx.x; i < NW * B; i += kThreads) wbest[i] = 0ull;
-    __syncthreads();
-
-    const int lane = threadIdx.x & 31;
-    unsigned long long *mine = wbest + (threadIdx.x >> 5) * B;
-    const int64_t tile = (int64_t)kThreads * ST;
-    for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
-        const int64_t s0 = base + (int64_t)threadIdx.x * ST;
-        const bool full = s0 + ST <= n;
-        uint64_t px[ST][D];
-        if (full) {
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                float v[ST];
-                load_row<ST>(X + (size_t)a * ld + s0, v);
-#pragma unroll
-                for (int j = 0; j < ST; ++j) px[j][a] = pk(v[j], -v[j]);
-            }
-        } else {
-#pragma unroll
-            for (int a = 0; a < D; ++a)
-#pragma unroll
-                for (int j = 0; j < ST; ++j) {
-                    const float v = (s0 + j < n) ? X[(size_t)a * ld + s0 + j] : 0.f;
-                    px[j][a] = pk(v, -v);
-                }
-        }
-        eval_nodes<D, K, ST>(px, full, s0, n, sbox, B, mine, lane);
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < B; b += kThreads) {
-        unsigned long long m = 0ull;
-        for (int w = 0; w < NW; ++w) {
-            const unsigned long long v = wbest[w * B + b];
-            m = v > m ? v : m;
-        }
-        part[(size_t)blockIdx.x * B + b] = m;
-    }
-}
-
-// Float lower bound for any D <= DMAX and K (runtime).  Boxes are staged with
-// D padded to an even count by (0, -0) pairs, which add exactly zero.
-template <int DMAX>
-__global__ void __launch_bounds__(kThreads)
-lb_f32_generic(const float *__restrict__ X, int64_t ld, int64_t n, const float *__restrict__ lo,
-               const float *__restrict__ hi, int B, int K, int D, unsigned long long *__restrict__ part)
-{
-    constexpr int NW = kThreads / 32;
-    const int Dp = (D + 1) & ~1;
-    extern __shared__ __align__(16) unsigned char smem[];
-    uint64_t *sbox = reinterpret_cast<uint64_t *>(smem);                        // [B][K][Dp]
-    unsigned long long *wbest = reinterpret_cast<unsigned long long *>(sbox + (size_t)B * K * Dp);
-    for (int i = threadIdx.x; i < B * K * Dp; i += kThreads) {
-        const int a = i % Dp, bk = i / Dp;
-        sbox[i] = a < D ? pk(lo[(size_t)bk * D + a], -hi[(size_t)bk * D + a]) : pk(0.f, -0.f);
-    }
-    for (int i = threadIdx.x; i < NW * B; i += kThreads) wbest[i] = 0ull;
-    __syncthreads();
-
-    const int lane = threadIdx.x & 31;
-    unsigned long long *mine = wbest + (threadIdx.x >> 5) * B;
-    for (int64_t s = (int64_t)blockIdx.x * kThreads + threadIdx.x; s - threadIdx.x < n;
-         s += (int64_t)gridDim.x * kThreads) {
-        const bool valid = s < n;
-        uint64_t px[DMAX];
-#pragma unroll
-        for (int a = 0; a < DMAX; ++a) {
-            const float v = (valid && a < D) ? X[(size_t)a * ld + s] : 0.f;
-            px[a] = pk(v, -v);
-        }
-        for (int b = 0; b < B; ++b) {
-            float best = __int_as_float(0x7f800000);
-            for (int k = 0; k < K; ++k) {
-                const uint64_t *bx = sbox + ((size_t)b * K + k) * Dp;
-                uint64_t acc = 0;
-#pragma unroll
-                for (int a = 0; a < DMAX; a += 2) {
-                    if (a < Dp) {
-                        const float2 t0 = upk(sub2(bx[a], px[a]));
-                        const float2 t1 = upk(sub2(bx[a + 1], px[a + 1]));
-                        const uint64_t m = pk(max3f(t0.x, t0.y, 0.f), max3f(t1.x, t1.y, 0.f));
-                        acc = fma2(m, m, acc);
-                    }
-                }
-                const float2 sacc = upk(acc);
-                best = fminf(best, sacc.x + sacc.y);
-            }
-            const float m = valid ? best : -1.f;
-            const unsigned long long cur = mine[b];
-            const bool maybe = m >= key_val(cur);
-            if (__any_sync(0xffffffffu, maybe)) {
-                unsigned long long key = maybe ? key_max(m, (uint32_t)s) : 0ull;
-                key = warp_max_u64(key);
-                if (lane == 0 && key > cur) mine[b] = key;
-                __syncwarp();
-            }
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < B; b += kThreads) {
-        unsigned long long m = 0ull;
-        for (int w = 0; w < NW; ++w) {
-            const unsigned long long v = wbest[w * B + b];
-            m = v > m ? v : m;
-        }
-        part[(size_t)blockIdx.x * B + b] = m;
-    }
-}
 
 // Double lower bound: mid{lo, x, hi}, d = x - mid, acc = acc + d*d in attribute
 // order with separate roundings -- the serial evaluation, bit for bit.
@@ -397,28 +195,22 @@ lb_refine_f32(const float *__restrict__ X, int64_t ld, int64_t n, const float *_
     }
 }
 
-__global__ void lb_finalize_f32(const unsigned long long *__restrict__ part, int nparts, int B,
-                                const uint32_t *__restrict__ ids, double defl, double slack,
-                                double *__restrict__ lb, double *__restrict__ lb_raw,
+// Keys (value bits, ~position) -> certified bound, value and sample per node.
+// The keys go back to zero, as the next launch wants them.
+__global__ void lb_finalize_f32(unsigned long long *__restrict__ keys, int B, const uint32_t *__restrict__ ids,
+                                double defl, double slack, double *__restrict__ lb, double *__restrict__ lb_raw,
                                 int64_t *__restrict__ arg)
 {
-    const int b = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
+    const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    unsigned long long m = 0ull;
-    for (int p = lane; p < nparts; p += 32) {
-        const unsigned long long v = part[(size_t)p * B + b];
-        m = v > m ? v : m;
-    }
-    m = warp_max_u64(m);
-    if (lane == 0) {
-        const double raw = m ? (double)key_val(m) : 0.0;
-        if (lb_raw) lb_raw[b] = raw;
-        if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(raw, defl), slack));
-        if (arg) {
-            const int64_t pos = m ? (int64_t)key_pos(m) : -1;
-            arg[b] = (pos < 0 || !ids) ? pos : (int64_t)ids[pos];
-        }
+    const unsigned long long m = keys[b];
+    keys[b] = 0ull;
+    const double raw = m ? (double)key_val(m) : 0.0;
+    if (lb_raw) lb_raw[b] = raw;
+    if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(raw, defl), slack));
+    if (arg) {
+        const int64_t pos = m ? (int64_t)key_pos(m) : -1;
+        arg[b] = (pos < 0 || !ids) ? pos : (int64_t)ids[pos];
     }
 }
 
@@ -454,23 +246,72 @@ __global__ void lb_finalize_f64(const double *__restrict__ pval, const uint32_t 
 
 // ---------------------------------------------------------------- dispatch
 
-using FastFn = void (*)(const float *, int64_t, int64_t, const float *, const float *, int,
-                        unsigned long long *);
-
-struct FastEntry {
-    int D, K, ST;
-    FastFn fn;
+// Attribute pairs with a compiled kernel; other D take the next larger one
+// (padding pairs add exactly zero).
+using PruneFn = void (*)(const PruneArgs);
+struct PruneEntry {
+    int P, ST, T, NT;
+    PruneFn fn;
 };
-
-// Shapes of the measured workloads get compile-time kernels; others use the
-// generic ones.
-const FastEntry kFast[] = {
-    {2, 3, 4, lb_f32_fast<2, 3, 4>}, {2, 3, 2, lb_f32_fast<2, 3, 2>},
-    {2, 4, 4, lb_f32_fast<2, 4, 4>}, {2, 4, 2, lb_f32_fast<2, 4, 2>},
-    {3, 3, 4, lb_f32_fast<3, 3, 4>}, {3, 3, 2, lb_f32_fast<3, 3, 2>},
-    {4, 3, 4, lb_f32_fast<4, 3, 4>}, {4, 3, 2, lb_f32_fast<4, 3, 2>},
-    {8, 5, 4, lb_f32_fast<8, 5, 4>}, {8, 5, 2, lb_f32_fast<8, 5, 2>},
+template <int P, int ST = PruneShape<P>::ST>
+PruneEntry prune_entry()
+{
+    constexpr int NT = PruneShape<P>::NT, T = NT * ST;
+    return PruneEntry{P, ST, T, NT, prune_max_kernel<P, ST, NT>};
+}
+const PruneEntry kPrune[] = {
+    prune_entry<1>(), prune_entry<1, 2>(), prune_entry<2>(), prune_entry<2, 2>(), prune_entry<3>(),
+    prune_entry<3, 2>(), prune_entry<4>(), prune_entry<4, 2>(), prune_entry<6>(), prune_entry<8>(),
+    prune_entry<12>(), prune_entry<16>(), prune_entry<24>(), prune_entry<34>(), prune_entry<48>(), prune_entry<64>(),
 };
+// Launches the float maxima of A.B nodes into A.keys (zeroed by the caller) on
+// `stream`; st (samples per thread: 4 or 2, where both exist) and chunk (nodes
+// per CTA) of 0 are chosen here.
+cudaError_t launch_max_f32(PruneArgs A, int sms, size_t smem_cap, int st, int chunk, cudaStream_t stream)
+{
+    const int P = (A.D + 1) / 2;
+    A.vec = (uintptr_t)A.X % 16 == 0 && A.ld % 4 == 0;
+    if (use_stream_f32(A.B, A.K, A.D)) return launch_stream_f32(A, sms, stream);
+    const PruneEntry *e = kPrune;
+    while (e->P < P) ++e;
+    if (P <= 4) {
+        // two entries: 4 and 2 samples per thread
+        const int64_t t4 = (A.n + e->T - 1) / e->T;
+        if (st == 2 || (st != 4 && t4 < 8 * (int64_t)sms)) ++e;
+    }
+    const int64_t tiles = (A.n + e->T - 1) / e->T;
+    const auto fits = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32).end <= smem_cap; };
+    int per = A.B;
+    if (chunk > 0 && chunk < per) per = chunk;
+    if (tiles < sms) {
+        // few tiles: spread the nodes over the SMs as well, whole groups to a CTA
+        const int64_t want = std::max<int64_t>(1, sms / tiles);
+        per = (int)std::min<int64_t>(per, ((A.B + want - 1) / want + kPG - 1) / kPG * kPG);
+    }
+    while (per > 1 && !fits(per)) per = per > 2 * kPG ? (per - 1) / kPG * kPG : per - 1;
+    A.per = per;
+    const size_t smem = PruneLayout(per, A.K, e->P, e->T, e->NT / 32).end;
+    if (smem > smem_cap) return cudaErrorInvalidConfiguration;
+    if (smem > 48 * 1024) {
+        const cudaError_t r = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (r != cudaSuccess) return r;
+    }
+    // at most 65535 node ranges to a launch
+    const int B = A.B, step = (int)std::min<int64_t>((int64_t)per * 65535, B);
+    const size_t box = (size_t)A.K * A.D * 4;
+    for (int b0 = 0; b0 < B; b0 += step) {
+        PruneArgs C = A;
+        C.B = std::min(step, B - b0);
+        C.lo = static_cast<const char *>(A.lo) + b0 * box;
+        C.hi = static_cast<const char *>(A.hi) + b0 * box;
+        C.keys = A.keys + b0;
+        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, sms)), (unsigned)((C.B + per - 1) / per));
+        e->fn<<<grid, e->NT, smem, stream>>>(C);
+        const cudaError_t r = cudaGetLastError();
+        if (r != cudaSuccess) return r;
+    }
+    return cudaSuccess;
+}
 
 template <typename F>
 kc_status prep_kernel(kc_ctx *c, F fn, size_t smem, int *grid, int64_t tiles)
@@ -503,47 +344,27 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
     const size_t smem_cap = c->smem_optin > 0 ? c->smem_optin : 48 * 1024;
     const int NW = kThreads / 32;
     if (c->dt == KC_F32) {
-        const FastFn *fast = nullptr;
-        int st = st_override > 0 ? st_override : (c->lb_st > 0 ? c->lb_st : 4);
-        for (const auto &e : kFast)
-            if (e.D == D && e.K == K && e.ST == st) fast = &e.fn;
-        const int Dp = fast ? D : ((D + 1) & ~1);
-        const size_t per_node = (size_t)K * Dp * 8 + NW * 8;
-        // chunk the node batch so two CTAs fit per SM where possible
-        int chunk = (int)std::min<size_t>((size_t)B, (smem_cap / 2 > per_node ? (smem_cap / 2) / per_node : 1));
-        const int chunk_pref = chunk_override > 0 ? chunk_override : c->lb_chunk;
-        if (chunk_pref > 0 && chunk_pref < chunk) chunk = chunk_pref;
-        if (chunk < 1) chunk = 1;
-        for (int b0 = 0; b0 < B; b0 += chunk) {
-            const int nb = std::min(chunk, B - b0);
-            const size_t smem = per_node * nb;
-            const float *l = static_cast<const float *>(lo) + (size_t)b0 * K * D;
-            const float *h = static_cast<const float *>(hi) + (size_t)b0 * K * D;
-            int grid = 1;
-            if (fast) {
-                const int64_t tiles = (v.n + (int64_t)kThreads * st - 1) / ((int64_t)kThreads * st);
-                KC_TRY(prep_kernel(c, *fast, smem, &grid, tiles));
-                KC_TRY(ensure(c, c->part, (size_t)grid * nb * 8));
-                if (v.n > 0)
-                    (*fast)<<<grid, kThreads, smem, c->stream>>>(
-                        static_cast<const float *>(v.X), v.ld, v.n, l, h, nb,
-                        static_cast<unsigned long long *>(c->part.p));
-            } else {
-                const int64_t tiles = (v.n + kThreads - 1) / kThreads;
-                auto g = D <= 16 ? lb_f32_generic<16> : (D <= 64 ? lb_f32_generic<64> : lb_f32_generic<128>);
-                KC_TRY(prep_kernel(c, g, smem, &grid, tiles));
-                KC_TRY(ensure(c, c->part, (size_t)grid * nb * 8));
-                if (v.n > 0)
-                    g<<<grid, kThreads, smem, c->stream>>>(static_cast<const float *>(v.X), v.ld, v.n, l, h, nb, K, D,
-                                                           static_cast<unsigned long long *>(c->part.p));
-            }
-            if (v.n > 0) KC_TRY(after_launch(c, "lower bound"));
-            const int nparts = v.n > 0 ? grid : 0;
-            lb_finalize_f32<<<(nb + 3) / 4, 128, 0, c->stream>>>(
-                static_cast<const unsigned long long *>(c->part.p), nparts, nb, v.ids, defl, slack,
-                lb ? lb + b0 : nullptr, lb_raw ? lb_raw + b0 : nullptr, arg ? arg + b0 : nullptr);
-            KC_TRY(after_launch(c, "lower bound finalize"));
+        if (c->keys.bytes < (size_t)B * 8) {
+            KC_TRY(ensure(c, c->keys, (size_t)B * 8));
+            KC_CUDA(c, cudaMemsetAsync(c->keys.p, 0, c->keys.bytes, c->stream));
         }
+        PruneArgs A{};
+        A.X = v.X;
+        A.ld = v.ld;
+        A.n = v.n;
+        A.lo = lo;
+        A.hi = hi;
+        A.B = B;
+        A.K = K;
+        A.D = D;
+        A.keys = static_cast<unsigned long long *>(c->keys.p);
+        if (v.n > 0) {
+            KC_CUDA(c, launch_max_f32(A, c->num_sms, smem_cap, st_override > 0 ? st_override : c->lb_st,
+                                      chunk_override > 0 ? chunk_override : c->lb_chunk, c->stream));
+            ++c->launches;
+        }
+        lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B, v.ids, defl, slack, lb, lb_raw, arg);
+        KC_TRY(after_launch(c, "lower bound finalize"));
     } else {
         const size_t per_node = (size_t)K * D * 16 + NW * 12;
         int chunk = (int)std::min<size_t>((size_t)B, (smem_cap / 2 > per_node ? (smem_cap / 2) / per_node : 1));
@@ -632,7 +453,7 @@ kc_status launch_lower_bounds_refine(kc_ctx *c, const View &v, const void *lo, c
 }
 
 // Times the float lower-bound kernel's launch shapes on the given node batch
-// (samples per thread x node chunk: occupancy against extra sample passes)
+// (samples per thread x nodes per CTA: occupancy against extra sample passes)
 // and keeps the fastest in the context.  Untimed work for the caller.
 kc_status autotune_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B, double *lb_scratch, int *st_out,
                                 int *chunk_out, float *ms_out)
@@ -679,21 +500,19 @@ kc_status autotune_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B
 }  // namespace kc
 
 // ------------------------------------------------------------------------
-// kc_lower_bounds_noalloc: the float lower-bound kernel with its per-CTA
-// partial results in a fixed device array instead of a context's buffers.
+// kc_lower_bounds_noalloc: the float lower-bound kernels with their keys in a
+// fixed device array instead of a context's buffers.
 // Nothing here allocates; see include/kc.h for who needs this.
 
 namespace kc {
 namespace {
 
-constexpr int kNoAllocMaxCtas = 512;      // partial slots per node
-constexpr int kNoAllocChunk = 256;        // nodes per launch
 constexpr int kNoAllocMaxNodes = 4096;    // nodes per call
 constexpr int kNoAllocMaxDevices = 64;
 
-// One CTA's best key per node of the current chunk: 512 x 256 x 8 bytes = 1 MiB,
-// held by every GPU that loads the library until the process exits.
-static __device__ __align__(256) unsigned long long g_noalloc_partials[kNoAllocMaxCtas * kNoAllocChunk];
+// The best key of each node of a call, zero between calls: 32 KiB, held by every
+// GPU that loads the library until the process exits.
+static __device__ __align__(256) unsigned long long g_noalloc_keys[kNoAllocMaxNodes];
 
 std::atomic<void *> g_noalloc_ptr[kNoAllocMaxDevices];
 
@@ -735,59 +554,26 @@ extern "C" kc_status kc_lower_bounds_noalloc(const float *X, int64_t N, int64_t 
     // the address up once per device, with that device current.
     void *scratch = g_noalloc_ptr[dev].load();
     if (!scratch) {
-        if (cudaGetSymbolAddress(&scratch, g_noalloc_partials) != cudaSuccess || !scratch) return KC_ECUDA;
+        if (cudaGetSymbolAddress(&scratch, g_noalloc_keys) != cudaSuccess || !scratch) return KC_ECUDA;
         g_noalloc_ptr[dev].store(scratch);
     }
     int sms = 0, optin = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return KC_ECUDA;
-    const int NW = kThreads / 32;
     const double defl = deflate_factor(KC_F32, D), slack = underflow_slack(KC_F32, D);
-    const bool aligned = ((uintptr_t)X % 16 == 0) && (ld % 4 == 0);
-    FastFn fast = nullptr;
-    for (const auto &e : kFast)
-        if (aligned && e.D == D && e.K == K && e.ST == 4) fast = e.fn;
-    const int Dp = fast ? D : ((D + 1) & ~1);
-    const size_t per_node = (size_t)K * Dp * 8 + NW * 8;
-    int chunk = (int)std::min<size_t>(kNoAllocChunk, (size_t)optin / per_node);
-    if (chunk < 1) return KC_EINVAL;
-    unsigned long long *part = static_cast<unsigned long long *>(scratch);
-    for (int b0 = 0; b0 < B; b0 += chunk) {
-        const int nb = std::min(chunk, B - b0);
-        const size_t smem = per_node * nb;
-        const float *l = lo + (size_t)b0 * K * D, *h = hi + (size_t)b0 * K * D;
-        int per_sm = 0, grid = 1;
-        if (fast) {
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(fast, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return KC_ECUDA;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fast, kThreads, smem) != cudaSuccess)
-                return KC_ECUDA;
-        } else {
-            auto g = D <= 16 ? lb_f32_generic<16> : (D <= 64 ? lb_f32_generic<64> : lb_f32_generic<128>);
-            if (smem > 48 * 1024 &&
-                cudaFuncSetAttribute(g, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-                return KC_ECUDA;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, g, kThreads, smem) != cudaSuccess)
-                return KC_ECUDA;
-        }
-        if (per_sm < 1) return KC_EINVAL;
-        const int64_t tile = (int64_t)kThreads * (fast ? 4 : 1);
-        const int64_t tiles = (N + tile - 1) / tile;
-        grid = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)per_sm * sms, tiles, (int64_t)kNoAllocMaxCtas}));
-        if (N > 0) {
-            if (fast)
-                fast<<<grid, kThreads, smem, st>>>(X, ld, N, l, h, nb, part);
-            else
-                (D <= 16 ? lb_f32_generic<16> : (D <= 64 ? lb_f32_generic<64> : lb_f32_generic<128>))
-                    <<<grid, kThreads, smem, st>>>(X, ld, N, l, h, nb, K, D, part);
-            if (cudaGetLastError() != cudaSuccess) return KC_ECUDA;
-        }
-        lb_finalize_f32<<<(nb + 3) / 4, 128, 0, st>>>(part, N > 0 ? grid : 0, nb, nullptr, defl, slack, lb_out + b0,
-                                                      lb_raw_out ? lb_raw_out + b0 : nullptr,
-                                                      argmax_out ? argmax_out + b0 : nullptr);
-        if (cudaGetLastError() != cudaSuccess) return KC_ECUDA;
-    }
+    PruneArgs A{};
+    A.X = X;
+    A.ld = ld;
+    A.n = N;
+    A.lo = lo;
+    A.hi = hi;
+    A.B = B;
+    A.K = K;
+    A.D = D;
+    A.keys = static_cast<unsigned long long *>(scratch);
+    if (N > 0 && launch_max_f32(A, sms, (size_t)optin, 0, 0, st) != cudaSuccess) return KC_ECUDA;
+    lb_finalize_f32<<<(B + 127) / 128, 128, 0, st>>>(A.keys, B, nullptr, defl, slack, lb_out, lb_raw_out, argmax_out);
+    if (cudaGetLastError() != cudaSuccess) return KC_ECUDA;
     return KC_OK;
 }
