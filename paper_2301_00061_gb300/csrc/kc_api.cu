@@ -114,7 +114,8 @@ void kc_destroy(kc_ctx *ctx)
 {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->stream);
-    for (DevBuf *b : {&ctx->part, &ctx->keys, &ctx->stage_in, &ctx->stage_out, &ctx->work, &ctx->vs.buf, &ctx->vs.jbuf})
+    for (DevBuf *b : {&ctx->part, &ctx->keys, &ctx->stage_in, &ctx->stage_out, &ctx->work, &ctx->obj, &ctx->exact,
+                      &ctx->tmax, &ctx->center, &ctx->vs.buf, &ctx->vs.jbuf})
         if (b->p) cudaFree(b->p);
     if (ctx->X) cudaFree(ctx->X);
     if (ctx->pinned) cudaFreeHost(ctx->pinned);
@@ -212,6 +213,11 @@ kc_status kc_create(const void *X, int64_t N, int32_t D, int32_t K, kc_dtype dt,
     st = launch_root_box(c, so, so + (size_t)kMaxD * 8, flag_dev);
     if (st != KC_OK) return fail(st);
     int flag = 0;
+    double box[2][kMaxD];
+    if (dt == KC_F64 && cudaMemcpyAsync(box, so, sizeof(box), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess) {
+        set_err(c, KC_ECUDA, "kc_create: %s", cudaGetErrorString(cudaGetLastError()));
+        return fail(KC_ECUDA);
+    }
     if (cudaMemcpyAsync(&flag, flag_dev, sizeof(int), cudaMemcpyDeviceToHost, c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess) {
         set_err(c, KC_ECUDA, "kc_create: %s", cudaGetErrorString(cudaGetLastError()));
@@ -220,6 +226,23 @@ kc_status kc_create(const void *X, int64_t N, int32_t D, int32_t K, kc_dtype dt,
     if (flag) {
         set_err(c, KC_EINVAL, "kc_create: the data contain NaN or infinite values");
         return fail(KC_EINVAL);
+    }
+    if (dt == KC_F64) {
+        // double data are screened in float about the middle of their range
+        double r2 = 0.0;
+        for (int a = 0; a < D; ++a) {
+            const double lo = box[0][a], hi = box[1][a], mid = 0.5 * lo + 0.5 * hi;
+            const double r = std::max(hi - mid, mid - lo);
+            r2 += r * r;
+            box[0][a] = mid;
+        }
+        c->half_range = std::sqrt(r2) * (1.0 + 1e-12);
+        st = ensure(c, c->center, (size_t)D * 8);
+        if (st == KC_OK &&
+            cudaMemcpyAsync(c->center.p, box[0], (size_t)D * 8, cudaMemcpyHostToDevice, c->stream) != cudaSuccess)
+            st = set_err(c, KC_ECUDA, "kc_create: %s", cudaGetErrorString(cudaGetLastError()));
+        if (st == KC_OK && cudaStreamSynchronize(c->stream) != cudaSuccess) st = set_err(c, KC_ECUDA, "kc_create: sync");
+        if (st != KC_OK) return fail(st);
     }
     if (src_bytes > ((size_t)64 << 20) && c->work.p) {   // release the upload staging buffer of large datasets
         cudaFree(c->work.p);

@@ -58,6 +58,12 @@ struct kc_ctx {
     kc::DevBuf stage_in;         // staged host inputs
     kc::DevBuf stage_out;        // device-side outputs destined for host
     kc::DevBuf work;             // per-call work arrays
+    kc::DevBuf obj;              // coordinates of the centers being evaluated
+    kc::DevBuf exact;            // kc_exact.cu: screen keys and exact maxima, zero between calls
+    kc::DevBuf tmax;             // kc_exact.cu: the screen's largest value per tile and node
+    int exact_b = 0;             // nodes that `exact` is laid out for
+    kc::DevBuf center;           // double data: [D] middle of the data's range
+    double half_range = 0.0;     // double data: 2-norm over the attributes of half the range
     kc::VisitScratch vs;         // tightening workspace
     kc_mlp *scorer = nullptr;    // learned node scorer used by kc_solve with order = 1
     void *pinned = nullptr;      // pinned host staging
@@ -204,6 +210,11 @@ kc_status autotune_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B
 // instead of sample indices (centers is then ignored).
 kc_status launch_objective(kc_ctx *c, const View &v, const int64_t *centers, int S, int Kc,
                            double alpha_cut, double *val, int64_t *arg, const void *pts = nullptr);
+
+// Exact maxima over the samples of min_k of the squared distance to box k
+// (kc_exact.cu): the objective (lo = hi) and, for double data, the lower bound.
+kc_status launch_exact_max(kc_ctx *c, const View &v, const void *lo, const void *hi, int B, int K, double cut, double *lb,
+                           double *val, int64_t *arg);
 
 // Per-attribute min/max of the data; *nonfinite set if any NaN/Inf.
 kc_status launch_root_box(kc_ctx *c, void *lo, void *hi, int *nonfinite_dev);

@@ -5,8 +5,7 @@
 // nodes the streaming kernel (kc_stream.cu); both raise one (value, position)
 // key per node with 64-bit atomics (the largest value, the smallest position
 // on ties), which a small second kernel turns into the outputs.  Double data:
-// every thread sweeps the batch's nodes for one sample in the serial order of
-// operations, and per-CTA partials are reduced by a second kernel.
+// the exact maxima of kc_exact.cu, in the serial order of operations.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -18,80 +17,6 @@
 namespace kc {
 
 namespace {
-
-// Double lower bound: mid{lo, x, hi}, d = x - mid, acc = acc + d*d in attribute
-// order with separate roundings -- the serial evaluation, bit for bit.
-template <int DMAX>
-__global__ void __launch_bounds__(kThreads)
-lb_f64(const double *__restrict__ X, int64_t ld, int64_t n, const double *__restrict__ lo,
-       const double *__restrict__ hi, int B, int K, int D, double *__restrict__ pval,
-       uint32_t *__restrict__ ppos)
-{
-    constexpr int NW = kThreads / 32;
-    extern __shared__ __align__(16) unsigned char smem[];
-    double *slo = reinterpret_cast<double *>(smem);
-    double *shi = slo + (size_t)B * K * D;
-    double *wval = shi + (size_t)B * K * D;                       // [NW][B]
-    uint32_t *wpos = reinterpret_cast<uint32_t *>(wval + NW * B); // [NW][B]
-    for (int i = threadIdx.x; i < B * K * D; i += kThreads) { slo[i] = lo[i]; shi[i] = hi[i]; }
-    for (int i = threadIdx.x; i < NW * B; i += kThreads) { wval[i] = -1.0; wpos[i] = 0xFFFFFFFFu; }
-    __syncthreads();
-
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int64_t s = (int64_t)blockIdx.x * kThreads + threadIdx.x; s - threadIdx.x < n;
-         s += (int64_t)gridDim.x * kThreads) {
-        const bool valid = s < n;
-        double x[DMAX];
-#pragma unroll
-        for (int a = 0; a < DMAX; ++a) x[a] = (valid && a < D) ? X[(size_t)a * ld + s] : 0.0;
-        for (int b = 0; b < B; ++b) {
-            double best = __longlong_as_double(0x7ff0000000000000ll);
-            for (int k = 0; k < K; ++k) {
-                const double *l = slo + ((size_t)b * K + k) * D, *h = shi + ((size_t)b * K + k) * D;
-                double acc = 0.0;
-#pragma unroll
-                for (int a = 0; a < DMAX; ++a) {
-                    if (a < D) {
-                        const double mu = mid3d(l[a], x[a], h[a]);
-                        const double d = __dsub_rn(x[a], mu);
-                        acc = __dadd_rn(acc, __dmul_rn(d, d));
-                    }
-                }
-                if (acc < best) best = acc;
-            }
-            const double m = valid ? best : -1.0;
-            const double cur = wval[w * B + b];
-            const bool maybe = m >= cur && m >= 0.0;
-            if (__any_sync(0xffffffffu, maybe)) {
-                double v = maybe ? m : -1.0;
-                uint32_t p = maybe ? (uint32_t)s : 0xFFFFFFFFu;
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    const double v2 = __shfl_xor_sync(0xffffffffu, v, o);
-                    const uint32_t p2 = __shfl_xor_sync(0xffffffffu, p, o);
-                    if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
-                }
-                if (lane == 0 && (v > cur || (v == cur && p < wpos[w * B + b]))) {
-                    wval[w * B + b] = v;
-                    wpos[w * B + b] = p;
-                }
-                __syncwarp();
-            }
-        }
-    }
-    __syncthreads();
-    for (int b = threadIdx.x; b < B; b += kThreads) {
-        double v = -1.0;
-        uint32_t p = 0xFFFFFFFFu;
-        for (int q = 0; q < NW; ++q) {
-            const double v2 = wval[q * B + b];
-            const uint32_t p2 = wpos[q * B + b];
-            if (v2 > v || (v2 == v && p2 < p)) { v = v2; p = p2; }
-        }
-        pval[(size_t)blockIdx.x * B + b] = v;
-        ppos[(size_t)blockIdx.x * B + b] = p;
-    }
-}
 
 // Exact refinement of float-data lower bounds: each node comes with a float
 // threshold below which no sample can attain the double maximum (from the
@@ -246,71 +171,14 @@ __global__ void lb_finalize_f64(const double *__restrict__ pval, const uint32_t 
 
 // ---------------------------------------------------------------- dispatch
 
-// Attribute pairs with a compiled kernel; other D take the next larger one
-// (padding pairs add exactly zero).
-using PruneFn = void (*)(const PruneArgs);
-struct PruneEntry {
-    int P, ST, T, NT;
-    PruneFn fn;
-};
-template <int P, int ST = PruneShape<P>::ST>
-PruneEntry prune_entry()
-{
-    constexpr int NT = PruneShape<P>::NT, T = NT * ST;
-    return PruneEntry{P, ST, T, NT, prune_max_kernel<P, ST, NT>};
-}
-const PruneEntry kPrune[] = {
-    prune_entry<1>(), prune_entry<1, 2>(), prune_entry<2>(), prune_entry<2, 2>(), prune_entry<3>(),
-    prune_entry<3, 2>(), prune_entry<4>(), prune_entry<4, 2>(), prune_entry<6>(), prune_entry<8>(),
-    prune_entry<12>(), prune_entry<16>(), prune_entry<24>(), prune_entry<34>(), prune_entry<48>(), prune_entry<64>(),
-};
 // Launches the float maxima of A.B nodes into A.keys (zeroed by the caller) on
 // `stream`; st (samples per thread: 4 or 2, where both exist) and chunk (nodes
 // per CTA) of 0 are chosen here.
 cudaError_t launch_max_f32(PruneArgs A, int sms, size_t smem_cap, int st, int chunk, cudaStream_t stream)
 {
-    const int P = (A.D + 1) / 2;
     A.vec = (uintptr_t)A.X % 16 == 0 && A.ld % 4 == 0;
     if (use_stream_f32(A.B, A.K, A.D)) return launch_stream_f32(A, sms, stream);
-    const PruneEntry *e = kPrune;
-    while (e->P < P) ++e;
-    if (P <= 4) {
-        // two entries: 4 and 2 samples per thread
-        const int64_t t4 = (A.n + e->T - 1) / e->T;
-        if (st == 2 || (st != 4 && t4 < 8 * (int64_t)sms)) ++e;
-    }
-    const int64_t tiles = (A.n + e->T - 1) / e->T;
-    const auto fits = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32).end <= smem_cap; };
-    int per = A.B;
-    if (chunk > 0 && chunk < per) per = chunk;
-    if (tiles < sms) {
-        // few tiles: spread the nodes over the SMs as well, whole groups to a CTA
-        const int64_t want = std::max<int64_t>(1, sms / tiles);
-        per = (int)std::min<int64_t>(per, ((A.B + want - 1) / want + kPG - 1) / kPG * kPG);
-    }
-    while (per > 1 && !fits(per)) per = per > 2 * kPG ? (per - 1) / kPG * kPG : per - 1;
-    A.per = per;
-    const size_t smem = PruneLayout(per, A.K, e->P, e->T, e->NT / 32).end;
-    if (smem > smem_cap) return cudaErrorInvalidConfiguration;
-    if (smem > 48 * 1024) {
-        const cudaError_t r = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (r != cudaSuccess) return r;
-    }
-    // at most 65535 node ranges to a launch
-    const int B = A.B, step = (int)std::min<int64_t>((int64_t)per * 65535, B);
-    const size_t box = (size_t)A.K * A.D * 4;
-    for (int b0 = 0; b0 < B; b0 += step) {
-        PruneArgs C = A;
-        C.B = std::min(step, B - b0);
-        C.lo = static_cast<const char *>(A.lo) + b0 * box;
-        C.hi = static_cast<const char *>(A.hi) + b0 * box;
-        C.keys = A.keys + b0;
-        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, sms)), (unsigned)((C.B + per - 1) / per));
-        e->fn<<<grid, e->NT, smem, stream>>>(C);
-        const cudaError_t r = cudaGetLastError();
-        if (r != cudaSuccess) return r;
-    }
-    return cudaSuccess;
+    return prune_run(prune_pick(prune_table<false, false>(), A.D, A.n, sms, st), A, false, sms, smem_cap, chunk, stream);
 }
 
 template <typename F>
@@ -329,6 +197,43 @@ kc_status prep_kernel(kc_ctx *c, F fn, size_t smem, int *grid, int64_t tiles)
 
 }  // namespace
 
+cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t smem_cap, int chunk, cudaStream_t stream)
+{
+    const int64_t tiles = (A.n + e->T - 1) / e->T;
+    const auto bytes = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32, tm).end; };
+    int per = A.B;
+    if (chunk > 0 && chunk < per) per = chunk;
+    if (tiles < sms) {
+        // few tiles: spread the nodes over the SMs as well, whole groups to a CTA
+        const int64_t want = std::max<int64_t>(1, sms / tiles);
+        per = (int)std::min<int64_t>(per, ((A.B + want - 1) / want + kPG - 1) / kPG * kPG);
+    }
+    while (per > 1 && bytes(per) > smem_cap) per = per > 2 * kPG ? (per - 1) / kPG * kPG : per - 1;
+    A.per = per;
+    const size_t smem = bytes(per);
+    if (smem > smem_cap) return cudaErrorInvalidConfiguration;
+    if (smem > 48 * 1024) {
+        const cudaError_t r = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (r != cudaSuccess) return r;
+    }
+    // at most 65535 node ranges to a launch
+    const int B = A.B, step = (int)std::min<int64_t>((int64_t)per * 65535, B);
+    const size_t box = (size_t)A.K * A.D * (A.off ? 8 : 4);
+    if (tm && step < B) return cudaErrorInvalidConfiguration;   // (screens come in batches far smaller)
+    for (int b0 = 0; b0 < B; b0 += step) {
+        PruneArgs C = A;
+        C.B = std::min(step, B - b0);
+        C.lo = static_cast<const char *>(A.lo) + b0 * box;
+        C.hi = static_cast<const char *>(A.hi) + b0 * box;
+        C.keys = A.keys + b0;
+        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, sms)), (unsigned)((C.B + per - 1) / per));
+        e->fn<<<grid, e->NT, smem, stream>>>(C);
+        const cudaError_t r = cudaGetLastError();
+        if (r != cudaSuccess) return r;
+    }
+    return cudaSuccess;
+}
+
 kc_status launch_lower_bounds_view(kc_ctx *c, const View &v, const void *lo, const void *hi, int B,
                                    double *lb, double *lb_raw, int64_t *arg, int st_override)
 {
@@ -342,7 +247,6 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
     const int D = c->D, K = c->K;
     const double defl = deflate_factor(c->dt, D), slack = underflow_slack(c->dt, D);
     const size_t smem_cap = c->smem_optin > 0 ? c->smem_optin : 48 * 1024;
-    const int NW = kThreads / 32;
     if (c->dt == KC_F32) {
         if (c->keys.bytes < (size_t)B * 8) {
             KC_TRY(ensure(c, c->keys, (size_t)B * 8));
@@ -366,31 +270,7 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
         lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B, v.ids, defl, slack, lb, lb_raw, arg);
         KC_TRY(after_launch(c, "lower bound finalize"));
     } else {
-        const size_t per_node = (size_t)K * D * 16 + NW * 12;
-        int chunk = (int)std::min<size_t>((size_t)B, (smem_cap / 2 > per_node ? (smem_cap / 2) / per_node : 1));
-        if (chunk < 1) chunk = 1;
-        for (int b0 = 0; b0 < B; b0 += chunk) {
-            const int nb = std::min(chunk, B - b0);
-            const size_t smem = per_node * nb;
-            const double *l = static_cast<const double *>(lo) + (size_t)b0 * K * D;
-            const double *h = static_cast<const double *>(hi) + (size_t)b0 * K * D;
-            const int64_t tiles = (v.n + kThreads - 1) / kThreads;
-            int grid = 1;
-            auto g = D <= 16 ? lb_f64<16> : (D <= 64 ? lb_f64<64> : lb_f64<128>);
-            KC_TRY(prep_kernel(c, g, smem, &grid, tiles));
-            KC_TRY(ensure(c, c->part, (size_t)grid * nb * 12));
-            double *pval = static_cast<double *>(c->part.p);
-            uint32_t *ppos = reinterpret_cast<uint32_t *>(pval + (size_t)grid * nb);
-            if (v.n > 0) {
-                g<<<grid, kThreads, smem, c->stream>>>(static_cast<const double *>(v.X), v.ld, v.n, l, h, nb, K, D, pval,
-                                                       ppos);
-                KC_TRY(after_launch(c, "lower bound f64"));
-            }
-            lb_finalize_f64<<<(nb + 3) / 4, 128, 0, c->stream>>>(
-                pval, ppos, v.n > 0 ? grid : 0, nb, v.ids, defl, slack, lb ? lb + b0 : nullptr,
-                lb_raw ? lb_raw + b0 : nullptr, arg ? arg + b0 : nullptr);
-            KC_TRY(after_launch(c, "lower bound finalize f64"));
-        }
+        KC_TRY(launch_exact_max(c, v, lo, hi, B, K, __builtin_huge_val(), lb, lb_raw, arg));
     }
     return KC_OK;
 }

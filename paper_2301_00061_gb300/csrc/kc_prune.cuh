@@ -37,6 +37,9 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <type_traits>
+
 #include "kc_device.cuh"
 #include "kc_internal.cuh"
 
@@ -54,7 +57,21 @@ struct PruneArgs {
     int per;                  // nodes per CTA range (blockIdx.y), a multiple of kPG unless B is smaller
     int vec;                  // rows may be read with 16-byte loads (X 16-byte aligned, ld a multiple of 16 bytes)
     unsigned long long *keys; // [B] (value bits, ~position), zero before the launch
+    // screens of an exact maximum (kc_exact.cu): the largest float value of each
+    // node in each tile, of all samples that may attain the exact maximum
+    float *tmax;              // [tiles][B]
+    float c1, eps;            // such a sample's float value reaches screen_floor(best, c1, eps)
+    float cut;                // nodes proved to reach this float value are done
+    const double *off;        // [D] double data: subtracted before the conversion to float
 };
+
+// Below this float value a sample cannot attain a maximum whose largest float
+// value is m (rounded down; 0: any may): (c1 sqrt(m) - eps)^2.
+__device__ __forceinline__ float screen_floor(float m, float c1, float eps)
+{
+    const float s = __fsub_rd(__fmul_rd(__fsqrt_rd(fminf(m, 3.0e38f)), c1), eps);
+    return s > 0.f ? fmaxf(__fsub_rd(__fmul_rd(s, s), 1e-37f), 0.f) : 0.f;
+}
 
 // Threads and samples per thread of the kernel for P attribute pairs: the tile
 // of NT ST samples stays in shared memory (8 P bytes each, 64 KB or so) beside
@@ -76,8 +93,8 @@ __host__ __device__ inline size_t al16(size_t v) { return (v + 15) & ~(size_t)15
 
 // Shared memory of a CTA with nb nodes, K clusters, P pairs and a tile of T samples.
 struct PruneLayout {
-    size_t box, gbox, sbox, stage, ref, cand, key, thr, gmin, smin, hist, pos, queue, fk, fg, fs, rr, end;
-    __host__ __device__ PruneLayout(int nb, int K, int P, int T, int warps)
+    size_t box, gbox, sbox, stage, ref, cand, key, thr, gmin, smin, hist, pos, queue, tmx, fk, fg, fs, rr, end;
+    __host__ __device__ PruneLayout(int nb, int K, int P, int T, int warps, bool tm)
     {
         const int ng = (nb + kPG - 1) / kPG, ns = (ng + kPSG - 1) / kPSG;
         size_t o = 0;
@@ -95,6 +112,7 @@ struct PruneLayout {
         hist = o; o += (2 * kMaxK + 4) * 4;   // counts, bases, queue lengths
         pos = o; o += (size_t)T * 4;
         queue = o; o += al16((size_t)warps * ng * 4) + (size_t)2 * pair_cap(P) * 4;
+        tmx = o; o += tm ? al16((size_t)nb * 4) : 0;
         fk = o; o += al16((size_t)nb * K);
         fg = o; o += al16((size_t)ng * K);
         fs = o; o += al16((size_t)ns * K);
@@ -235,7 +253,46 @@ __device__ __forceinline__ bool push_pairs(unsigned m, int c, int *count, uint32
     return fits;
 }
 
-template <int P, int ST, int NT>
+// The same for double data: the samples less off, rounded to float.
+template <int ST, int P>
+__device__ __forceinline__ void load_samples(const double *__restrict__ X, int64_t ld, int64_t n, int D, bool vec,
+                                             int64_t s0, uint64_t (&x)[ST][P], const double *__restrict__ off)
+{
+    const bool full = vec && s0 + ST <= n;
+#pragma unroll
+    for (int p = 0; p < P; ++p) {
+        float v[2][ST];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int a = 2 * p + h;
+#pragma unroll
+            for (int j = 0; j < ST; ++j) v[h][j] = 0.f;
+            if (a < D) {
+                const double *row = X + (size_t)a * ld, c = __ldg(off + a);
+                double w[ST];
+                if (full && ST % 2 == 0) {
+#pragma unroll
+                    for (int j = 0; j + 1 < ST; j += 2) {
+                        const double2 q = __ldg(reinterpret_cast<const double2 *>(row + s0 + j));
+                        w[j] = q.x;
+                        w[j + 1] = q.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int j = 0; j < ST; ++j) w[j] = __ldg(row + (s0 + j < n ? s0 + j : n - 1));
+                }
+#pragma unroll
+                for (int j = 0; j < ST; ++j) v[h][j] = __double2float_rn(w[j] - c);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < ST; ++j) x[j][p] = pk(v[0][j], v[1][j]);
+    }
+}
+
+// F64: double data, boxes rounded inwards after the offset, so that the float
+// values bound the exact ones (kc_exact.cu).  TM: a screen that fills A.tmax.
+template <int P, int ST, int NT, bool F64, bool TM>
 __global__ void __launch_bounds__(NT, 1)
 prune_max_kernel(const PruneArgs A)
 {
@@ -245,7 +302,7 @@ prune_max_kernel(const PruneArgs A)
     const int K = A.K, D = A.D, KP = K * P, KR = K * RW;
     const int b0 = blockIdx.y * A.per, nb = min(A.per, A.B - b0);
     const int ng = (nb + kPG - 1) / kPG, ns = (ng + kPSG - 1) / kPSG;
-    const PruneLayout L(nb, K, P, T, NWP);
+    const PruneLayout L(nb, K, P, T, NWP, TM);
     ulonglong2 *box = reinterpret_cast<ulonglong2 *>(smem + L.box), *gbox = reinterpret_cast<ulonglong2 *>(smem + L.gbox);
     ulonglong2 *sbox = reinterpret_cast<ulonglong2 *>(smem + L.sbox);
     uint64_t *ref = reinterpret_cast<uint64_t *>(smem + L.ref), *stage = reinterpret_cast<uint64_t *>(smem + L.stage);
@@ -257,8 +314,19 @@ prune_max_kernel(const PruneArgs A)
     uint32_t *spos = reinterpret_cast<uint32_t *>(smem + L.pos), *queue = reinterpret_cast<uint32_t *>(smem + L.queue);
     uint32_t *qb = queue + ((NWP * ng + 3) & ~3), *qc = qb + CAP;
     uint8_t *fk = smem + L.fk, *fg = smem + L.fg, *fs = smem + L.fs, *rr = smem + L.rr;
-    const float *lo = static_cast<const float *>(A.lo) + (size_t)b0 * K * D;
-    const float *hi = static_cast<const float *>(A.hi) + (size_t)b0 * K * D;
+    using T_ = typename std::conditional<F64, double, float>::type;
+    const T_ *lo = static_cast<const T_ *>(A.lo) + (size_t)b0 * K * D;
+    const T_ *hi = static_cast<const T_ *>(A.hi) + (size_t)b0 * K * D;
+    const T_ *X = static_cast<const T_ *>(A.X);
+    auto load = [&](int64_t s0, uint64_t (&x)[ST][P]) {
+        if constexpr (F64) load_samples<ST, P>(X, A.ld, A.n, D, A.vec != 0, s0, x, A.off);
+        else load_samples<ST, P>(X, A.ld, A.n, D, A.vec != 0, s0, x);
+    };
+    auto floor_of = [&](float v) {   // values below it can be dismissed
+        if constexpr (TM)
+            return v >= A.cut && A.cut < __int_as_float(0x7f800000) ? __int_as_float(0x7f800000) : screen_floor(v, A.c1, A.eps);
+        else return v;
+    };
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float INF = __int_as_float(0x7f800000);
 
@@ -268,9 +336,24 @@ prune_max_kernel(const PruneArgs A)
         const int p = i % P, bk = i / P, a = 2 * p;
         const size_t o = (size_t)bk * D + a;
         const bool two = a + 1 < D;
-        box[bk * RW + p] = a < D ? make_ulonglong2(pk(lo[o], two ? lo[o + 1] : 0.f), pk(hi[o], two ? hi[o + 1] : 0.f))
-                                 : make_ulonglong2(0ull, 0ull);
+        if constexpr (F64) {
+            auto in = [&](int e, float &l, float &h) {
+                const double c = A.off[a + e];
+                l = __double2float_ru(__dsub_ru(lo[o + e], c));
+                h = __double2float_rd(__dsub_rd(hi[o + e], c));
+            };
+            float l0 = 0.f, h0 = 0.f, l1 = 0.f, h1 = 0.f;
+            if (a < D) in(0, l0, h0);
+            if (two) in(1, l1, h1);
+            box[bk * RW + p] = make_ulonglong2(pk(l0, l1), pk(h0, h1));
+        } else {
+            box[bk * RW + p] = a < D ? make_ulonglong2(pk(lo[o], two ? lo[o + 1] : 0.f), pk(hi[o], two ? hi[o + 1] : 0.f))
+                                     : make_ulonglong2(0ull, 0ull);
+        }
     }
+    unsigned *tmx = reinterpret_cast<unsigned *>(smem + L.tmx);
+    if constexpr (TM)
+        for (int i = tid; i < nb; i += NT) tmx[i] = 0u;
     if (tid < 32) cand[tid] = 0ull;
     __syncthreads();
     auto meet = [&](const ulonglong2 *src, int cnt, ulonglong2 *dst, int e) {
@@ -321,27 +404,34 @@ prune_max_kernel(const PruneArgs A)
     // raise node b's best value by a warp whose lanes hold keys (0: none)
     auto raise = [&](int b, unsigned long long k) {
         k = warp_max_u64(k);
+        if (TM && lane == 0) atomicMax(&tmx[b], (unsigned)(k >> 32));
         if (lane == 0 && k > key[b]) {
             atomicMax(const_cast<unsigned long long *>(&key[b]), k);
-            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(key_val(k)));
+            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(floor_of(key_val(k))));
         }
         __syncwarp();
     };
 
+    auto coord = [&](int a, int64_t s) {
+        const T_ v = X[(size_t)a * A.ld + s];
+        if constexpr (F64) return __double2float_rn(v - A.off[a]);
+        else return v;
+    };
     // the same for one lane's value
     auto lift = [&](int b, float v, uint32_t pos) {
         const unsigned long long k = key_max(v, pos);
-        if (v >= thr[b] && k > key[b]) {
+        if (!(v >= thr[b])) return;
+        if (TM) atomicMax(&tmx[b], __float_as_uint(v));
+        if (k > key[b]) {
             atomicMax(const_cast<unsigned long long *>(&key[b]), k);
-            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(v));
+            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(floor_of(v)));
         }
     };
 
-    const float *X = static_cast<const float *>(A.X);
     const int64_t tiles = (A.n + T - 1) / T;
     const int w0 = warp * 32 * ST;   // the warp's slots of the sorted tile
     uint64_t x[ST][P];
-    load_samples<ST, P>(X, A.ld, A.n, D, A.vec != 0, (int64_t)blockIdx.x * T + (int64_t)tid * ST, x);
+    load((int64_t)blockIdx.x * T + (int64_t)tid * ST, x);
     bool seed = true;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int64_t s0 = tile * T + (int64_t)tid * ST;
@@ -390,7 +480,7 @@ prune_max_kernel(const PruneArgs A)
             unsigned long long m = seed ? 0ull : key[b];
             m = g > m ? g : m;
             key[b] = m;
-            thr[b] = key_val(m);
+            thr[b] = floor_of(key_val(m));
         }
         // slots of the samples, sorted by reference
         int off[ST];
@@ -414,8 +504,7 @@ prune_max_kernel(const PruneArgs A)
             uint64_t xc[1][P];
 #pragma unroll
             for (int p = 0; p < P; ++p)
-                xc[0][p] = pk(2 * p < D ? X[(size_t)(2 * p) * A.ld + cp] : 0.f,
-                              2 * p + 1 < D ? X[(size_t)(2 * p + 1) * A.ld + cp] : 0.f);
+                xc[0][p] = pk(2 * p < D ? coord(2 * p, cp) : 0.f, 2 * p + 1 < D ? coord(2 * p + 1, cp) : 0.f);
             for (int b = warp; b < nb; b += NWP) {
                 float best = INF;
                 for (int k = 0; k < K; ++k) {
@@ -481,7 +570,7 @@ prune_max_kernel(const PruneArgs A)
         // the next tile's samples, in flight while the queue is worked off
         constexpr bool AHEAD = P < 48;   // (where the registers hold both)
         const bool more = tile + gridDim.x < tiles;
-        if (AHEAD && more) load_samples<ST, P>(X, A.ld, A.n, D, A.vec != 0, s0 + (int64_t)gridDim.x * T, x);
+        if (AHEAD && more) load(s0 + (int64_t)gridDim.x * T, x);
         __syncthreads();
         const int items = qn[0], pairs = min(qn[1], CAP);
         for (int it = warp; it < items; it += NWP) {
@@ -529,7 +618,8 @@ prune_max_kernel(const PruneArgs A)
                     const unsigned long long q = key_max(v[j], spos[q0 + j * 32 + lane]);
                     top = q > top ? q : top;
                 }
-                if (__any_sync(ALL, top > cur)) raise(b, top > cur ? top : 0ull);
+                if constexpr (TM) raise(b, top);
+                else if (__any_sync(ALL, top > cur)) raise(b, top > cur ? top : 0ull);
             }
         }
         // (group, sample) pairs, one to a lane
@@ -582,15 +672,55 @@ prune_max_kernel(const PruneArgs A)
             }
             lift(b, v, spos[slot]);
         }
-        if (!AHEAD && more) load_samples<ST, P>(X, A.ld, A.n, D, A.vec != 0, s0 + (int64_t)gridDim.x * T, x);
+        if (!AHEAD && more) load(s0 + (int64_t)gridDim.x * T, x);
         __syncthreads();
         // publish what this tile raised
         for (int b = tid; b < nb; b += NT) {
             const unsigned long long k = key[b];
             if (k > peek(&A.keys[b0 + b])) atomicMax(&A.keys[b0 + b], k);
+            if constexpr (TM) {
+                A.tmax[(size_t)tile * A.B + b0 + b] = __uint_as_float(tmx[b]);
+                tmx[b] = 0u;
+            }
         }
     }
 }
+
+// Attribute pairs with a compiled kernel (other D take the next larger one:
+// padding pairs add exactly zero) and their launch.
+struct PruneEntry {
+    int P, ST, T, NT;
+    void (*fn)(const PruneArgs);
+};
+template <int P, bool F64, bool TM, int ST = PruneShape<P>::ST>
+PruneEntry prune_entry()
+{
+    constexpr int NT = PruneShape<P>::NT;
+    return PruneEntry{P, ST, NT * ST, NT, prune_max_kernel<P, ST, NT, F64, TM>};
+}
+// Table of the kernels in ascending P, two entries (4 and 2 samples a thread)
+// for each P <= 4.
+template <bool F64, bool TM>
+const PruneEntry *prune_table()
+{
+    static const PruneEntry t[] = {
+        prune_entry<1, F64, TM>(),  prune_entry<1, F64, TM, 2>(), prune_entry<2, F64, TM>(), prune_entry<2, F64, TM, 2>(),
+        prune_entry<3, F64, TM>(),  prune_entry<3, F64, TM, 2>(), prune_entry<4, F64, TM>(), prune_entry<4, F64, TM, 2>(),
+        prune_entry<6, F64, TM>(),  prune_entry<8, F64, TM>(),    prune_entry<12, F64, TM>(), prune_entry<16, F64, TM>(),
+        prune_entry<24, F64, TM>(), prune_entry<34, F64, TM>(),   prune_entry<48, F64, TM>(), prune_entry<64, F64, TM>()};
+    return t;
+}
+// The entry for D attributes and n samples (st: 4 or 2 samples a thread where
+// both exist, 0: by size -- 2 where the tiles of 4 would not fill 8 rounds).
+inline const PruneEntry *prune_pick(const PruneEntry *e, int D, int64_t n, int sms, int st)
+{
+    const int P = (D + 1) / 2;
+    while (e->P < P) ++e;
+    if (P <= 4 && (st == 2 || (st != 4 && (n + e->T - 1) / e->T < 8 * (int64_t)sms))) ++e;
+    return e;
+}
+// chunk: nodes per CTA at most (0: as many as fit).  A.B = all nodes.
+cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t smem_cap, int chunk, cudaStream_t stream);
 
 // The streaming path for few nodes (kc_stream.cu): taken at up to
 // kStreamTerms node x cluster x attribute terms for D <= 8, and at up to two
@@ -604,5 +734,6 @@ inline bool use_stream_f32(int B, int K, int D)
     return (D <= 8 && B * K * D <= kStreamTerms) || (B <= 2 && B * K <= kStreamCols);
 }
 cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream);
+constexpr int kStreamTile = 128;   // samples of a tmax row of the streaming screen
 
 }  // namespace kc

@@ -118,7 +118,7 @@ __device__ __forceinline__ void stream_finish(const PruneArgs &A, int b, unsigne
 // K fixed, the loop over the clusters unrolled; 0: any K, about 8 % slower).
 // MANY (more than two nodes): each warp keeps its nodes' keys in shared memory
 // and reduces over its lanes only when one of them may beat the key.
-template <int DC, int KC, int Q, int CTAS, bool MANY>
+template <int DC, int KC, int Q, int CTAS, bool MANY, bool TM>
 __global__ void __launch_bounds__(kThreads, CTAS)
 stream_max_small(const PruneArgs A)
 {
@@ -129,7 +129,7 @@ stream_max_small(const PruneArgs A)
     unsigned long long *mine = wkey + (threadIdx.x >> 5) * A.B;
     __shared__ unsigned long long red[NWP];
     stream_boxes(A, box);
-    if (MANY)
+    if (MANY || TM)
         for (int i = threadIdx.x; i < NWP * A.B; i += kThreads) wkey[i] = 0ull;
     __syncthreads();
     const float *X = static_cast<const float *>(A.X);
@@ -191,7 +191,15 @@ stream_max_small(const PruneArgs A)
 #pragma unroll
                 for (int j = 0; j < ST; ++j) m[j] = min3f(m[j], d0[j], d1[j]);
             }
-            if constexpr (MANY) {
+            if constexpr (TM) {
+                const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(max_of<ST>(m)));
+                if ((threadIdx.x & 31) == 0) {
+                    const int64_t row = (base >> 7) + (threadIdx.x >> 5);
+                    if (row * kStreamTile < A.n) A.tmax[row * A.B + b] = __uint_as_float(w);
+                    const unsigned long long key = ((unsigned long long)w << 32) | 1ull;
+                    if (key > mine[b]) mine[b] = key;
+                }
+            } else if constexpr (MANY) {
                 const unsigned long long cur = mine[b];
                 const bool may = max_of<ST>(m) >= key_val(cur);
                 if (__any_sync(0xffffffffu, may)) {
@@ -217,7 +225,7 @@ stream_max_small(const PruneArgs A)
             }
         }
     }
-    if constexpr (MANY) {
+    if constexpr (MANY || TM) {
         __syncthreads();
         for (int b = threadIdx.x; b < A.B; b += kThreads) {
             unsigned long long k = 0ull;
@@ -232,7 +240,7 @@ stream_max_small(const PruneArgs A)
 
 // Any D: the attributes stream through, KC >= nodes x clusters accumulators in
 // registers.
-template <int KC>
+template <int KC, bool TM>
 __global__ void __launch_bounds__(kThreads, KC <= 4 ? 4 : (KC <= 8 ? 2 : 1))
 stream_max_wide(const PruneArgs A)
 {
@@ -280,8 +288,17 @@ stream_max_wide(const PruneArgs A)
                 m0 = fresh ? d0 : make_float2(fminf(m0.x, d0.x), fminf(m0.y, d0.y));
                 m1 = fresh ? d1 : make_float2(fminf(m1.x, d1.x), fminf(m1.y, d1.y));
                 const float d[4] = {m0.x, m0.y, m1.x, m1.y};
-                if (c == K - 1) best0.take<1>(d, s0, A.n);
-                else if (c == C - 1) best1.take<1>(d, s0, A.n);
+                if (c != K - 1 && c != C - 1) continue;
+                StreamBest &best = c == K - 1 ? best0 : best1;
+                if constexpr (TM) {
+                    const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(max_of<4>(d)));
+                    const int64_t row = (base >> 7) + (threadIdx.x >> 5);
+                    if ((threadIdx.x & 31) == 0 && row * kStreamTile < A.n)
+                        A.tmax[row * A.B + (c == K - 1 ? 0 : 1)] = __uint_as_float(w);
+                    best.v = fmaxf(best.v, __uint_as_float(w));
+                } else {
+                    best.take<1>(d, s0, A.n);
+                }
             }
     }
     stream_finish(A, 0, best0.key(), red);
@@ -293,40 +310,47 @@ using StreamKernel = void (*)(const PruneArgs);
 // Registers: a sample takes 4 D with its swapped copy, so D <= 4 keeps two
 // quads a thread (half the box reads per sample) at 3 or 4 CTAs an SM.
 template <int DC, int KC>
-constexpr StreamKernel small_kernel(bool many)
+constexpr StreamKernel small_kernel(bool many, bool tm)
 {
     constexpr int Q = DC <= 4 ? 2 : 1, CT = DC <= 2 ? 4 : 3;
-    return many ? stream_max_small<DC, KC, Q, CT, true> : stream_max_small<DC, KC, Q, CT, false>;
+    return tm ? stream_max_small<DC, KC, 1, CT, false, true>
+              : (many ? stream_max_small<DC, KC, Q, CT, true, false> : stream_max_small<DC, KC, Q, CT, false, false>);
 }
 template <int DC>
-StreamKernel small_kernel_k(int K, bool many)
+StreamKernel small_kernel_k(int K, bool many, bool tm)
 {
-    return K == 3 ? small_kernel<DC, 3>(many) : K == 4 ? small_kernel<DC, 4>(many) : K == 5 ? small_kernel<DC, 5>(many)
-                                                                                            : small_kernel<DC, 0>(many);
+    return K == 3 ? small_kernel<DC, 3>(many, tm) : K == 4 ? small_kernel<DC, 4>(many, tm)
+         : K == 5 ? small_kernel<DC, 5>(many, tm) : small_kernel<DC, 0>(many, tm);
 }
-StreamKernel small_kernel_of(int D, int K, bool many)
+StreamKernel small_kernel_of(int D, int K, bool many, bool tm)
 {
     switch (D) {
-    case 1: return small_kernel_k<1>(K, many);
-    case 2: return small_kernel_k<2>(K, many);
-    case 3: return small_kernel_k<3>(K, many);
-    case 4: return small_kernel_k<4>(K, many);
-    case 5: return small_kernel_k<5>(K, many);
-    case 6: return small_kernel_k<6>(K, many);
-    case 7: return small_kernel_k<7>(K, many);
-    default: return small_kernel_k<8>(K, many);
+    case 1: return small_kernel_k<1>(K, many, tm);
+    case 2: return small_kernel_k<2>(K, many, tm);
+    case 3: return small_kernel_k<3>(K, many, tm);
+    case 4: return small_kernel_k<4>(K, many, tm);
+    case 5: return small_kernel_k<5>(K, many, tm);
+    case 6: return small_kernel_k<6>(K, many, tm);
+    case 7: return small_kernel_k<7>(K, many, tm);
+    default: return small_kernel_k<8>(K, many, tm);
     }
+}
+template <bool TM>
+StreamKernel wide_kernel_of(int cols)
+{
+    return cols <= 4 ? stream_max_wide<4, TM> : (cols <= 8 ? stream_max_wide<8, TM> : stream_max_wide<16, TM>);
 }
 
 }  // namespace
 
 cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream)
 {
-    const int cols = A.B * A.K, Q = A.D <= 4 ? 2 : 1;
+    const bool tm = A.tmax != nullptr;
+    const int cols = A.B * A.K, Q = A.D <= 4 && !tm ? 2 : 1;
     size_t smem = (size_t)cols * A.D * 16;   // at most 32 KB for both forms
-    StreamKernel fn = cols <= 4 ? stream_max_wide<4> : (cols <= 8 ? stream_max_wide<8> : stream_max_wide<16>);
+    StreamKernel fn = tm ? wide_kernel_of<true>(cols) : wide_kernel_of<false>(cols);
     if (A.D <= 8) {
-        fn = small_kernel_of(A.D, A.K, A.B > 2);
+        fn = small_kernel_of(A.D, A.K, A.B > 2, tm);
         smem += (size_t)kThreads / 32 * A.B * 8;
     }
     int per_sm = 0;
