@@ -106,39 +106,48 @@ __device__ __forceinline__ bool node_cut(float m, double gam, double cut)
     return gam >= 0.0 && __ddiv_rd((double)m, 1.0 + gam) >= cut;
 }
 
-// One thread per (tile, node): does the tile hold a sample that may attain the
-// node's maximum?  The warp then goes through the tile: four samples per lane
-// at a time in float, those that reach the floor in double.
+// A CTA looks over 256 (node, tile) entries at a time: does the tile hold a
+// sample that may attain the node's maximum?  All its threads then go through
+// each such tile, four samples a thread at a time: in float, and those that
+// reach the floor in double.  (The tiles of one sample far from everything are
+// hits of every node; entries are ordered by node, so they meet different CTAs:
+// with one warp to a hit and 32 nodes to a warp this took 375 us of 450.)
 template <typename T>
 __global__ void __launch_bounds__(256)
-exact_hits_kernel(const HitArgs H, int64_t total)
+exact_hits_kernel(const HitArgs H)
 {
     constexpr bool F64 = sizeof(T) == 8;
     constexpr int U = 4;
+    __shared__ int64_t hits[256];
+    __shared__ float floors[256];
+    __shared__ int count;
     const PruneArgs &A = H.A;
-    const int lane = threadIdx.x & 31, K = A.K, D = A.D;
+    const int tid = threadIdx.x, K = A.K, D = A.D;
     const T *X = static_cast<const T *>(A.X);
-    for (int64_t i0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) & ~31ll; i0 < total;
-         i0 += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t i = i0 + lane;
-        bool hit = false;
-        float t = 0.f;
+    const int64_t total = A.rows * A.B;
+    for (int64_t i0 = (int64_t)blockIdx.x * 256; i0 < total; i0 += (int64_t)gridDim.x * 256) {
+        if (tid == 0) count = 0;
+        __syncthreads();
+        const int64_t i = i0 + tid;
         if (i < total) {
-            const float m = key_val(A.keys[i % A.B]);
-            t = screen_floor(m, A.c1, A.eps);
-            hit = A.tmax[i] >= t && !node_cut(m, H.gam, H.cut);
+            const float m = key_val(A.keys[i / A.rows]), t = screen_floor(m, A.c1, A.eps);
+            if (A.tmax[i] >= t && !node_cut(m, H.gam, H.cut)) {
+                const int o = atomicAdd(&count, 1);
+                hits[o] = i;
+                floors[o] = t;
+            }
         }
-        for (unsigned bal = __ballot_sync(0xffffffffu, hit); bal; bal &= bal - 1) {
-            const int src = __ffs(bal) - 1;
-            const int64_t q = i0 + src;
-            const float tq = __shfl_sync(0xffffffffu, t, src);
-            const int b = (int)(q % A.B);
-            const int64_t s0 = q / A.B * H.T, s1 = s0 + H.T < A.n ? s0 + H.T : A.n;
+        __syncthreads();
+        for (int o = 0; o < count; ++o) {
+            const int64_t q = hits[o];
+            const float tq = floors[o];
+            const int b = (int)(q / A.rows);
+            const int64_t s0 = q % A.rows * H.T, s1 = s0 + H.T < A.n ? s0 + H.T : A.n;
             const T *lo = static_cast<const T *>(A.lo) + (size_t)b * K * D;
             const T *hi = static_cast<const T *>(A.hi) + (size_t)b * K * D;
             double v = -1.0;
             uint32_t pos = 0xFFFFFFFFu;
-            for (int64_t s = s0; s < s1; s += 32 * U) {
+            for (int64_t s = s0 + tid; s < s1; s += 256 * U) {
                 float near[U];
 #pragma unroll
                 for (int u = 0; u < U; ++u) near[u] = __int_as_float(0x7f800000);
@@ -150,27 +159,28 @@ exact_hits_kernel(const HitArgs H, int64_t total)
                     for (int a = 0; a < D; ++a) {
                         float l, h, c[U];
                         if constexpr (F64) {
-                            const double o = A.off[a];
-                            l = __double2float_ru(__dsub_ru(lo[k * D + a], o));
-                            h = __double2float_rd(__dsub_rd(hi[k * D + a], o));
+                            const double f = A.off[a];
+                            l = __double2float_ru(__dsub_ru(lo[k * D + a], f));
+                            h = __double2float_rd(__dsub_rd(hi[k * D + a], f));
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
-                                const int64_t w = s + u * 32 + lane;
-                                c[u] = __double2float_rn(X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)] - o);
+                                const int64_t w = s + u * 256;
+                                c[u] = __double2float_rn(X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)] - f);
                             }
                         } else {
                             l = lo[k * D + a];
                             h = hi[k * D + a];
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
-                                const int64_t w = s + u * 32 + lane;
+                                const int64_t w = s + u * 256;
                                 c[u] = X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)];
                             }
                         }
 #pragma unroll
                         for (int u = 0; u < U; ++u) {
                             const float m = max3f(l - c[u], c[u] - h, 0.f);
-                            acc[a & 1][u] = fmaf(m, m, acc[a & 1][u]);
+                            if (a & 1) acc[1][u] = fmaf(m, m, acc[1][u]);
+                            else acc[0][u] = fmaf(m, m, acc[0][u]);
                         }
                     }
 #pragma unroll
@@ -178,15 +188,16 @@ exact_hits_kernel(const HitArgs H, int64_t total)
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const int64_t w = s + u * 32 + lane;
+                    const int64_t w = s + u * 256;
                     if (w < s1 && near[u] >= tq) {
                         const double e = exact_value<T>(X, A.ld, w, lo, hi, K, D);
                         if (e > v) { v = e; pos = (uint32_t)w; }   // (w increases)
                     }
                 }
             }
-            warp_raise128(&H.best[b], v, pos);
+            if (__any_sync(0xffffffffu, v >= 0.0)) warp_raise128(&H.best[b], v, pos);
         }
+        __syncthreads();
     }
 }
 
@@ -328,16 +339,16 @@ kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *
             const int64_t rows = (v.n + H.T - 1) / H.T;
             KC_TRY(ensure(c, c->tmax, (size_t)rows * B * 4));
             A.tmax = static_cast<float *>(c->tmax.p);
+            A.rows = rows;
             if (stream) KC_CUDA(c, launch_stream_f32(A, c->num_sms, c->stream));
             else KC_CUDA(c, prune_run(e, A, true, c->num_sms, c->smem_optin > 0 ? c->smem_optin : 48 * 1024, 0, c->stream));
             ++c->launches;
             H.gam = f64 ? -1.0 : gam;
             H.cut = cut;
             H.best = best;
-            const int64_t total = rows * B;
-            const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)c->num_sms * 8);
-            if (f64) exact_hits_kernel<double><<<grid, 256, 0, c->stream>>>(H, total);
-            else exact_hits_kernel<float><<<grid, 256, 0, c->stream>>>(H, total);
+            const int grid = (int)std::min<int64_t>((rows * B + 255) / 256, (int64_t)c->num_sms * 8);
+            if (f64) exact_hits_kernel<double><<<grid, 256, 0, c->stream>>>(H);
+            else exact_hits_kernel<float><<<grid, 256, 0, c->stream>>>(H);
             KC_TRY(after_launch(c, "exact maximum of the screened samples"));
         }
     }

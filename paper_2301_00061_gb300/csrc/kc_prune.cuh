@@ -59,7 +59,8 @@ struct PruneArgs {
     unsigned long long *keys; // [B] (value bits, ~position), zero before the launch
     // screens of an exact maximum (kc_exact.cu): the largest float value of each
     // node in each tile, of all samples that may attain the exact maximum
-    float *tmax;              // [tiles][B]
+    float *tmax;              // [B][rows], a row a tile
+    int64_t rows;
     float c1, eps;            // such a sample's float value reaches screen_floor(best, c1, eps)
     float cut;                // nodes proved to reach this float value are done
     const double *off;        // [D] double data: subtracted before the conversion to float
@@ -124,7 +125,8 @@ struct PruneLayout {
 // Distances of ST samples to one box (q.x = (lo_2p, lo_2p+1), q.y = (hi_2p, hi_2p+1)).
 // Each attribute's max(lo - x, x - hi, 0), squares in two interleaved fused
 // chains: the evaluation of box_dist_f32, with half the registers per sample.
-template <int ST, int P>
+// PT: the box is the point q.x (lo = hi); the same value, as |x - c| squared.
+template <int ST, int P, bool PT = false>
 __device__ __forceinline__ void box_dists(const uint64_t (&x)[ST][P], const ulonglong2 *bx, float (&d)[ST])
 {
     uint64_t acc[ST];
@@ -132,6 +134,15 @@ __device__ __forceinline__ void box_dists(const uint64_t (&x)[ST][P], const ulon
     for (int j = 0; j < ST; ++j) acc[j] = 0;
 #pragma unroll
     for (int p = 0; p < P; ++p) {
+        if constexpr (PT) {
+            const uint64_t c = bx[p].x;
+#pragma unroll
+            for (int j = 0; j < ST; ++j) {
+                const uint64_t t = sub2(x[j][p], c);
+                acc[j] = fma2(t, t, acc[j]);
+            }
+            continue;
+        }
         const ulonglong2 q = bx[p];
 #pragma unroll
         for (int j = 0; j < ST; ++j) {
@@ -214,17 +225,17 @@ __device__ __forceinline__ bool strip_refs(const uint8_t *rr, int lane, uint8_t 
 }
 
 // Distances of a strip to the boxes named by first[reference].
-template <int ST, int P>
+template <int ST, int P, bool PT = false>
 __device__ __forceinline__ void strip_dists(const uint64_t (&x)[ST][P], const ulonglong2 *rows, const uint8_t *first,
                                             const uint8_t (&rj)[ST], bool one, float (&d)[ST])
 {
     if (one) {
-        box_dists<ST, P>(x, rows + first[rj[0]] * row_words(P), d);
+        box_dists<ST, P, PT>(x, rows + first[rj[0]] * row_words(P), d);
     } else {
 #pragma unroll
         for (int j = 0; j < ST; ++j) {
             float e[1];
-            box_dists<1, P>(reinterpret_cast<const uint64_t (&)[1][P]>(x[j]), rows + first[rj[j]] * row_words(P), e);
+            box_dists<1, P, PT>(reinterpret_cast<const uint64_t (&)[1][P]>(x[j]), rows + first[rj[j]] * row_words(P), e);
             d[j] = e[0];
         }
     }
@@ -297,6 +308,7 @@ __global__ void __launch_bounds__(NT, 1)
 prune_max_kernel(const PruneArgs A)
 {
     constexpr int T = NT * ST, NWP = NT / 32, RW = row_words(P), CAP = pair_cap(P);
+    constexpr bool PT = TM && !F64;   // float screens are of center sets
     constexpr unsigned ALL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smem[];
     const int K = A.K, D = A.D, KP = K * P, KR = K * RW;
@@ -509,7 +521,7 @@ prune_max_kernel(const PruneArgs A)
                 float best = INF;
                 for (int k = 0; k < K; ++k) {
                     float d[1];
-                    box_dists<1, P>(xc, box + ((size_t)b * K + k) * RW, d);
+                    box_dists<1, P, PT>(xc, box + ((size_t)b * K + k) * RW, d);
                     best = fminf(best, d[0]);
                 }
                 raise(b, key_max(best, (uint32_t)cp));
@@ -584,9 +596,10 @@ prune_max_kernel(const PruneArgs A)
             uint8_t rj[ST];
             const bool one = strip_refs(rr + q0, lane, rj);
             unsigned m = 0u;   // bit i ST + j: sample j may matter in node bg + i
+#pragma unroll(P <= 4 ? 2 : 1)
             for (int i = 0; i < nn; ++i) {
                 float d[ST];
-                strip_dists<ST, P>(y, box + (bg + i) * KR, fk + (bg + i) * K, rj, one, d);
+                strip_dists<ST, P, PT>(y, box + (bg + i) * KR, fk + (bg + i) * K, rj, one, d);
                 const float t = thr[bg + i];
                 unsigned mi = 0u;
 #pragma unroll
@@ -604,10 +617,10 @@ prune_max_kernel(const PruneArgs A)
                 const int b = bg + i;
                 if (!__any_sync(ALL, (m >> (i * ST) & ((1u << ST) - 1u)) != 0u)) continue;
                 float v[ST];
-                box_dists<ST, P>(y, box + b * KR, v);
+                box_dists<ST, P, PT>(y, box + b * KR, v);
                 for (int k = 1; k < K; ++k) {
                     float e[ST];
-                    box_dists<ST, P>(y, box + b * KR + k * RW, e);
+                    box_dists<ST, P, PT>(y, box + b * KR + k * RW, e);
 #pragma unroll
                     for (int j = 0; j < ST; ++j) v[j] = fminf(v[j], e[j]);
                 }
@@ -635,7 +648,7 @@ prune_max_kernel(const PruneArgs A)
             for (int i = 0; i < kPG; ++i) {
                 const int b = min(bg + i, nb - 1);
                 float d[1];
-                box_dists<1, P>(y, box + b * KR + fk[b * K + rs] * RW, d);
+                box_dists<1, P, PT>(y, box + b * KR + fk[b * K + rs] * RW, d);
                 if (on && bg + i < nb && d[0] >= thr[b]) m |= 1u << i;
             }
             const int c = (int)__reduce_add_sync(ALL, (unsigned)__popc(m));
@@ -648,7 +661,7 @@ prune_max_kernel(const PruneArgs A)
                 float v = INF;
                 for (int k = 0; k < K; ++k) {
                     float d[1];
-                    box_dists<1, P>(y, box + b * KR + k * RW, d);
+                    box_dists<1, P, PT>(y, box + b * KR + k * RW, d);
                     v = fminf(v, d[0]);
                 }
                 lift(b, v, spos[slot]);
@@ -667,7 +680,7 @@ prune_max_kernel(const PruneArgs A)
             float v = INF;
             for (int k = 0; k < K; ++k) {
                 float d[1];
-                box_dists<1, P>(y, box + b * KR + k * RW, d);
+                box_dists<1, P, PT>(y, box + b * KR + k * RW, d);
                 v = fminf(v, d[0]);
             }
             lift(b, v, spos[slot]);
@@ -679,7 +692,7 @@ prune_max_kernel(const PruneArgs A)
             const unsigned long long k = key[b];
             if (k > peek(&A.keys[b0 + b])) atomicMax(&A.keys[b0 + b], k);
             if constexpr (TM) {
-                A.tmax[(size_t)tile * A.B + b0 + b] = __uint_as_float(tmx[b]);
+                A.tmax[(size_t)(b0 + b) * A.rows + tile] = __uint_as_float(tmx[b]);
                 tmx[b] = 0u;
             }
         }

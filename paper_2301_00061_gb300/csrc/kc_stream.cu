@@ -195,7 +195,7 @@ stream_max_small(const PruneArgs A)
                 const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(max_of<ST>(m)));
                 if ((threadIdx.x & 31) == 0) {
                     const int64_t row = (base >> 7) + (threadIdx.x >> 5);
-                    if (row * kStreamTile < A.n) A.tmax[row * A.B + b] = __uint_as_float(w);
+                    if (row * kStreamTile < A.n) A.tmax[b * A.rows + row] = __uint_as_float(w);
                     const unsigned long long key = ((unsigned long long)w << 32) | 1ull;
                     if (key > mine[b]) mine[b] = key;
                 }
@@ -294,7 +294,7 @@ stream_max_wide(const PruneArgs A)
                     const unsigned w = __reduce_max_sync(0xffffffffu, __float_as_uint(max_of<4>(d)));
                     const int64_t row = (base >> 7) + (threadIdx.x >> 5);
                     if ((threadIdx.x & 31) == 0 && row * kStreamTile < A.n)
-                        A.tmax[row * A.B + (c == K - 1 ? 0 : 1)] = __uint_as_float(w);
+                        A.tmax[(c == K - 1 ? 0 : A.rows) + row] = __uint_as_float(w);
                     best.v = fmaxf(best.v, __uint_as_float(w));
                 } else {
                     best.take<1>(d, s0, A.n);
