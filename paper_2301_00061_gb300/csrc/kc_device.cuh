@@ -152,4 +152,34 @@ __device__ __forceinline__ void list_item(const int64_t *__restrict__ tile_prefi
     *start_out = (int64_t)(w - tile_prefix[lo]) * tile;
 }
 
+// ---- 128-bit keys (ordered value, ~position): double values with positions
+
+__device__ __forceinline__ ulonglong2 cas128(ulonglong2 *p, ulonglong2 c, ulonglong2 v)
+{
+    ulonglong2 r;
+    asm volatile("{ .reg .b128 c, v, r;\n"
+                 "mov.b128 c, {%2, %3};\n"
+                 "mov.b128 v, {%4, %5};\n"
+                 "atom.global.cas.b128 r, [%6], c, v;\n"
+                 "mov.b128 {%0, %1}, r; }"
+                 : "=l"(r.x), "=l"(r.y)
+                 : "l"(c.x), "l"(c.y), "l"(v.x), "l"(v.y), "l"(p)
+                 : "memory");
+    return r;
+}
+
+// Raises *p (16-byte aligned) to (value, rest).  Each failed exchange means
+// another thread raised it, so this ends.
+__device__ __forceinline__ void raise_key128(ulonglong2 *p, unsigned long long value, unsigned long long rest)
+{
+    const ulonglong2 k = make_ulonglong2(value, rest);
+    ulonglong2 cur = make_ulonglong2(0ull, 0ull);
+    for (;;) {
+        const ulonglong2 old = cas128(p, cur, k);
+        if (old.x == cur.x && old.y == cur.y) return;
+        cur = old;
+        if (!(k.x > cur.x || (k.x == cur.x && k.y > cur.y))) return;
+    }
+}
+
 }  // namespace kc

@@ -36,32 +36,9 @@ namespace kc {
 
 namespace {
 
-// (ordered value, ~position) of a node's exact maximum.
-__device__ __forceinline__ ulonglong2 cas128(ulonglong2 *p, ulonglong2 c, ulonglong2 v)
-{
-    ulonglong2 r;
-    asm volatile("{ .reg .b128 c, v, r;\n"
-                 "mov.b128 c, {%2, %3};\n"
-                 "mov.b128 v, {%4, %5};\n"
-                 "atom.global.cas.b128 r, [%6], c, v;\n"
-                 "mov.b128 {%0, %1}, r; }"
-                 : "=l"(r.x), "=l"(r.y)
-                 : "l"(c.x), "l"(c.y), "l"(v.x), "l"(v.y), "l"(p)
-                 : "memory");
-    return r;
-}
-
-// Each failed exchange means another CTA raised the key, so this ends.
 __device__ __forceinline__ void raise128(ulonglong2 *p, double v, uint32_t pos)
 {
-    const ulonglong2 k = make_ulonglong2(ord_f64(v), 0xFFFFFFFFull - pos);
-    ulonglong2 cur = make_ulonglong2(0ull, 0ull);
-    for (;;) {
-        const ulonglong2 old = cas128(p, cur, k);
-        if (old.x == cur.x && old.y == cur.y) return;
-        cur = old;
-        if (!(k.x > cur.x || (k.x == cur.x && k.y > cur.y))) return;
-    }
+    raise_key128(p, ord_f64(v), 0xFFFFFFFFull - pos);
 }
 
 __device__ __forceinline__ void warp_raise128(ulonglong2 *p, double v, uint32_t pos)

@@ -7,9 +7,11 @@
 // register accumulators, then reduces them across the warp once per (node,
 // tile) and merges them into global accumulators with atomics.  Extremes that
 // must also name a sample (the representatives) are (value, position) keys:
-// packed into 64 bits and merged with 64-bit atomics for float data; for
-// double data (two words) the kernels run as one CTA whose warps own disjoint
-// nodes, and the owning lane merges them without atomics.
+// packed into 64 bits and merged with 64-bit atomics for float data, two words
+// merged with 128-bit compare-and-swap for double data (when those kernels ran
+// as one CTA, to have a single writer, 256 nodes over 1000 samples took 5.4 ms
+// a call against 0.14 ms).  A work unit is a tile and a share of the nodes, so that few
+// tiles still fill the SMs and many end together.
 //
 // Float data take every exclusion only where the float evaluation proves it:
 // a distance d evaluated as d' satisfies d' (1 - g) <= d <= d' / (1 - g), so
@@ -47,7 +49,7 @@ struct Key<float> {
     __device__ static void atomic_max(K *p, const K &v, unsigned *) { atomicMax(p, v); }
 };
 
-struct K128 {
+struct __align__(16) K128 {
     unsigned long long hi, lo;
 };
 
@@ -66,14 +68,10 @@ struct Key<double> {
     __device__ static double vmax(const K &k) { return unord_f64(k.hi); }
     __device__ static double vmin(const K &k) { return unord_f64(~k.hi); }
     __device__ static uint32_t pos(const K &k) { return (uint32_t)(0xFFFFFFFFull - k.lo); }
-    // Double keys do not fit one 64-bit atomic.  The double-data kernels run
-    // as a single CTA in which node b belongs to warp b % 8 alone, so lane 0
-    // of that warp is the only writer of the node's keys: a plain
-    // read-compare-write merge is race-free there.
+    // 128-bit compare-and-swap; a key read as equal or larger costs one exchange
     __device__ static void atomic_max(K *p, const K &v, unsigned *)
     {
-        const K cur = *p;
-        if (gt(v, cur)) *p = v;
+        raise_key128(reinterpret_cast<ulonglong2 *>(p), v.hi, v.lo);
     }
 };
 
@@ -333,17 +331,23 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
     acc_lb = warp_kmax<T>(acc_lb);
     if (lane == 0 && !KT::is_none(acc_lb)) KT::atomic_max(&lbkey[b], acc_lb, &flags[b]);
     if constexpr (!F32) {
+        // one key to a lane: their exchanges overlap
+        KY own = KT::none();
+        KY *at = nullptr;
+        int i = 0;
 #pragma unroll
         for (int k = 0; k < KM; ++k)
 #pragma unroll
             for (int a = 0; a < DM; ++a)
                 if (k < K && a < D) {
-                    const KY m1 = warp_kmax<T>(acc_max[k][a]);
-                    const KY m2 = warp_kmax<T>(acc_min[k][a]);
                     const size_t o = ((size_t)b * K + k) * D + a;
-                    if (lane == 0 && !KT::is_none(m1)) KT::atomic_max(&amax[o], m1, &flags[b]);
-                    if (lane == 0 && !KT::is_none(m2)) KT::atomic_max(&amin[o], m2, &flags[b]);
+                    const KY m1 = warp_kmax<T>(acc_max[k][a]), m2 = warp_kmax<T>(acc_min[k][a]);
+                    if (lane == i) { own = m1; at = &amax[o]; }
+                    if (lane == i + 1) { own = m2; at = &amin[o]; }
+                    i += 2;
                 }
+        static_assert(2 * KM * DM <= 32 || F32, "one key to a lane");
+        if (at && !KT::is_none(own)) KT::atomic_max(at, own, &flags[b]);
     }
     if (__any_sync(0xffffffffu, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
     if constexpr (F32) {
@@ -381,7 +385,7 @@ __device__ __forceinline__ void stage_tile_a(const T *__restrict__ X, int64_t ld
 
 template <typename T, int KM, int DM>
 __global__ void __launch_bounds__(kThreads)
-visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, const T *__restrict__ lo,
+visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, const T *__restrict__ lo,
                const T *__restrict__ hi, int B, int K, int D, double alpha, Margins mg,
                typename Key<T>::K *__restrict__ lbkey, typename Key<T>::K *__restrict__ amax,
                typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags, int ndir,
@@ -396,12 +400,14 @@ visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, const T
                       reinterpret_cast<unsigned long long *>(smem + (size_t)D * tile * 8) +
                           (size_t)warp * warp_key_words(K, D, ndir),
                       dmax, dmin};
-    for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
+    const int64_t units = (n + tile - 1) / tile * split;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const int64_t base = u / split * tile;
         const int tn = (int)((n - base) < (int64_t)tile ? (n - base) : (int64_t)tile);
         __syncthreads();
         stage_tile_a<T>(X, ld, D, tile, tn, base, nullptr, tp, td);
         __syncthreads();
-        for (int b = warp; b < B; b += NWV)
+        for (int b = (int)(u % split) * NWV + warp; b < B; b += split * NWV)
             pass_a_node<T, KM, DM>(tp, td, tile, tn, lane, 32, nullptr, base, lo, hi, b, K, D, alpha, mg, lbkey, amax,
                                    amin, flags, dk);
     }
@@ -883,7 +889,7 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
 
 template <typename T, int KM, int DM>
 __global__ void __launch_bounds__(kThreads, 3)
-visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int B, int K, int D, int RM,
+visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, int B, int K, int D, int RM,
                const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
                const T *__restrict__ bhi, const T *__restrict__ repx, const int *__restrict__ nreps,
                const int *__restrict__ allhave, double alpha, Margins mg, const int64_t *__restrict__ seeds,
@@ -901,7 +907,9 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int B, 
     const int warp = threadIdx.x >> 5;
     uint32_t *list = lists + warp * kSub;
     uint64_t *wrep = reinterpret_cast<uint64_t *>(slots + NWV) + (size_t)warp * KM * RM * rep_words<T, DM>();
-    for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
+    const int64_t units = (n + tile - 1) / tile * split;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+        const int64_t base = u / split * tile;
         const int tn = (int)((n - base) < (int64_t)tile ? (n - base) : (int64_t)tile);
         __syncthreads();
         for (int i = threadIdx.x; i < D * tile; i += kThreads) {
@@ -909,7 +917,7 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int B, 
             tx[i] = j < tn ? X[(size_t)a * ld + base + j] : T(0);
         }
         __syncthreads();
-        for (int b = warp; b < B; b += NWV)
+        for (int b = (int)(u % split) * NWV + warp; b < B; b += split * NWV)
             pass_b_node<T, KM, DM>(tx, tile, tn, 0, 32, nullptr, ids, base, list, slots + warp, wrep, b, K, D, RM,
                                         lo_in, hi_in, blo, bhi, repx, nreps, allhave, alpha, mg, seed_id, cnt, smax,
                                         smin, jmax, jmin, cand, flags);
@@ -1133,6 +1141,18 @@ kc_status grid_of(kc_ctx *c, F fn, size_t smem, int64_t work, int *grid)
     return KC_OK;
 }
 
+// Samples per tile (at most most, a multiple of 32) and shares of the nodes per
+// tile for n samples and B nodes: small data take tiles down to 256 samples, and
+// the units (tiles x shares, a share at least a node per warp) come to eight
+// per SM and more, so that the last round leaves little idle.
+void tile_units(const kc_ctx *c, int64_t n, int B, int most, int *tile, int *split)
+{
+    const int64_t want = (n / (2 * c->num_sms) + 31) / 32 * 32;
+    *tile = (int)std::max<int64_t>(256, std::min<int64_t>(most, want));
+    const int64_t tiles = std::max<int64_t>(1, (n + *tile - 1) / *tile);
+    *split = (int)std::max<int64_t>(1, std::min<int64_t>((B + NWV - 1) / NWV, (24 * c->num_sms + tiles - 1) / tiles));
+}
+
 Margins make_margins(kc_ctx *c, double alpha, double beta_glob)
 {
     Margins m{};
@@ -1223,11 +1243,13 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const Margins mg = make_margins(c, alpha, 0.0);
     const double r_up = nextafter(std::sqrt(alpha), __builtin_huge_val());
     // pass A
-    const int tileA = (int)std::max<int64_t>(256, std::min<int64_t>(2048, (64 * 1024) / (D * 8)) / 32 * 32);
+    int tileA, splitA;
+    tile_units(c, v.n, B, (int)std::max<int64_t>(256, std::min<int64_t>(2048, (64 * 1024) / (D * 8)) / 32 * 32), &tileA,
+               &splitA);
     const size_t dkA = sizeof(T) == 4 ? (size_t)NWV * warp_key_words(K_, D, ndir) * 8 : 0;   // per-warp key slots
     const size_t smemA = (size_t)D * tileA * 8 + dkA;
     int gA = 1;
-    const int64_t tilesA = (v.n + tileA - 1) / tileA;
+    const int64_t unitsA = (v.n + tileA - 1) / tileA * splitA;
     auto kA = visit_a_kernel<T, KM, DM>;
     if (L) {
         // list mode (float data): one node per work item, tile = list_tile() gathered ids
@@ -1246,10 +1268,9 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
             return set_err(c, KC_EINTERNAL, "list-mode tightening is for float data");
         }
     } else {
-        KC_TRY(grid_of(c, kA, smemA, tilesA, &gA));
-        if (sizeof(T) == 8) gA = 1;   // single-writer key merge (see Key<double>)
+        KC_TRY(grid_of(c, kA, smemA, unitsA, &gA));
         if (v.n > 0) {
-            kA<<<gA, kThreads, smemA, c->stream>>>(static_cast<const T *>(v.X), v.ld, v.n, tileA, lo, hi, B, K_, D,
+            kA<<<gA, kThreads, smemA, c->stream>>>(static_cast<const T *>(v.X), v.ld, v.n, tileA, splitA, lo, hi, B, K_, D,
                                                   alpha, mg, lbkey, amax, amin, flags, ndir, dmax, dmin);
             KC_TRY(after_launch(c, "tighten pass A"));
         }
@@ -1272,7 +1293,10 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
         repx, have, lb, lb_raw, lbarg);
     KC_TRY(after_launch(c, "tighten finalize A"));
     // pass B
-    const int tileB = (int)std::max<int64_t>(256, std::min<int64_t>(2048, (32 * 1024) / (D * (int64_t)sizeof(T))) / 32 * 32);
+    int tileB, splitB;
+    tile_units(c, v.n, B,
+               (int)std::max<int64_t>(256, std::min<int64_t>(2048, (32 * 1024) / (D * (int64_t)sizeof(T))) / 32 * 32),
+               &tileB, &splitB);
     static_assert(kThreads / 32 * kSub * 4 <= 16 * 1024, "pass B lists");
     const size_t slotB = (size_t)NWV * sizeof(PBSlot<T, KM, DM>);
     const size_t repB = (size_t)NWV * KM * RM * rep_words<T, DM>() * 8;   // per-warp representatives
@@ -1294,10 +1318,9 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
             }
         }
     } else {
-    KC_TRY(grid_of(c, kB, smemB, (v.n + tileB - 1) / tileB, &gB));
-    if (sizeof(T) == 8) gB = 1;   // single-writer key merge (see Key<double>)
+    KC_TRY(grid_of(c, kB, smemB, (v.n + tileB - 1) / tileB * splitB, &gB));
     if (v.n > 0) {
-        kB<<<gB, kThreads, smemB, c->stream>>>(static_cast<const T *>(v.X), v.ld, v.n, tileB, B, K_, D, RM, lo, hi, blo,
+        kB<<<gB, kThreads, smemB, c->stream>>>(static_cast<const T *>(v.X), v.ld, v.n, tileB, splitB, B, K_, D, RM, lo, hi, blo,
                                               bhi, repx, nreps, have, alpha, mg, seeds, v.ids, cnt, smax, smin, jmax, jmin,
                                               cand, flags);
         KC_TRY(after_launch(c, "tighten pass B"));
