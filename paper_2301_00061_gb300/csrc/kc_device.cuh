@@ -182,4 +182,26 @@ __device__ __forceinline__ void raise_key128(ulonglong2 *p, unsigned long long v
     }
 }
 
+// ---- is some representative of a cluster farther than a threshold T?
+// Float decision: some evaluated distance d' > T.  With c near the centroid of
+// the representatives (within err), radius the largest distance from c to one,
+// and d' off by a relative g at most, an evaluated distance dc from a sample to c
+//   <= near: (sqrt(d) + radius)^2 bounds every distance, so none is above T;
+//   >  far:  a ball about the sample that holds every representative holds their
+//            centroid, so some distance is at least (sqrt(d) - err)^2, above T;
+// and only between the two are the representatives scanned.  g4 = 4 g covers the
+// evaluations of dc and of the representatives' distances.
+struct BallTest {
+    float near, far;
+};
+__device__ __forceinline__ BallTest ball_test(float T, float radius, float err, float g4)
+{
+    BallTest b;
+    const float s = __fsub_rd(__fsqrt_rd(__fmul_rd(T, __fsub_rd(1.f, g4))), radius);
+    b.near = s > 0.f ? __fmul_rd(__fmul_rd(s, s), __fsub_rd(1.f, g4)) : -1.f;
+    const float t = __fadd_ru(__fsqrt_ru(__fmul_ru(T, __fadd_ru(1.f, g4))), err);
+    b.far = fmaxf(__fmul_ru(__fmul_ru(t, t), __fadd_ru(1.f, g4)), 1e-30f);
+    return b;
+}
+
 }  // namespace kc

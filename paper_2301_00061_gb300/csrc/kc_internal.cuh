@@ -34,6 +34,7 @@ struct VisitScratch {
     const int64_t *reps = nullptr;   // [B][K][RM] representative sample ids (-1 unused)
     const int *nreps = nullptr;      // [B][K]
     const void *repx = nullptr;      // [B][K][RM][D] their coordinates
+    const float *ball = nullptr;     // [B][K][D + 2] a ball around them (float data, BallTest)
     int RM = 0;
 };
 
@@ -168,6 +169,7 @@ struct Margins {
     // single-compare proofs: a float distance d' > t_alpha proves d > alpha,
     // d' > t_four proves d > 4 alpha (t = RU((RU(target) + slack) / defl * (1 + 1e-6)))
     float t_alpha, t_four;
+    float g4;                    // 4 g, rounded up
 };
 
 // Per-node sample-id lists of a batch of nodes (device arrays).  Nodes that
@@ -256,7 +258,7 @@ kc_status launch_wide_a(kc_ctx *c, const View &v, const ListBatch *L, const floa
                         unsigned long long *dmin);
 kc_status launch_wide_b(kc_ctx *c, const View &v, const ListBatch *L, const float *lo, const float *hi, int B,
                         const Margins &mg, const float *blo, const float *bhi, const float *repx, const int *nreps,
-                        const int *allhave, const int64_t *seeds, int RM, unsigned long long *cnt,
+                        const int *allhave, const float *ball, const int64_t *seeds, int RM, unsigned long long *cnt,
                         unsigned long long *cand, unsigned *smax, unsigned *smin, unsigned *jmax, unsigned *jmin,
                         unsigned *flags);
 
@@ -351,7 +353,8 @@ kc_status launch_seg_refine(kc_ctx *c, const ListBatch &L, const void *lo, const
 kc_status launch_seg_objective(kc_ctx *c, const ListBatch &L, const int64_t *centers, int B, double alpha_cut,
                                unsigned long long *keys, unsigned long long *vmax, float *thr, double *val);
 kc_status launch_seg_filter(kc_ctx *c, const ListBatch &L, const void *lo, const void *hi, int B,
-                            const float *beta_dn_dev, double alpha, const void *repx, const int *nreps, int RM,
+                            const float *beta_dn_dev, double alpha, const void *repx, const int *nreps,
+                            const float *ball, int RM,
                             const int *rmap, uint32_t *out_pool, const int64_t *out_off, const int64_t *out_cap,
                             unsigned long long *out_n, const int *cvar, const float *csplit,
                             unsigned long long *ckeys, double *child_lb, double *child_raw, int64_t *child_arg);

@@ -284,8 +284,8 @@ template <int DMAX>
 __global__ void __launch_bounds__(256)
 seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float *__restrict__ lo,
                const float *__restrict__ hi, int K, int D, const float *__restrict__ beta_dn, float infl, float slack,
-               float t_alpha, const float *__restrict__ repx, const int *__restrict__ nreps, int RM,
-               const int *__restrict__ rmap, uint32_t *__restrict__ out_pool, const int64_t *__restrict__ out_off,
+               float t_alpha, float g4, const float *__restrict__ repx, const int *__restrict__ nreps,
+               const float *__restrict__ ball, int RM, const int *__restrict__ rmap, uint32_t *__restrict__ out_pool, const int64_t *__restrict__ out_off,
                const int64_t *__restrict__ out_cap, unsigned long long *__restrict__ out_n,
                const int *__restrict__ cvar, const float *__restrict__ csplit, unsigned long long *__restrict__ ckeys)
 {
@@ -294,6 +294,8 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
     __shared__ float sl[kMaxK * DMAX], sh[kMaxK * DMAX];
     __shared__ unsigned long long red[8];
     __shared__ int snr[kMaxK];
+    __shared__ BallTest sball[kMaxK];              // the representatives' balls against alpha
+    __shared__ uint64_t sc0[kMaxK * DMAX / 2];
     // the node's representatives as packed coordinate pairs [K][RM][Dp / 2]
     extern __shared__ uint64_t srep[];
     const int Dp = (D + 1) & ~1, H = Dp / 2;
@@ -314,12 +316,22 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
         }
         const size_t rb = rmap ? (size_t)rmap[b] : (size_t)b;   // row of the node's representatives
         for (int k = threadIdx.x; k < K; k += blockDim.x) snr[k] = nreps ? nreps[rb * K + k] : 0;
-        if (nreps)
+        if (nreps) {
+            for (int k = threadIdx.x; k < K; k += blockDim.x) {
+                const float *c = ball + (rb * K + k) * (D + 2) + D;
+                sball[k] = ball_test(t_alpha, c[0], c[1], g4);
+            }
+            for (int i = threadIdx.x; i < K * H; i += blockDim.x) {
+                const int k = i / H, p = i % H;
+                const float *c = ball + (rb * K + k) * (D + 2);
+                sc0[i] = pk(c[2 * p], 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
+            }
             for (int i = threadIdx.x; i < K * RM * H; i += blockDim.x) {
                 const int k = i / (RM * H), r = (i / H) % RM, p = i % H;
                 const float *c = repx + ((rb * K + k) * RM + r) * D;
                 if (r < nreps[rb * K + k]) srep[i] = pk(c[2 * p], 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
             }
+        }
         __syncthreads();
         const float bth = beta_dn[b];
         // the children's split: box ks, attribute as_, at (cm | cs)
@@ -366,8 +378,22 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                         if (x[a] < sl[k * D + a] || x[a] > sh[k * D + a]) inb = false;
                     if (!inb) continue;
                     bool excl = false;
-                    const int nr = snr[k];
+                    int nr = snr[k];
                     const uint64_t *ck = srep + (size_t)k * RM * H;
+                    if (nr > 0) {
+                        // the ball decides most samples
+                        uint64_t acc = 0;
+#pragma unroll
+                        for (int p = 0; p < DMAX / 2; ++p)
+                            if (p < H) {
+                                const uint64_t t = sub2(pxx[p], sc0[k * H + p]);
+                                acc = fma2(t, t, acc);
+                            }
+                        const float2 s2 = upk(acc);
+                        const float dc = s2.x + s2.y;
+                        if (dc > sball[k].far) excl = true;
+                        if (dc <= sball[k].near) nr = 0;
+                    }
                     // chunks of 4 representatives decided by their largest distance
                     // (a short last chunk repeats the last representative)
                     for (int r0 = 0; r0 < nr && !excl; r0 += 4) {
@@ -579,7 +605,8 @@ kc_status launch_seg_objective(kc_ctx *c, const ListBatch &L, const int64_t *cen
 }
 
 kc_status launch_seg_filter(kc_ctx *c, const ListBatch &L, const void *lo, const void *hi, int B,
-                            const float *beta_dn_dev, double alpha, const void *repx, const int *nreps, int RM,
+                            const float *beta_dn_dev, double alpha, const void *repx, const int *nreps,
+                            const float *ball, int RM,
                             const int *rmap, uint32_t *out_pool, const int64_t *out_off, const int64_t *out_cap,
                             unsigned long long *out_n, const int *cvar, const float *csplit,
                             unsigned long long *ckeys, double *child_lb, double *child_raw, int64_t *child_arg)
@@ -598,14 +625,16 @@ kc_status launch_seg_filter(kc_ctx *c, const ListBatch &L, const void *lo, const
     if ((double)aup < alpha) aup = nextafterf(aup, 3.4e38f);
     float t_alpha = (float)(((double)aup + (double)slack) / (double)defl * (1.0 + 1e-6));
     if ((double)t_alpha < ((double)aup + (double)slack) / (double)defl * (1.0 + 1e-6)) t_alpha = nextafterf(t_alpha, 3.4e38f);
+    float g4 = (float)(4.0 * g);
+    if ((double)g4 < 4.0 * g) g4 = nextafterf(g4, 1.f);
     const int gr = grid_items(c, L.W);
     const size_t srep = nreps ? (size_t)c->K * RM * (((c->D + 1) & ~1) / 2) * 8 : 0;
     if (srep > 48 * 1024)
         KC_CUDA(c, cudaFuncSetAttribute(seg_filter_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srep));
     seg_filter_f32<8><<<gr, 256, srep, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                  static_cast<const float *>(lo), static_cast<const float *>(hi), c->K,
-                                                 c->D, beta_dn_dev, infl, slack, t_alpha,
-                                                 static_cast<const float *>(repx), nreps, RM, rmap, out_pool, out_off,
+                                                 c->D, beta_dn_dev, infl, slack, t_alpha, g4,
+                                                 static_cast<const float *>(repx), nreps, ball, RM, rmap, out_pool, out_off,
                                                  out_cap, out_n, cvar, csplit, ckeys);
     KC_TRY(after_launch(c, "list filter"));
     if (ckeys) {

@@ -941,7 +941,7 @@ kc_status solve_impl(kc_ctx *c, const kc_solve_opts &o, kc_result *res)
                 KC_TRY(make_lb(3, nf, [&](int q) { return batch[rows[q]].list; }, rows.data(), &Lf, &rows_dev));
                 const bool bt = o.use_bt != 0;
                 KC_TRY(launch_seg_filter(c, Lf, d_llo, d_lhi, nf, d_beta, alpha, bt ? c->vs.repx : nullptr,
-                                         bt ? c->vs.nreps : nullptr, c->vs.RM, rows_dev, arena.ids(), d_outoff,
+                                         bt ? c->vs.nreps : nullptr, bt ? c->vs.ball : nullptr, c->vs.RM, rows_dev, arena.ids(), d_outoff,
                                          d_outcap, d_outn, d_cvar, d_csplit, d_ckeys, d_clb, d_craw, d_carg));
                 std::vector<unsigned long long> kept(nf);
                 flb.resize((size_t)2 * nf);
@@ -1015,7 +1015,7 @@ kc_status solve_impl(kc_ctx *c, const kc_solve_opts &o, kc_result *res)
                         const int *rows2_dev = nullptr;
                         KC_TRY(make_lb(3, n2, [&](int t) { return batch[rows2[t]].list; }, rows2.data(), &L2, &rows2_dev));
                         KC_TRY(launch_seg_filter(c, L2, d_llo, d_lhi, n2, d_beta, alpha, bt ? c->vs.repx : nullptr,
-                                                 bt ? c->vs.nreps : nullptr, c->vs.RM, rows2_dev, arena.ids(), d_outoff,
+                                                 bt ? c->vs.nreps : nullptr, bt ? c->vs.ball : nullptr, c->vs.RM, rows2_dev, arena.ids(), d_outoff,
                                                  d_outcap, d_outn, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr));
                         std::vector<unsigned long long> kept2(n2);
                         KC_CUDA(c, cudaMemcpyAsync(kept2.data(), d_outn, (size_t)n2 * 8, cudaMemcpyDeviceToHost, c->stream));

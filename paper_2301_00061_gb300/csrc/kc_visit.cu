@@ -186,8 +186,10 @@ __device__ __forceinline__ bool proved_lt(float dhat, float infl, float slack, f
 // was gathered from a list of sample ids, else by its position base + j.
 
 // Float data keep the node's arg-extreme keys in the warp's shared-memory
-// slot sk, updated with atomics that a plain read skips when they cannot
-// change the value, and merged into global memory at the end of the node:
+// slot sk: they start from the global ones (what every tile so far has raised),
+// are updated with atomics that a plain read skips when they cannot change the
+// value, and are merged into global memory at the end of the node if any was
+// raised:
 // per cluster and attribute (max, min) at sk [K][D][2], then, with ndir > 0,
 // per cluster and pair direction at sk [2KD + (k ndir + q) 2] -- the keys of
 // x_a + x_b and x_a - x_b (added in float) for the first ndir / 2 attribute
@@ -199,25 +201,70 @@ struct WarpKeys {
     unsigned long long *__restrict__ dmax, *__restrict__ dmin;
 };
 
-// u64 words of a warp's key slot
-__host__ __device__ constexpr int warp_key_words(int K, int D, int ndir) { return 2 * K * D + 2 * K * ndir; }
+// u64 words of a warp's key slot: the keys, then a (lo, hi) pair of floats per
+// cluster and attribute (its core)
+__host__ __device__ constexpr int warp_key_words(int K, int D, int ndir) { return 2 * K * D + 2 * K * ndir + K * D; }
+
+// The core of cluster k: an open box in which no sample can raise a key of the
+// cluster, so that an assigned sample is one test of D intervals instead of
+// D + ndir pairs of compares (an assigned sample took about 200 instructions, and
+// all but one in a thousand lie in the core once the first tiles are in).  The
+// attributes' ranges shrunk about their middles by one factor until every pair
+// direction's extremes lie outside: x_a < H_a and x_b < H_b give
+// fl(x_a + x_b) <= fl(H_a + H_b), which is checked to be below the key.
+__device__ __forceinline__ void core_of(const unsigned long long *sk, int k, int K, int D, int ndir, uint64_t *core)
+{
+    using KT = Key<float>;
+    const int lane = threadIdx.x & 31;
+    const unsigned long long *sa = sk + (size_t)k * D * 2, *sd = sk + (size_t)2 * K * D + (size_t)k * ndir * 2;
+    const float INF = __int_as_float(0x7f800000);
+    bool ok = sa[0] != 0ull;
+    float t = 1.f;
+    auto mid = [&](int a) { return 0.5f * KT::vmax(sa[2 * a]) + 0.5f * KT::vmin(sa[2 * a + 1]); };
+    auto half = [&](int a) { return 0.5f * KT::vmax(sa[2 * a]) - 0.5f * KT::vmin(sa[2 * a + 1]); };
+    int pa = 0, pb = 0;
+    const bool pair = ok && lane < ndir / 2;
+    float smx = 0.f, smn = 0.f, dmx = 0.f, dmn = 0.f;
+    if (pair) {
+        int r = lane;
+        while (r >= D - 1 - pa) r -= D - 1 - pa++;
+        pb = pa + 1 + r;
+        const unsigned long long *q = sd + 4 * lane;   // sum (max, min), difference (max, min)
+        smx = KT::vmax(q[0]), smn = KT::vmin(q[1]), dmx = KT::vmax(q[2]), dmn = KT::vmin(q[3]);
+        const float ms = mid(pa) + mid(pb), md = mid(pa) - mid(pb), w = half(pa) + half(pb);
+        t = 0.999f * fminf(fminf(smx - ms, ms - smn), fminf(dmx - md, md - dmn)) / w;
+        if (!(t > 0.f)) t = 0.f;   // (also 0 / 0)
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
+    auto low = [&](int a) { return fmaxf(mid(a) - t * half(a), KT::vmin(sa[2 * a + 1])); };
+    auto high = [&](int a) { return fminf(mid(a) + t * half(a), KT::vmax(sa[2 * a])); };
+    if (pair) {
+        const float la = low(pa), ha = high(pa), lb = low(pb), hb = high(pb);
+        ok = __fadd_rn(ha, hb) < smx && __fadd_rn(la, lb) > smn && __fsub_rn(ha, lb) < dmx && __fsub_rn(la, hb) > dmn;
+    }
+    ok = __all_sync(0xffffffffu, ok) && t > 0.f;
+    if (lane < D) core[k * D + lane] = ok ? pk(low(lane), high(lane)) : pk(INF, -INF);
+}
 
 // Raise the float key at `slot` (max) and `slot + 1` (min) by value v of the
 // sample at position pos.  A key's high word is the ordered value, so a 32-bit
 // read of it decides all but the ties; the stored keys only grow, so a stale
 // read can only cost an atomic that changes nothing.
-__device__ __forceinline__ void raise_keys(unsigned long long *slot, float v, uint32_t pos)
+__device__ __forceinline__ bool raise_keys(unsigned long long *slot, float v, uint32_t pos)
 {
+    bool raised = false;
     const uint32_t o = ord_f32(v);
     const uint32_t *w = reinterpret_cast<const uint32_t *>(slot);   // little-endian: high words at 1, 3
     if (o >= w[1]) {
         const unsigned long long k = ((unsigned long long)o << 32) | (unsigned long long)(0xFFFFFFFFu - pos);
-        if (k > slot[0]) atomicMax(&slot[0], k);
+        if (k > slot[0]) { atomicMax(&slot[0], k); raised = true; }
     }
     if (~o >= w[3]) {
         const unsigned long long k = ((unsigned long long)(~o) << 32) | (unsigned long long)(0xFFFFFFFFu - pos);
-        if (k > slot[1]) atomicMax(&slot[1], k);
+        if (k > slot[1]) { atomicMax(&slot[1], k); raised = true; }
     }
+    return raised;
 }
 
 template <typename T, int KM, int DM>
@@ -232,10 +279,27 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
     using KY = typename KT::K;
     constexpr bool F32 = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
+    uint64_t *core = nullptr;
     if constexpr (F32) {
-        for (int i = lane; i < warp_key_words(K, D, dk.ndir); i += 32) dk.sk[i] = 0ull;
+        core = reinterpret_cast<uint64_t *>(dk.sk) + 2 * K * (D + dk.ndir);
+        for (int i = lane; i < K * D; i += 32) {
+            const size_t o = (size_t)b * K * D + i;
+            dk.sk[2 * i] = *const_cast<const volatile unsigned long long *>(&amax[o]);
+            dk.sk[2 * i + 1] = *const_cast<const volatile unsigned long long *>(&amin[o]);
+        }
+        unsigned long long *sd = dk.sk + (size_t)2 * K * D;
+        for (int i = lane; i < K * dk.ndir; i += 32) {
+            const size_t o = (size_t)b * K * dk.ndir + i;
+            sd[2 * i] = *const_cast<const volatile unsigned long long *>(&dk.dmax[o]);
+            sd[2 * i + 1] = *const_cast<const volatile unsigned long long *>(&dk.dmin[o]);
+        }
+        __syncwarp();
+        for (int k = 0; k < K; ++k) core_of(dk.sk, k, K, D, dk.ndir, core);
         __syncwarp();
     }
+    bool raised = false;
+    float top = -1.f;          // float data: the largest minimum distance and its sample
+    uint32_t top_pos = ~0u;
     // node boxes into registers
     uint64_t bx[KM][DM];
     double blo[KM][DM], bhi[KM][DM];
@@ -292,7 +356,14 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
                 if (!excl) { ++left; k1 = k; }
             }
         }
-        acc_lb = kmax<T>(acc_lb, KT::max_of(bmin, pos));
+        if constexpr (F32) {
+            if (bmin >= top && (bmin > top || pos < top_pos)) {
+                top = bmin;
+                top_pos = pos;
+            }
+        } else {
+            acc_lb = kmax<T>(acc_lb, KT::max_of(bmin, pos));
+        }
         if (left == 0) infeasible = true;
         if (left == 1) {
             if constexpr (!F32) {
@@ -307,10 +378,18 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
                             }
                     }
             } else {
+                bool in = true;
+#pragma unroll
+                for (int a = 0; a < DM; ++a)
+                    if (a < D) {
+                        const float2 c = upk(core[k1 * D + a]);
+                        in = in && x[a] > c.x && x[a] < c.y;
+                    }
+                if (in) continue;
                 unsigned long long *sa = dk.sk + (size_t)k1 * D * 2;
 #pragma unroll
                 for (int a = 0; a < DM; ++a)
-                    if (a < D) raise_keys(sa + 2 * a, x[a], pos);
+                    if (a < D) raised |= raise_keys(sa + 2 * a, x[a], pos);
                 if (dk.ndir > 0) {
                     unsigned long long *s = dk.sk + (size_t)2 * K * D + (size_t)k1 * dk.ndir * 2;
                     int q = 0;
@@ -319,8 +398,8 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
 #pragma unroll
                         for (int c = a + 1; c < DM; ++c)
                             if (c < D && q < dk.ndir) {
-                                raise_keys(s + 2 * q, __fadd_rn(x[a], x[c]), pos);
-                                raise_keys(s + 2 * q + 2, __fsub_rn(x[a], x[c]), pos);
+                                raised |= raise_keys(s + 2 * q, __fadd_rn(x[a], x[c]), pos);
+                                raised |= raise_keys(s + 2 * q + 2, __fsub_rn(x[a], x[c]), pos);
                                 q += 2;
                             }
                 }
@@ -328,6 +407,9 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
         }
     }
     // warp reduction, then one atomic per accumulator and warp
+    if constexpr (F32) {
+        if (top >= 0.f) acc_lb = KT::max_of(top, top_pos);
+    }
     acc_lb = warp_kmax<T>(acc_lb);
     if (lane == 0 && !KT::is_none(acc_lb)) KT::atomic_max(&lbkey[b], acc_lb, &flags[b]);
     if constexpr (!F32) {
@@ -352,6 +434,7 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
     if (__any_sync(0xffffffffu, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
     if constexpr (F32) {
         __syncwarp();
+        if (!__any_sync(0xffffffffu, raised)) return;
         for (int i = lane; i < K * D; i += 32) {
             const size_t o = (size_t)b * K * D + i;
             if (dk.sk[2 * i]) atomicMax(&amax[o], dk.sk[2 * i]);
@@ -481,115 +564,112 @@ struct FinA {
     // lexicographic order, x_a + x_b for even q, x_a - x_b for odd q)
     int ndir;
     const unsigned long long *dmax, *dmin;
+    float *ball;                // float data: [B][K][D + 2], see BallTest
 };
 
+// One warp per (node, cluster): lanes over the attributes, the pair directions
+// and the representatives (one thread per node took 94 us at D = 4, K = 3, 256
+// nodes and 1.3 ms at D = 12, K = 5, 32 nodes).  allhave[b] counts the clusters
+// that have representatives.
 template <typename T>
-__global__ void finalize_a_kernel(int B, int K, int D, const T *__restrict__ lo, const T *__restrict__ hi,
-                                  const typename Key<T>::K *__restrict__ lbkey,
-                                  const typename Key<T>::K *__restrict__ amax,
-                                  const typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags,
-                                  const T *__restrict__ Xf, int64_t ldf, FinA f, T *__restrict__ blo,
-                                  T *__restrict__ bhi, int64_t *__restrict__ reps, int *__restrict__ nreps,
-                                  T *__restrict__ repx, int *__restrict__ allhave, double *__restrict__ lb,
-                                  double *__restrict__ lb_raw, int64_t *__restrict__ lbarg)
+__global__ void __launch_bounds__(128)
+finalize_a_kernel(int B, int K, int D, const T *__restrict__ lo, const T *__restrict__ hi,
+                  const typename Key<T>::K *__restrict__ lbkey, const typename Key<T>::K *__restrict__ amax,
+                  const typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags, const T *__restrict__ Xf,
+                  int64_t ldf, FinA f, T *__restrict__ blo, T *__restrict__ bhi, int64_t *__restrict__ reps,
+                  int *__restrict__ nreps, T *__restrict__ repx, int *__restrict__ allhave, double *__restrict__ lb,
+                  double *__restrict__ lb_raw, int64_t *__restrict__ lbarg)
 {
     using KT = Key<T>;
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    bool inf = (flags[b] & 1u) != 0;
+    constexpr unsigned ALL = 0xffffffffu;
+    __shared__ int64_t cands[4][1 + 2 * kMaxD + 4 * kMaxPairs];   // candidate ids in order, -1: none
+    const int lane = threadIdx.x & 31, wk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (wk >= B * K) return;
+    const int b = wk / K, k = wk % K;
+    int64_t *cand = cands[threadIdx.x >> 5];
+    bool inf = false;
     // lower bound of the input box
-    {
-        const auto k = lbkey[b];
-        const bool none = KT::is_none(k);
-        const double raw = none ? 0.0 : (double)KT::vmax(k);
+    if (k == 0 && lane == 0) {
+        const auto key = lbkey[b];
+        const bool none = KT::is_none(key);
+        const double raw = none ? 0.0 : (double)KT::vmax(key);
         if (lb_raw) lb_raw[b] = raw;
         if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(raw, f.defl), f.slack));
         if (lbarg) {
-            const int64_t p = none ? -1 : (int64_t)KT::pos(k);
+            const int64_t p = none ? -1 : (int64_t)KT::pos(key);
             lbarg[b] = (p < 0 || !f.ids) ? p : (int64_t)f.ids[p];
         }
     }
-    int have = 1;
-    for (int k = 0; k < K; ++k) {
-        const size_t o0 = ((size_t)b * K + k) * D;
-        int64_t seed = f.seeds ? f.seeds[k] : -1;
-        if (seed >= 0) {
-            // seed consistency: box k farther than alpha from seed k
+    auto id_of = [&](int64_t p) { return f.ids ? (int64_t)f.ids[p] : p; };
+    const size_t o0 = (size_t)wk * D;
+    const int64_t seed = f.seeds ? f.seeds[k] : -1;
+    if (seed >= 0) {
+        // seed consistency: box k farther than alpha from seed k (squares by
+        // lane, summed in attribute order)
+        double *sq = reinterpret_cast<double *>(cand);
+        for (int a = lane; a < D; a += 32) {
+            const double x = (double)Xf[(size_t)a * ldf + seed];
+            const double d = __dsub_rn(x, mid3d((double)lo[o0 + a], x, (double)hi[o0 + a]));
+            sq[a] = __dmul_rn(d, d);
+        }
+        __syncwarp();
+        if (lane == 0) {
             double acc = 0.0;
-            for (int a = 0; a < D; ++a) {
-                const double x = (double)Xf[(size_t)a * ldf + seed];
-                const double mu = mid3d((double)lo[o0 + a], x, (double)hi[o0 + a]);
-                const double d = __dsub_rn(x, mu);
-                acc = __dadd_rn(acc, __dmul_rn(d, d));
-            }
+            for (int a = 0; a < D; ++a) acc = __dadd_rn(acc, sq[a]);
             if (__dmul_rd(acc, f.seed_defl) > f.alpha) inf = true;
         }
-        bool nonempty = seed >= 0;
-        int64_t amin_id[kMaxD], amax_id[kMaxD];
-        for (int a = 0; a < D; ++a) {
-            const size_t o = o0 + a;
-            double vmx = 0, vmn = 0;
-            int64_t imx = -1, imn = -1;
-            if (!KT::is_none(amax[o])) {
-                vmx = (double)KT::vmax(amax[o]);
-                const int64_t p = KT::pos(amax[o]);
-                imx = f.ids ? (int64_t)f.ids[p] : p;
-                vmn = (double)KT::vmin(amin[o]);
-                const int64_t q = KT::pos(amin[o]);
-                imn = f.ids ? (int64_t)f.ids[q] : q;
-                nonempty = true;
-            }
-            if (seed >= 0) {
-                const double sx = (double)Xf[(size_t)a * ldf + seed];
-                if (imx < 0 || sx > vmx || (sx == vmx && seed < imx)) { vmx = sx; imx = seed; }
-                if (imn < 0 || sx < vmn || (sx == vmn && seed < imn)) { vmn = sx; imn = seed; }
-            }
-            amin_id[a] = imn;
-            amax_id[a] = imx;
-            T l = lo[o], h = hi[o];
-            if (imx >= 0) {
-                const T l2 = round_dn<T>(nextafter(__dsub_rn(vmx, f.r_up), -__builtin_huge_val()));
-                const T h2 = round_up<T>(nextafter(__dadd_rn(vmn, f.r_up), __builtin_huge_val()));
-                if (l2 > l) l = l2;
-                if (h2 < h) h = h2;
-            }
-            if (l > h) inf = true;
-            blo[o] = l;
-            bhi[o] = h;
+        __syncwarp();
+    }
+    bool some = seed >= 0;
+    for (int a = lane; a < D; a += 32) {
+        const size_t o = o0 + a;
+        double vmx = 0, vmn = 0;
+        int64_t imx = -1, imn = -1;
+        if (!KT::is_none(amax[o])) {
+            vmx = (double)KT::vmax(amax[o]);
+            imx = id_of(KT::pos(amax[o]));
+            vmn = (double)KT::vmin(amin[o]);
+            imn = id_of(KT::pos(amin[o]));
+            some = true;
         }
-        // representatives: seed, then arg-min / arg-max of each attribute
-        int nr = 0;
-        int64_t *rp = reps + ((size_t)b * K + k) * f.RM;
-        auto add = [&](int64_t v) {
-            if (v < 0 || nr >= f.cap) return;
-            for (int q = 0; q < nr; ++q)
-                if (rp[q] == v) return;
-            rp[nr++] = v;
-        };
-        add(seed);
-        if (nonempty)
-            for (int a = 0; a < D; ++a) {
-                add(amin_id[a]);
-                add(amax_id[a]);
-            }
-        if constexpr (sizeof(T) == 4) {
-            // then the arg-min and arg-max along each pair direction, the seed
-            // taking part as an assigned sample of cluster k
-            int pa = 0, pb = 1;
-            for (int q = 0; q < f.ndir && nonempty && nr < f.cap; ++q) {
-                if (q > 0 && !(q & 1)) {
-                    if (++pb == D) { ++pa; pb = pa + 1; }
-                }
-                const size_t o = ((size_t)b * K + k) * f.ndir + q;
+        if (seed >= 0) {
+            const double sx = (double)Xf[(size_t)a * ldf + seed];
+            if (imx < 0 || sx > vmx || (sx == vmx && seed < imx)) { vmx = sx; imx = seed; }
+            if (imn < 0 || sx < vmn || (sx == vmn && seed < imn)) { vmn = sx; imn = seed; }
+        }
+        cand[1 + 2 * a] = imn;
+        cand[2 + 2 * a] = imx;
+        T l = lo[o], h = hi[o];
+        if (imx >= 0) {
+            const T l2 = round_dn<T>(nextafter(__dsub_rn(vmx, f.r_up), -__builtin_huge_val()));
+            const T h2 = round_up<T>(nextafter(__dadd_rn(vmn, f.r_up), __builtin_huge_val()));
+            if (l2 > l) l = l2;
+            if (h2 < h) h = h2;
+        }
+        if (l > h) inf = true;
+        blo[o] = l;
+        bhi[o] = h;
+    }
+    some = __any_sync(ALL, some);
+    if (lane == 0) cand[0] = seed;
+    int total = some ? 1 + 2 * D : 1;
+    if constexpr (sizeof(T) == 4) {
+        // then the arg-min and arg-max along each pair direction, the seed
+        // taking part as an assigned sample of cluster k
+        if (some) {
+            total += 2 * f.ndir;
+            for (int q = lane; q < f.ndir; q += 32) {
+                int pa = 0, r = q >> 1;
+                while (r >= D - 1 - pa) r -= D - 1 - pa++;
+                const int pb = pa + 1 + r;
+                const size_t o = (size_t)wk * f.ndir + q;
                 float vmx = 0.f, vmn = 0.f;
                 int64_t imx = -1, imn = -1;
                 if (!KT::is_none(f.dmax[o])) {
                     vmx = KT::vmax(f.dmax[o]);
-                    const int64_t p = KT::pos(f.dmax[o]);
-                    imx = f.ids ? (int64_t)f.ids[p] : p;
+                    imx = id_of(KT::pos(f.dmax[o]));
                     vmn = KT::vmin(f.dmin[o]);
-                    const int64_t p2 = KT::pos(f.dmin[o]);
-                    imn = f.ids ? (int64_t)f.ids[p2] : p2;
+                    imn = id_of(KT::pos(f.dmin[o]));
                 }
                 if (seed >= 0) {
                     const float xa = Xf[(size_t)pa * ldf + seed], xb = Xf[(size_t)pb * ldf + seed];
@@ -597,19 +677,68 @@ __global__ void finalize_a_kernel(int B, int K, int D, const T *__restrict__ lo,
                     if (imx < 0 || sv > vmx || (sv == vmx && seed < imx)) { vmx = sv; imx = seed; }
                     if (imn < 0 || sv < vmn || (sv == vmn && seed < imn)) { vmn = sv; imn = seed; }
                 }
-                add(imn);
-                add(imx);
+                cand[1 + 2 * D + 2 * q] = imn;
+                cand[2 + 2 * D + 2 * q] = imx;
             }
         }
-        for (int q = nr; q < f.RM; ++q) rp[q] = -1;
-        nreps[(size_t)b * K + k] = nr;
-        T *rx = repx + ((size_t)b * K + k) * f.RM * D;
-        for (int q = 0; q < nr; ++q)
-            for (int a = 0; a < D; ++a) rx[(size_t)q * D + a] = Xf[(size_t)a * ldf + rp[q]];
-        if (nr == 0) have = 0;
     }
-    allhave[b] = have;
-    if (inf) atomicOr(&flags[b], 1u);
+    __syncwarp();
+    // the first f.cap distinct ones (lane l holds representatives l and l + 32)
+    int nr = 0;
+    int64_t r0 = -1, r1 = -1;
+    for (int i = 0; i < total && nr < f.cap; ++i) {
+        const int64_t v = cand[i];
+        if (v < 0 || __any_sync(ALL, r0 == v || r1 == v)) continue;
+        if (lane == (nr & 31)) (nr < 32 ? r0 : r1) = v;
+        ++nr;
+    }
+    __syncwarp();
+    cand[lane] = r0;
+    cand[lane + 32] = r1;
+    __syncwarp();
+    for (int q = lane; q < f.RM; q += 32) reps[(size_t)wk * f.RM + q] = q < nr ? cand[q] : -1;
+    T *rx = repx + (size_t)wk * f.RM * D;
+    for (int i = lane; i < nr * D; i += 32) rx[i] = Xf[(size_t)(i % D) * ldf + cand[i / D]];
+    if (lane == 0) {
+        nreps[wk] = nr;
+        if (nr > 0) atomicAdd(&allhave[b], 1);
+    }
+    if (__any_sync(ALL, inf) && lane == 0) atomicOr(&flags[b], 1u);
+    if constexpr (sizeof(T) == 4) {
+        // a ball around the representatives (see BallTest)
+        __syncwarp();
+        float *ball = f.ball + (size_t)wk * (D + 2);
+        float err = 0.f, rad = 0.f;
+        for (int a = lane; a < D; a += 32) {
+            float sum = 0.f, big = 0.f;
+            for (int r = 0; r < nr; ++r) {
+                sum += rx[(size_t)r * D + a];
+                big = fmaxf(big, fabsf(rx[(size_t)r * D + a]));
+            }
+            ball[a] = nr > 0 ? sum / (float)nr : 0.f;
+            const float e = big * ((float)(nr + 4) * 6.0e-8f);
+            err += e * e;
+        }
+        __syncwarp();
+        for (int r = lane; r < nr; r += 32) {
+            float acc = 0.f;
+            for (int a = 0; a < D; ++a) {
+                const float t = rx[(size_t)r * D + a] - ball[a];
+                acc = fmaf(t, t, acc);
+            }
+            rad = fmaxf(rad, acc);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            err += __shfl_xor_sync(ALL, err, o);
+            rad = fmaxf(rad, __shfl_xor_sync(ALL, rad, o));
+        }
+        if (lane == 0) {
+            const float up = 1.f + (float)(2 * D + 16) * 6.0e-8f;
+            ball[D] = nr > 0 ? __fmul_ru(__fsqrt_ru(rad), up) : -__int_as_float(0x7f800000);
+            ball[D + 1] = nr > 0 ? __fmul_ru(__fsqrt_ru(err), up) : __int_as_float(0x7f800000);
+        }
+    }
 }
 
 // ------------------------------------------------------------ pass B
@@ -633,6 +762,8 @@ struct PBSlot {
     T l[KM][DM], h[KM][DM], mid[KM][DM]; // box-BT boxes and their midpoints
     OrdT<T> smax[KM][DM], smin[KM][DM];  // bbox of S_+ (ordered integers)
     OrdT<T> jmax[KM][DM], jmin[KM][DM];  // bbox of the sample-based assigned samples
+    uint64_t c0[KM][(DM + 1) / 2];       // float data: the representatives' ball (BallTest)
+    BallTest one[KM], four[KM];          // against alpha and 4 alpha
 };
 
 __device__ __forceinline__ unsigned to_ord(float v) { return ord_f32(v); }
@@ -650,8 +781,8 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
                                             const T *__restrict__ lo_in, const T *__restrict__ hi_in,
                                             const T *__restrict__ blo, const T *__restrict__ bhi,
                                             const T *__restrict__ repx, const int *__restrict__ nreps,
-                                            const int *__restrict__ allhave, double alpha, const Margins &mg,
-                                            const int64_t *seed_id, unsigned long long *__restrict__ cnt,
+                                            const int *__restrict__ allhave, const float *__restrict__ ball, double alpha,
+                                            const Margins &mg, const int64_t *seed_id, unsigned long long *__restrict__ cnt,
                                             OrdT<T> *__restrict__ smax, OrdT<T> *__restrict__ smin,
                                             OrdT<T> *__restrict__ jmax, OrdT<T> *__restrict__ jmin,
                                             typename Key<T>::K *__restrict__ cand, unsigned *__restrict__ flags)
@@ -683,7 +814,19 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
     int nr[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k) nr[k] = k < K ? nreps[(size_t)b * K + k] : 0;
-    const bool have = allhave[b] != 0;
+    const bool have = allhave[b] == K;
+    if constexpr (F32) {
+        for (int i = lane; i < KM * DH; i += 32) {
+            const int k = i / DH, p = i % DH;
+            const float *c = ball + ((size_t)b * K + k) * (D + 2);
+            ws->c0[k][p] = pk(k < K && 2 * p < D ? c[2 * p] : 0.f, k < K && 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
+        }
+        if (lane < K) {
+            const float *c = ball + ((size_t)b * K + lane) * (D + 2) + D;
+            ws->one[lane] = ball_test(mg.t_alpha, c[0], c[1], mg.g4);
+            ws->four[lane] = ball_test(mg.t_four, c[0], c[1], mg.g4);
+        }
+    }
     // the node's representatives into the warp's slot wrep [K][RM][words]
     constexpr int RW = rep_words<T, DM>();
     {
@@ -797,7 +940,17 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
                 far4[k] = far1[k] = false;
                 const bool need = k < K && ((fl & 1u) || (fl & (2u << k)));
                 if (!need) continue;
-                const bool want4 = (fl & 1u) != 0u;
+                bool want4 = (fl & 1u) != 0u;
+                if constexpr (F32) {
+                    // the ball decides most samples
+                    const float dc = pt_dist_f32<2 * DH>(px, ws->c0[k]);
+                    const BallTest b1 = ws->one[k], b4 = ws->four[k];
+                    if (dc > b1.far) far1[k] = true;
+                    if (dc > b4.far) far4[k] = true;
+                    want4 = want4 && !far4[k] && !(dc <= b4.near);
+                    const bool want1 = (fl & (2u << k)) && !far1[k] && !(dc <= b1.near);
+                    if (!want1 && !want4) continue;
+                }
                 const uint64_t *rk = wrep + (size_t)k * RM * RW;
                 const int nk = nr[k];
                 for (int r0 = 0; r0 < nk; r0 += 4) {
@@ -892,7 +1045,8 @@ __global__ void __launch_bounds__(kThreads, 3)
 visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, int B, int K, int D, int RM,
                const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
                const T *__restrict__ bhi, const T *__restrict__ repx, const int *__restrict__ nreps,
-               const int *__restrict__ allhave, double alpha, Margins mg, const int64_t *__restrict__ seeds,
+               const int *__restrict__ allhave, const float *__restrict__ ball, double alpha, Margins mg,
+               const int64_t *__restrict__ seeds,
                const uint32_t *__restrict__ ids, unsigned long long *__restrict__ cnt,
                OrdT<T> *__restrict__ smax, OrdT<T> *__restrict__ smin, OrdT<T> *__restrict__ jmax,
                OrdT<T> *__restrict__ jmin, typename Key<T>::K *__restrict__ cand, unsigned *__restrict__ flags)
@@ -919,7 +1073,7 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
         __syncthreads();
         for (int b = (int)(u % split) * NWV + warp; b < B; b += split * NWV)
             pass_b_node<T, KM, DM>(tx, tile, tn, 0, 32, nullptr, ids, base, list, slots + warp, wrep, b, K, D, RM,
-                                        lo_in, hi_in, blo, bhi, repx, nreps, allhave, alpha, mg, seed_id, cnt, smax,
+                                        lo_in, hi_in, blo, bhi, repx, nreps, allhave, ball, alpha, mg, seed_id, cnt, smax,
                                         smin, jmax, jmin, cand, flags);
     }
 }
@@ -930,7 +1084,8 @@ __global__ void __launch_bounds__(kThreads, 3)
 visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, int K,
                     int D, int RM, const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
                     const T *__restrict__ bhi, const T *__restrict__ repx, const int *__restrict__ nreps,
-                    const int *__restrict__ allhave, double alpha, Margins mg, const int64_t *__restrict__ seeds,
+                    const int *__restrict__ allhave, const float *__restrict__ ball, double alpha, Margins mg,
+               const int64_t *__restrict__ seeds,
                     unsigned long long *__restrict__ cnt, OrdT<T> *__restrict__ smax, OrdT<T> *__restrict__ smin,
                     OrdT<T> *__restrict__ jmax, OrdT<T> *__restrict__ jmin, typename Key<T>::K *__restrict__ cand,
                     unsigned *__restrict__ flags)
@@ -967,7 +1122,7 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, 
             for (int nd = n0 + team; nd < n1; nd += teams)
                 pass_b_node<T, KM, DM>(tx, tile, tn, (warp % wpt) * 32, wpt * 32, tids, nullptr, 0, list,
                                        slots + warp, wrep, nd, K, D, RM, lo_in, hi_in, blo, bhi, repx, nreps, allhave,
-                                       alpha, mg, seed_id, cnt, smax, smin, jmax, jmin, cand, flags);
+                                       ball, alpha, mg, seed_id, cnt, smax, smin, jmax, jmin, cand, flags);
         (void)lane;
     }
 }
@@ -1175,6 +1330,7 @@ Margins make_margins(kc_ctx *c, double alpha, double beta_glob)
     m.alpha_up = up(alpha);
     m.four_up = up(4.0 * alpha);
     m.beta_dn = dn(beta_glob);
+    m.g4 = up(4.0 * g);
     m.t_alpha = up(((double)m.alpha_up + (double)m.slack) / (double)m.defl * (1.0 + 1e-6));
     m.t_four = up(((double)m.four_up + (double)m.slack) / (double)m.defl * (1.0 + 1e-6));
     return m;
@@ -1219,6 +1375,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const size_t o_smin = take(KD * sizeof(OrdT<T>)), o_jmax = take(KD * sizeof(OrdT<T>));
     const size_t o_jmin = take(KD * sizeof(OrdT<T>)), o_cand = take(BK * sizeof(KY));
     const size_t o_dmax = take(BK * ndir * 8), o_dmin = take(BK * ndir * 8);
+    const size_t o_ball = take(sizeof(T) == 4 ? BK * (D + 2) * 4 : 0);
     KC_TRY(ensure(c, vs->buf, off));
     char *w = static_cast<char *>(vs->buf.p);
     KY *lbkey = reinterpret_cast<KY *>(w + o_lbkey), *amax = reinterpret_cast<KY *>(w + o_amax);
@@ -1230,6 +1387,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     int64_t *reps = reinterpret_cast<int64_t *>(w + o_reps);
     int *nreps = reinterpret_cast<int *>(w + o_nreps), *have = reinterpret_cast<int *>(w + o_have);
     T *repx = reinterpret_cast<T *>(w + o_repx);
+    float *ball = reinterpret_cast<float *>(w + o_ball);
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(w + o_cnt);
     OrdT<T> *smax = reinterpret_cast<OrdT<T> *>(w + o_smax), *smin = reinterpret_cast<OrdT<T> *>(w + o_smin);
     OrdT<T> *jmax = reinterpret_cast<OrdT<T> *>(w + o_jmax), *jmin = reinterpret_cast<OrdT<T> *>(w + o_jmin);
@@ -1288,7 +1446,8 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     fa.ndir = ndir;
     fa.dmax = dmax;
     fa.dmin = dmin;
-    finalize_a_kernel<T><<<(B + 127) / 128, 128, 0, c->stream>>>(
+    fa.ball = ball;
+    finalize_a_kernel<T><<<(B * K_ + 3) / 4, 128, 0, c->stream>>>(
         B, K_, D, lo, hi, lbkey, amax, amin, flags, static_cast<const T *>(c->X), c->ldx, fa, blo, bhi, reps, nreps,
         repx, have, lb, lb_raw, lbarg);
     KC_TRY(after_launch(c, "tighten finalize A"));
@@ -1312,7 +1471,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
             KC_TRY(grid_of(c, kBL, smem, std::max<int64_t>(1, L->W), &g));
             if (L->W > 0) {
                 kBL<<<g, kThreads, smem, c->stream>>>(static_cast<const T *>(c->X), c->ldx, *L, lt, K_, D, RM, lo, hi,
-                                                      blo, bhi, repx, nreps, have, alpha, mg, seeds, cnt, smax, smin,
+                                                      blo, bhi, repx, nreps, have, ball, alpha, mg, seeds, cnt, smax, smin,
                                                       jmax, jmin, cand, flags);
                 KC_TRY(after_launch(c, "tighten pass B (lists)"));
             }
@@ -1321,7 +1480,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     KC_TRY(grid_of(c, kB, smemB, (v.n + tileB - 1) / tileB * splitB, &gB));
     if (v.n > 0) {
         kB<<<gB, kThreads, smemB, c->stream>>>(static_cast<const T *>(v.X), v.ld, v.n, tileB, splitB, B, K_, D, RM, lo, hi, blo,
-                                              bhi, repx, nreps, have, alpha, mg, seeds, v.ids, cnt, smax, smin, jmax, jmin,
+                                              bhi, repx, nreps, have, ball, alpha, mg, seeds, v.ids, cnt, smax, smin, jmax, jmin,
                                               cand, flags);
         KC_TRY(after_launch(c, "tighten pass B"));
     }
@@ -1333,6 +1492,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     vs->reps = reps;
     vs->nreps = nreps;
     vs->repx = repx;
+    vs->ball = sizeof(T) == 4 ? ball : nullptr;
     vs->RM = RM;
     return KC_OK;
 }
@@ -1368,6 +1528,7 @@ kc_status tighten_wide(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const size_t o_smin = take(KD * 4), o_jmax = take(KD * 4);
     const size_t o_jmin = take(KD * 4), o_cand = take(BK * sizeof(KY));
     const size_t o_dmax = take(BK * ndir * sizeof(KY)), o_dmin = take(BK * ndir * sizeof(KY));
+    const size_t o_ball = take(BK * (D + 2) * 4);
     KC_TRY(ensure(c, vs->buf, off));
     char *w = static_cast<char *>(vs->buf.p);
     KY *lbkey = reinterpret_cast<KY *>(w + o_lbkey), *amax = reinterpret_cast<KY *>(w + o_amax);
@@ -1378,6 +1539,7 @@ kc_status tighten_wide(kc_ctx *c, const View &v, const void *lo_, const void *hi
     int64_t *reps = reinterpret_cast<int64_t *>(w + o_reps);
     int *nreps = reinterpret_cast<int *>(w + o_nreps), *have = reinterpret_cast<int *>(w + o_have);
     T *repx = reinterpret_cast<T *>(w + o_repx);
+    float *ball = reinterpret_cast<float *>(w + o_ball);
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(w + o_cnt);
     unsigned *smax = reinterpret_cast<unsigned *>(w + o_smax), *smin = reinterpret_cast<unsigned *>(w + o_smin);
     unsigned *jmax = reinterpret_cast<unsigned *>(w + o_jmax), *jmin = reinterpret_cast<unsigned *>(w + o_jmin);
@@ -1403,7 +1565,8 @@ kc_status tighten_wide(kc_ctx *c, const View &v, const void *lo_, const void *hi
     fa.ndir = ndir;
     fa.dmax = dmax;
     fa.dmin = dmin;
-    finalize_a_kernel<T><<<(B + 127) / 128, 128, 0, c->stream>>>(
+    fa.ball = ball;
+    finalize_a_kernel<T><<<(B * K_ + 3) / 4, 128, 0, c->stream>>>(
         B, K_, D, lo, hi, lbkey, amax, amin, flags, static_cast<const T *>(c->X), c->ldx, fa, blo, bhi, reps, nreps,
         repx, have, lb, lb_raw, lbarg);
     KC_TRY(after_launch(c, "tighten finalize A"));
@@ -1411,7 +1574,7 @@ kc_status tighten_wide(kc_ctx *c, const View &v, const void *lo_, const void *hi
         KC_TRY(launch_wide_ball_all(c, v, lo, hi, B, mg, blo, bhi, have, seeds, cnt, cand, smax, smin, jmax, jmin, flags,
                                     vs));
     else
-        KC_TRY(launch_wide_b(c, v, L, lo, hi, B, mg, blo, bhi, repx, nreps, have, seeds, RM, cnt, cand, smax, smin,
+        KC_TRY(launch_wide_b(c, v, L, lo, hi, B, mg, blo, bhi, repx, nreps, have, ball, seeds, RM, cnt, cand, smax, smin,
                              jmax, jmin, flags));
     finalize_b_kernel<T><<<(B + 127) / 128, 128, 0, c->stream>>>(B, K_, D, cnt, smax, smin, jmax, jmin, cand, flags,
                                                                 L ? nullptr : v.ids, r_up, static_cast<T *>(lo_out_),
@@ -1420,6 +1583,7 @@ kc_status tighten_wide(kc_ctx *c, const View &v, const void *lo_, const void *hi
     vs->reps = reps;
     vs->nreps = nreps;
     vs->repx = repx;
+    vs->ball = sizeof(T) == 4 ? ball : nullptr;
     vs->RM = RM;
     return KC_OK;
 }

@@ -191,7 +191,7 @@ __device__ __forceinline__ void wide_a_node(const uint64_t *tp, int tile, int tn
 }
 
 __global__ void __launch_bounds__(kWT, 2)
-wide_a_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, ListBatch L, int B, int K, int D,
+wide_a_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, int split, ListBatch L, int B, int K, int D,
               const float *__restrict__ lo, const float *__restrict__ hi, Margins mg,
               unsigned long long *__restrict__ lbkey, unsigned long long *__restrict__ amax,
               unsigned long long *__restrict__ amin, unsigned *__restrict__ flags, int ndir,
@@ -233,11 +233,13 @@ wide_a_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, List
                             amin, flags, dv);
         }
     } else {
-        for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
+        const int64_t units = (n + tile - 1) / tile * split;
+        for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+            const int64_t base = u / split * tile;
             const int tn = (int)((n - base) < (int64_t)tile ? (n - base) : (int64_t)tile);
             __syncthreads();
             wide_stage(X, ld, D, tile, tn, base, nullptr, tp);
-            for (int b = 0; b < B; ++b)
+            for (int b = (int)(u % split); b < B; b += split)
                 wide_a_node(tp, tile, tn, nullptr, base, lo, hi, b, K, D, mg, sbx, samax, samin, slb, sflag, lbkey,
                             amax, amin, flags, dv);
         }
@@ -253,9 +255,15 @@ wide_a_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, List
 // | box-BT lo, hi, mid [K][D] f32 | smax, smin, jmax, jmin [K][D] u32 |
 // counts [K] u64 | cand [K] u64 | nr [K] int | flag.
 
+__host__ __device__ inline size_t wide_b_node_bytes(int K, int D)
+{
+    return ((size_t)K * D * (8 + 12 + 16 + 4) + 16 + (size_t)K * (20 + 16) + 16 + 15) & ~(size_t)15;
+}
+
 struct WideB {
     const float *blo, *bhi, *repx;
     const int *nreps, *allhave;
+    const float *ball;   // [B][K][D + 2], see BallTest
     const int64_t *seeds;
     int RM;
     unsigned long long *cnt, *cand;
@@ -276,9 +284,18 @@ __device__ __forceinline__ void wide_b_node(const uint64_t *tp, int tile, int tn
     unsigned long long *scand = scnt + K;
     int *snr = reinterpret_cast<int *>(scand + K);
     unsigned *sflag = reinterpret_cast<unsigned *>(snr + K);
+    BallTest *one = reinterpret_cast<BallTest *>((reinterpret_cast<uintptr_t>(sflag + 1) + 7) & ~(uintptr_t)7);
+    BallTest *four = one + K;
+    float *sc0 = reinterpret_cast<float *>(four + K);
     __syncthreads();
+    for (int k = threadIdx.x; k < K; k += kWT) {
+        const float *c = p.ball + ((size_t)b * K + k) * (D + 2) + D;
+        one[k] = ball_test(mg.t_alpha, c[0], c[1], mg.g4);
+        four[k] = ball_test(mg.t_four, c[0], c[1], mg.g4);
+    }
     for (int i = threadIdx.x; i < KD; i += kWT) {
         const size_t o = (size_t)b * KD + i;
+        sc0[i] = p.ball[((size_t)b * K + i / D) * (D + 2) + i % D];
         sbx[i] = pk(lo[o], -hi[o]);
         const float lv = p.blo[o], hv = p.bhi[o];
         sl[i] = lv;
@@ -296,7 +313,7 @@ __device__ __forceinline__ void wide_b_node(const uint64_t *tp, int tile, int tn
     }
     if (threadIdx.x == 0) *sflag = 0u;
     __syncthreads();
-    const bool have = p.allhave[b] != 0;
+    const bool have = p.allhave[b] == K;
     const float *rxb = p.repx + (size_t)b * K * p.RM * D;
     bool infeasible = false;
     for (int j = threadIdx.x; j < tn; j += kWT) {
@@ -323,12 +340,20 @@ __device__ __forceinline__ void wide_b_node(const uint64_t *tp, int tile, int tn
             }
             if (!open && !inb) continue;
             // distances to the representatives of cluster k
-            bool far4 = false, far1 = false;
-            for (int r = 0; r < snr[k]; ++r) {
-                const float d = wide_pt_dist(tp, tile, j, rxb + ((size_t)k * p.RM + r) * D, D);
-                if (d > mg.t_four) far4 = true;
-                if (d > mg.t_alpha) far1 = true;
-            }
+            // (the ball decides most samples; far4 implies far1)
+            const float dc = wide_pt_dist(tp, tile, j, sc0 + (size_t)k * D, D);
+            bool far1 = dc > one[k].far, far4 = dc > four[k].far;
+            const bool want4 = open && !far4 && !(dc <= four[k].near);
+            const bool want1 = inb && !far1 && !(dc <= one[k].near);
+            if (want4 || want1)
+                for (int r = 0; r < snr[k]; ++r) {
+                    const float d = wide_pt_dist(tp, tile, j, rxb + ((size_t)k * p.RM + r) * D, D);
+                    if (d > mg.t_alpha) {
+                        far1 = true;
+                        if (d > mg.t_four) { far4 = true; break; }
+                        if (!want4) break;
+                    }
+                }
             if (open && !far4) { ++left4; k4 = k; }
             if (inb && !far1) {
                 // ball-based tightening and centers on samples
@@ -371,14 +396,14 @@ __device__ __forceinline__ void wide_b_node(const uint64_t *tp, int tile, int tn
 }
 
 __global__ void __launch_bounds__(kWT, 2)
-wide_b_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, ListBatch L, int B, int K, int D,
+wide_b_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, int split, ListBatch L, int B, int K, int D,
               const float *__restrict__ lo, const float *__restrict__ hi, Margins mg, const uint32_t *__restrict__ ids,
               WideB p)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *tp = reinterpret_cast<uint64_t *>(smem);
     unsigned char *ns = reinterpret_cast<unsigned char *>(tp + (size_t)D * tile);
-    const size_t node_bytes = ((size_t)K * D * (8 + 12 + 16) + 16 + (size_t)K * 20 + 8 + 15) & ~(size_t)15;
+    const size_t node_bytes = wide_b_node_bytes(K, D);
     uint32_t *tids = reinterpret_cast<uint32_t *>(ns + node_bytes);
     if (L.pool) {
         for (int64_t w = blockIdx.x; w < L.W; w += gridDim.x) {
@@ -395,11 +420,14 @@ wide_b_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int tile, List
             for (int b = n0; b < n1; ++b) wide_b_node(tp, tile, tn, tids, nullptr, 0, lo, hi, b, K, D, mg, ns, p);
         }
     } else {
-        for (int64_t base = (int64_t)blockIdx.x * tile; base < n; base += (int64_t)gridDim.x * tile) {
+        const int64_t units = (n + tile - 1) / tile * split;
+        for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+            const int64_t base = u / split * tile;
             const int tn = (int)((n - base) < (int64_t)tile ? (n - base) : (int64_t)tile);
             __syncthreads();
             wide_stage(X, ld, D, tile, tn, base, nullptr, tp);
-            for (int b = 0; b < B; ++b) wide_b_node(tp, tile, tn, nullptr, ids, base, lo, hi, b, K, D, mg, ns, p);
+            for (int b = (int)(u % split); b < B; b += split)
+                wide_b_node(tp, tile, tn, nullptr, ids, base, lo, hi, b, K, D, mg, ns, p);
         }
     }
 }
@@ -534,7 +562,7 @@ ball_all_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int K, int D
     if (threadIdx.x == 0) *sflag = 0u;
     __syncthreads();
     const int j = threadIdx.x;
-    const bool valid = j < tn, have = p.allhave[b] != 0;
+    const bool valid = j < tn, have = p.allhave[b] == K;
     const uint32_t pos = (uint32_t)(base + j);
     // clusters the center-based rule leaves open; an open sample that is not
     // a seed gets the sample-based rule
@@ -637,9 +665,10 @@ ball_all_kernel(const float *__restrict__ X, int64_t ld, int64_t n, int K, int D
 
 }  // namespace
 
-size_t wide_b_node_bytes(int K, int D)
+// Shares of the nodes per tile: about eight work units per SM and more.
+static int wide_split(const kc_ctx *c, int64_t tiles, int B)
 {
-    return ((size_t)K * D * (8 + 12 + 16) + 16 + (size_t)K * 20 + 8 + 15) & ~(size_t)15;
+    return (int)std::max<int64_t>(1, std::min<int64_t>(B, (16 * c->num_sms + tiles - 1) / std::max<int64_t>(1, tiles)));
 }
 
 // Pass A and pass B of the wide path on the context's stream; the caller
@@ -662,17 +691,19 @@ kc_status launch_wide_a(kc_ctx *c, const View &v, const ListBatch *L, const floa
     KC_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide_a_kernel, kWT, smem));
     if (per_sm < 1) return set_err(c, KC_EINTERNAL, "wide tightening pass A does not fit (smem %zu)", smem);
     ListBatch Lz;
-    const int64_t work = L ? L->W : (v.n + tile - 1) / tile;
+    const int64_t tiles = (v.n + tile - 1) / tile;
+    const int split = wide_split(c, tiles, B);
+    const int64_t work = L ? L->W : tiles * split;
     if (work <= 0) return KC_OK;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(work, (int64_t)per_sm * c->num_sms));
-    wide_a_kernel<<<grid, kWT, smem, c->stream>>>(static_cast<const float *>(v.X), v.ld, v.n, tile, L ? *L : Lz, B,
+    wide_a_kernel<<<grid, kWT, smem, c->stream>>>(static_cast<const float *>(v.X), v.ld, v.n, tile, split, L ? *L : Lz, B,
                                                   K, D, lo, hi, mg, lbkey, amax, amin, flags, ndir, dmax, dmin);
     return after_launch(c, "tighten pass A (wide)");
 }
 
 kc_status launch_wide_b(kc_ctx *c, const View &v, const ListBatch *L, const float *lo, const float *hi, int B,
                         const Margins &mg, const float *blo, const float *bhi, const float *repx, const int *nreps,
-                        const int *allhave, const int64_t *seeds, int RM, unsigned long long *cnt,
+                        const int *allhave, const float *ball, const int64_t *seeds, int RM, unsigned long long *cnt,
                         unsigned long long *cand, unsigned *smax, unsigned *smin, unsigned *jmax, unsigned *jmin,
                         unsigned *flags)
 {
@@ -687,11 +718,13 @@ kc_status launch_wide_b(kc_ctx *c, const View &v, const ListBatch *L, const floa
     KC_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, wide_b_kernel, kWT, smem));
     if (per_sm < 1) return set_err(c, KC_EINTERNAL, "wide tightening pass B does not fit (smem %zu)", smem);
     ListBatch Lz;
-    const int64_t work = L ? L->W : (v.n + tile - 1) / tile;
+    const int64_t tiles = (v.n + tile - 1) / tile;
+    const int split = wide_split(c, tiles, B);
+    const int64_t work = L ? L->W : tiles * split;
     if (work <= 0) return KC_OK;
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(work, (int64_t)per_sm * c->num_sms));
-    WideB p{blo, bhi, repx, nreps, allhave, seeds, RM, cnt, cand, smax, smin, jmax, jmin, flags};
-    wide_b_kernel<<<grid, kWT, smem, c->stream>>>(static_cast<const float *>(v.X), v.ld, v.n, tile, L ? *L : Lz, B, K,
+    WideB p{blo, bhi, repx, nreps, allhave, ball, seeds, RM, cnt, cand, smax, smin, jmax, jmin, flags};
+    wide_b_kernel<<<grid, kWT, smem, c->stream>>>(static_cast<const float *>(v.X), v.ld, v.n, tile, split, L ? *L : Lz, B, K,
                                                   D, lo, hi, mg, L ? nullptr : v.ids, p);
     return after_launch(c, "tighten pass B (wide)");
 }
@@ -744,7 +777,7 @@ kc_status launch_wide_ball_all(kc_ctx *c, const View &v, const float *lo, const 
         return set_err(c, KC_EINVAL, "every-sample tightening: grid too large");
     if (D > kAllMaxD) return set_err(c, KC_EINVAL, "every-sample tightening: D <= %d", kAllMaxD);
     const dim3 grid((unsigned)((v.n + kWT - 1) / kWT), (unsigned)B);
-    WideB p{blo, bhi, nullptr, nullptr, allhave, seeds, 0, cnt, cand, smax, smin, jmax, jmin, flags};
+    WideB p{blo, bhi, nullptr, nullptr, allhave, nullptr, seeds, 0, cnt, cand, smax, smin, jmax, jmin, flags};
     auto kern = D <= 2 ? ball_all_kernel<2> : D <= 4 ? ball_all_kernel<4> : D <= 8 ? ball_all_kernel<8>
                                                                               : ball_all_kernel<16>;
     if (smemB > 48 * 1024)
