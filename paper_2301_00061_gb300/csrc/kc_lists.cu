@@ -43,6 +43,21 @@ __device__ __forceinline__ float box_dist_rt(const uint64_t *px, const uint64_t 
     return s.x + s.y;
 }
 
+// Squared distance of two points as H coordinate pairs: even attributes in .x,
+// odd in .y, each a fused chain in attribute order (zero padding adds 0).
+template <int H>
+__device__ __forceinline__ float pair_dist(const uint64_t (&x)[H], const uint64_t *c)
+{
+    uint64_t acc = 0;
+#pragma unroll
+    for (int p = 0; p < H; ++p) {
+        const uint64_t t = sub2(x[p], c[p]);
+        acc = fma2(t, t, acc);
+    }
+    const float2 s = upk(acc);
+    return s.x + s.y;
+}
+
 __device__ __forceinline__ unsigned long long block_max_u64(unsigned long long v, unsigned long long *red)
 {
     v = warp_max_u64(v);
@@ -291,14 +306,15 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
 {
     // out_pool NULL: count the surviving samples only
     __shared__ uint64_t sbox[kMaxK * DMAX];
-    __shared__ float sl[kMaxK * DMAX], sh[kMaxK * DMAX];
+    __shared__ uint64_t skid[2 * DMAX];            // box ks of the two children
     __shared__ unsigned long long red[8];
     __shared__ int snr[kMaxK];
     __shared__ BallTest sball[kMaxK];              // the representatives' balls against alpha
     __shared__ uint64_t sc0[kMaxK * DMAX / 2];
-    // the node's representatives as packed coordinate pairs [K][RM][Dp / 2]
+    // the node's representatives as packed coordinate pairs [K][RM][DMAX / 2]
     extern __shared__ uint64_t srep[];
-    const int Dp = (D + 1) & ~1, H = Dp / 2;
+    constexpr int H = DMAX / 2;
+    const int Dp = (D + 1) & ~1;
     const int lane = threadIdx.x & 31;
     for (int64_t w = blockIdx.x; w < L.W; w += gridDim.x) {
         int b;
@@ -308,11 +324,17 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
         const int tn = (int)((nb - st) < (int64_t)kLT ? (nb - st) : (int64_t)kLT);
         const uint32_t *ids = L.pool + L.seg_off[b] + st;
         __syncthreads();   // the previous item's readers of the boxes are done
-        for (int i = threadIdx.x; i < K * Dp; i += blockDim.x) {
-            const int k = i / Dp, a = i % Dp;
+        // the children's split: box ks, attribute as_, at (cm | cs)
+        const int cv = ckeys ? cvar[b] : 0, ks = cv / D, as_ = cv % D;
+        const float cm = ckeys ? csplit[2 * b] : 0.f, cs = ckeys ? csplit[2 * b + 1] : 0.f;
+        for (int i = threadIdx.x; i < K * DMAX; i += blockDim.x) {
+            const int k = i / DMAX, a = i % DMAX;
             const size_t o = ((size_t)b * K + k) * D + a;
             sbox[i] = a < D ? pk(lo[o], -hi[o]) : pk(0.f, -0.f);
-            if (a < D) { sl[k * D + a] = lo[o]; sh[k * D + a] = hi[o]; }
+            if (k == ks) {
+                skid[a] = a == as_ ? pk(lo[o], -cm) : sbox[i];
+                skid[DMAX + a] = a == as_ ? pk(cs, -hi[o]) : sbox[i];
+            }
         }
         const size_t rb = rmap ? (size_t)rmap[b] : (size_t)b;   // row of the node's representatives
         for (int k = threadIdx.x; k < K; k += blockDim.x) snr[k] = nreps ? nreps[rb * K + k] : 0;
@@ -324,32 +346,31 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
             for (int i = threadIdx.x; i < K * H; i += blockDim.x) {
                 const int k = i / H, p = i % H;
                 const float *c = ball + (rb * K + k) * (D + 2);
-                sc0[i] = pk(c[2 * p], 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
+                sc0[i] = pk(2 * p < D ? c[2 * p] : 0.f, 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
             }
             for (int i = threadIdx.x; i < K * RM * H; i += blockDim.x) {
                 const int k = i / (RM * H), r = (i / H) % RM, p = i % H;
                 const float *c = repx + ((rb * K + k) * RM + r) * D;
-                if (r < nreps[rb * K + k]) srep[i] = pk(c[2 * p], 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
+                if (r < nreps[rb * K + k])
+                    srep[i] = pk(2 * p < D ? c[2 * p] : 0.f, 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
             }
         }
         __syncthreads();
         const float bth = beta_dn[b];
-        // the children's split: box ks, attribute as_, at (cm | cs)
-        const int cv = ckeys ? cvar[b] : 0, ks = cv / D, as_ = cv % D;
-        const float cm = ckeys ? csplit[2 * b] : 0.f, cs = ckeys ? csplit[2 * b + 1] : 0.f;
         unsigned long long best0 = 0ull, best1 = 0ull;
+        float top0 = -1.f, top1 = -1.f;
+        uint32_t pos0 = ~0u, pos1 = ~0u;
         for (int j0 = 0; j0 < tn; j0 += blockDim.x) {
             const int j = j0 + threadIdx.x;
             bool keep = false;
             uint32_t id = 0;
             if (j < tn) {
                 id = ids[j];
-                float x[DMAX];
                 uint64_t px[DMAX];
 #pragma unroll
                 for (int a = 0; a < DMAX; ++a) {
-                    x[a] = a < D ? X[(size_t)a * ld + id] : 0.f;
-                    px[a] = pk(x[a], -x[a]);
+                    const float v = a < D ? X[(size_t)a * ld + id] : 0.f;
+                    px[a] = pk(v, -v);
                 }
                 // lower-bound redundancy: alpha_s(M) < beta (Eq. 13), proved in float
                 float as = __int_as_float(0x7f800000);
@@ -357,85 +378,63 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                     uint64_t acc = 0;
 #pragma unroll
                     for (int a = 0; a < DMAX; a += 2)
-                        if (a < Dp) {
-                            const float2 t0 = upk(sub2(sbox[k * Dp + a], px[a]));
-                            const float2 t1 = upk(sub2(sbox[k * Dp + a + 1], px[a + 1]));
+                        if (DMAX <= 4 || a < Dp) {
+                            const float2 t0 = upk(sub2(sbox[k * DMAX + a], px[a]));
+                            const float2 t1 = upk(sub2(sbox[k * DMAX + a + 1], px[a + 1]));
                             const uint64_t m = pk(fmaxf(fabsf(t0.x), fabsf(t0.y)), fmaxf(fabsf(t1.x), fabsf(t1.y)));
                             acc = fma2(m, m, acc);
                         }
                     const float2 s2 = upk(acc);
                     as = fminf(as, s2.x + s2.y);
                 }
-                const bool lbred = __fadd_ru(__fmul_ru(as, infl), slack) < bth;
+                bool redundant = __fadd_ru(__fmul_ru(as, infl), slack) < bth;
                 // the upper-bound test only matters for lower-bound redundant samples
-                bool ubred = lbred;
-                uint64_t pxx[DMAX / 2];
+                if (redundant) {
+                    uint64_t pxx[DMAX / 2];
 #pragma unroll
-                for (int p = 0; p < DMAX / 2; ++p) pxx[p] = pk(x[2 * p], x[2 * p + 1]);
-                for (int k = 0; k < K && ubred; ++k) {
-                    bool inb = true;
-                    for (int a = 0; a < D; ++a)
-                        if (x[a] < sl[k * D + a] || x[a] > sh[k * D + a]) inb = false;
-                    if (!inb) continue;
-                    bool excl = false;
-                    int nr = snr[k];
-                    const uint64_t *ck = srep + (size_t)k * RM * H;
-                    if (nr > 0) {
-                        // the ball decides most samples
-                        uint64_t acc = 0;
+                    for (int p = 0; p < DMAX / 2; ++p) pxx[p] = pk(upk(px[2 * p]).x, upk(px[2 * p + 1]).x);
+                    for (int k = 0; k < K && redundant; ++k) {
+                        // outside the box: some lo - x or x - hi is positive
+                        float out = 0.f;
 #pragma unroll
-                        for (int p = 0; p < DMAX / 2; ++p)
-                            if (p < H) {
-                                const uint64_t t = sub2(pxx[p], sc0[k * H + p]);
-                                acc = fma2(t, t, acc);
-                            }
-                        const float2 s2 = upk(acc);
-                        const float dc = s2.x + s2.y;
-                        if (dc > sball[k].far) excl = true;
-                        if (dc <= sball[k].near) nr = 0;
-                    }
-                    // chunks of 4 representatives decided by their largest distance
-                    // (a short last chunk repeats the last representative)
-                    for (int r0 = 0; r0 < nr && !excl; r0 += 4) {
-                        float d[4];
-#pragma unroll
-                        for (int u = 0; u < 4; ++u) {
-                            const uint64_t *cr = ck + (size_t)(r0 + u < nr ? r0 + u : nr - 1) * H;
-                            // squared distance: even attributes in .x, odd in .y, each
-                            // a fused chain in attribute order (zero padding adds 0)
-                            uint64_t acc = 0;
-#pragma unroll
-                            for (int p = 0; p < DMAX / 2; ++p)
-                                if (p < H) {
-                                    const uint64_t t = sub2(pxx[p], cr[p]);
-                                    acc = fma2(t, t, acc);
-                                }
-                            const float2 s2 = upk(acc);
-                            d[u] = s2.x + s2.y;
+                        for (int a = 0; a < DMAX; ++a) {
+                            const float2 t = upk(sub2(sbox[k * DMAX + a], px[a]));
+                            out = max3f(out, t.x, t.y);
                         }
-                        if (fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])) > t_alpha) excl = true;
+                        if (out > 0.f) continue;
+                        int nr = snr[k];
+                        bool excl = false;
+                        const uint64_t *ck = srep + (size_t)k * RM * (DMAX / 2);
+                        if (nr > 0) {
+                            // the ball decides most samples
+                            const float dc = pair_dist<DMAX / 2>(pxx, sc0 + k * (DMAX / 2));
+                            excl = dc > sball[k].far;
+                            if (dc <= sball[k].near) nr = 0;
+                        }
+                        // chunks of 4 representatives decided by their largest distance
+                        // (a short last chunk repeats the last representative)
+                        for (int r0 = 0; r0 < nr && !excl; r0 += 4) {
+                            float d[4];
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                d[u] = pair_dist<DMAX / 2>(pxx, ck + (size_t)(r0 + u < nr ? r0 + u : nr - 1) * (DMAX / 2));
+                            if (fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])) > t_alpha) excl = true;
+                        }
+                        if (!excl) redundant = false;
                     }
-                    if (!excl) ubred = false;
                 }
-                keep = !(lbred && ubred);
+                keep = !redundant;
                 if (keep && ckeys) {
                     // children's bounds over the surviving samples (the closed form
-                    // of Section 3.1 in the same float evaluation as seg_lb_f32)
+                    // of Section 3.1 in the same float evaluation as seg_lb_f32);
+                    // their boxes differ from the node's in cluster ks alone
                     float other = __int_as_float(0x7f800000);
                     for (int k = 0; k < K; ++k)
-                        if (k != ks) other = fminf(other, box_dist_rt<DMAX>(px, sbox + k * Dp, Dp));
-                    uint64_t cb[DMAX];
-#pragma unroll
-                    for (int a = 0; a < DMAX; ++a)
-                        cb[a] = a == as_ ? pk(sl[ks * D + as_], -cm) : (a < Dp ? sbox[ks * Dp + a] : pk(0.f, -0.f));
-                    const float d0 = box_dist_rt<DMAX>(px, cb, Dp);
-#pragma unroll
-                    for (int a = 0; a < DMAX; ++a)
-                        if (a == as_) cb[a] = pk(cs, -sh[ks * D + as_]);
-                    const float d1 = box_dist_rt<DMAX>(px, cb, Dp);
-                    const unsigned long long k0 = key_max(fminf(other, d0), id), k1 = key_max(fminf(other, d1), id);
-                    best0 = k0 > best0 ? k0 : best0;
-                    best1 = k1 > best1 ? k1 : best1;
+                        if (k != ks) other = fminf(other, box_dist_f32<DMAX>(px, sbox + k * DMAX));
+                    const float v0 = fminf(other, box_dist_f32<DMAX>(px, skid));
+                    const float v1 = fminf(other, box_dist_f32<DMAX>(px, skid + DMAX));
+                    if (v0 >= top0 && (v0 > top0 || id < pos0)) { top0 = v0; pos0 = id; }
+                    if (v1 >= top1 && (v1 > top1 || id < pos1)) { top1 = v1; pos1 = id; }
                 }
             }
             // one reservation per warp (no block barrier): lane 0 claims the
@@ -451,6 +450,8 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
             }
         }
         if (ckeys) {
+            if (top0 >= 0.f) best0 = key_max(top0, pos0);
+            if (top1 >= 0.f) best1 = key_max(top1, pos1);
             best0 = block_max_u64(best0, red);
             best1 = block_max_u64(best1, red);
             if (threadIdx.x == 0) {
@@ -522,7 +523,7 @@ kc_status launch_seg_lb(kc_ctx *c, const ListBatch &L, const void *lo, const voi
     KC_CUDA(c, cudaMemsetAsync(keys, 0, (size_t)B * 8, c->stream));
     if (L.W > 0) {
         const int g = grid_items(c, L.W);
-        seg_lb_f32<8><<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
+        (c->D <= 2 ? seg_lb_f32<2> : c->D <= 4 ? seg_lb_f32<4> : seg_lb_f32<8>)<<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                 static_cast<const float *>(lo), static_cast<const float *>(hi), c->K,
                                                 c->D, keys);
         KC_TRY(after_launch(c, "list lower bound"));
@@ -553,7 +554,7 @@ kc_status launch_seg_refine(kc_ctx *c, const ListBatch &L, const void *lo, const
     KC_CUDA(c, cudaMemsetAsync(vmax, 0, (size_t)B * 8, c->stream));
     if (L.W > 0) {
         const int g = grid_items(c, L.W);
-        seg_refine_f32<8><<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
+        (c->D <= 2 ? seg_refine_f32<2> : c->D <= 4 ? seg_refine_f32<4> : seg_refine_f32<8>)<<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                     static_cast<const float *>(lo), static_cast<const float *>(hi),
                                                     c->K, c->D, thr_dev, vmax, nullptr, nullptr);
         KC_TRY(after_launch(c, "list refinement"));
@@ -566,7 +567,7 @@ kc_status launch_seg_refine(kc_ctx *c, const ListBatch &L, const void *lo, const
         KC_CUDA(c, cudaMemsetAsync(wid, 0xFF, (size_t)B * 4, c->stream));
         if (L.W > 0) {
             const int g = grid_items(c, L.W);
-            seg_refine_f32<8><<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
+            (c->D <= 2 ? seg_refine_f32<2> : c->D <= 4 ? seg_refine_f32<4> : seg_refine_f32<8>)<<<g, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                         static_cast<const float *>(lo), static_cast<const float *>(hi),
                                                         c->K, c->D, thr_dev, nullptr, vmax, wid);
             KC_TRY(after_launch(c, "list refinement witness"));
@@ -590,14 +591,14 @@ kc_status launch_seg_objective(kc_ctx *c, const ListBatch &L, const int64_t *cen
     const float *X = static_cast<const float *>(c->X);
     const int g = grid_items(c, L.W);
     if (L.W > 0) {
-        seg_obj_screen<8><<<g, 256, 0, c->stream>>>(X, c->ldx, L, X, c->ldx, centers, c->K, c->D, keys);
+        (c->D <= 2 ? seg_obj_screen<2> : c->D <= 4 ? seg_obj_screen<4> : seg_obj_screen<8>)<<<g, 256, 0, c->stream>>>(X, c->ldx, L, X, c->ldx, centers, c->K, c->D, keys);
         KC_TRY(after_launch(c, "list objective screen"));
     }
     const double gam = gamma_n(f32_roundings(c->D), kU32) + 2 * gamma_n(f64_roundings(c->D), kU64) + 1e-15;
     screen_threshold<<<(B + 127) / 128, 128, 0, c->stream>>>(keys, B, gam, alpha_cut, thr);
     KC_TRY(after_launch(c, "list objective threshold"));
     if (L.W > 0) {
-        seg_obj_exact<8><<<g, 256, 0, c->stream>>>(X, c->ldx, L, X, c->ldx, centers, c->K, c->D, thr, vmax);
+        (c->D <= 2 ? seg_obj_exact<2> : c->D <= 4 ? seg_obj_exact<4> : seg_obj_exact<8>)<<<g, 256, 0, c->stream>>>(X, c->ldx, L, X, c->ldx, centers, c->K, c->D, thr, vmax);
         KC_TRY(after_launch(c, "list objective exact"));
     }
     vmax_finalize<<<(B + 127) / 128, 128, 0, c->stream>>>(vmax, B, 1.0, 0.0, val, thr);
@@ -628,10 +629,12 @@ kc_status launch_seg_filter(kc_ctx *c, const ListBatch &L, const void *lo, const
     float g4 = (float)(4.0 * g);
     if ((double)g4 < 4.0 * g) g4 = nextafterf(g4, 1.f);
     const int gr = grid_items(c, L.W);
-    const size_t srep = nreps ? (size_t)c->K * RM * (((c->D + 1) & ~1) / 2) * 8 : 0;
+    const int dm = c->D <= 2 ? 2 : c->D <= 4 ? 4 : 8;   // attributes the kernels are compiled for
+    const size_t srep = nreps ? (size_t)c->K * RM * (dm / 2) * 8 : 0;
+    const auto fn = dm == 2 ? seg_filter_f32<2> : dm == 4 ? seg_filter_f32<4> : seg_filter_f32<8>;
     if (srep > 48 * 1024)
-        KC_CUDA(c, cudaFuncSetAttribute(seg_filter_f32<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srep));
-    seg_filter_f32<8><<<gr, 256, srep, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
+        KC_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srep));
+    fn<<<gr, 256, srep, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                  static_cast<const float *>(lo), static_cast<const float *>(hi), c->K,
                                                  c->D, beta_dn_dev, infl, slack, t_alpha, g4,
                                                  static_cast<const float *>(repx), nreps, ball, RM, rmap, out_pool, out_off,
