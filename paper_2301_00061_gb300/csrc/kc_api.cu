@@ -114,7 +114,7 @@ void kc_destroy(kc_ctx *ctx)
 {
     if (!ctx) return;
     cudaStreamSynchronize(ctx->stream);
-    for (DevBuf *b : {&ctx->part, &ctx->keys, &ctx->stage_in, &ctx->stage_out, &ctx->work, &ctx->obj, &ctx->exact,
+    for (DevBuf *b : {&ctx->part, &ctx->keys, &ctx->stage_in, &ctx->stage_out, &ctx->work, &ctx->work2, &ctx->obj, &ctx->exact,
                       &ctx->tmax, &ctx->center, &ctx->vs.buf, &ctx->vs.jbuf})
         if (b->p) cudaFree(b->p);
     if (ctx->X) cudaFree(ctx->X);
@@ -386,17 +386,20 @@ __global__ void fft_put_kernel(int64_t *__restrict__ C, int S, int K, int t, con
         C[(size_t)s * K + t] = arg[s];
 }
 
-// largest id of a list (ordered max into *out, which starts at 0)
-__global__ void max_id_kernel(const uint32_t *__restrict__ ids, int64_t n, unsigned *__restrict__ out)
+// largest id of a list (ordered max into *out, which starts at 0); vec: ids is
+// 16-byte aligned
+__global__ void __launch_bounds__(256)
+max_id_kernel(const uint32_t *__restrict__ ids, int64_t n, bool vec, unsigned *__restrict__ out)
 {
     unsigned m = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = ids[i] > m ? ids[i] : m;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned w = __shfl_xor_sync(0xffffffffu, m, o);
-        m = w > m ? w : m;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t quads = vec ? n / 4 : 0;
+    for (int64_t i = t; i < quads; i += step) {
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(ids) + i);
+        m = max(m, max(max(v.x, v.y), max(v.z, v.w)));
     }
+    for (int64_t i = 4 * quads + t; i < n; i += step) m = max(m, ids[i]);
+    m = __reduce_max_sync(0xffffffffu, m);
     if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
 }
 
@@ -493,18 +496,14 @@ kc_status kc_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, cons
     const int iarg = sg.add(argmax_out, (size_t)B * 8, false);
     KC_TRY(sg.begin());
     const uint32_t *dids = static_cast<const uint32_t *>(sg.dev(iid));
-    // the batch descriptor: one group (every node shares the subset), then
-    // scratch for the per-node keys and the id check
-    const int LT = list_tile();
-    const size_t desc = 512, keys_off = desc, chk_off = keys_off + (((size_t)B * 8 + 255) & ~(size_t)255);
-    KC_TRY(ensure(c, c->work, chk_off + 256));
-    char *w = static_cast<char *>(c->work.p);
-    unsigned *dmax = reinterpret_cast<unsigned *>(w + chk_off);
+    // scratch of the id check
+    KC_TRY(ensure(c, c->work, 256));
+    unsigned *dmax = static_cast<unsigned *>(c->work.p);
     if (n > 0) {
         // every id must name a sample: one pass over the ids, checked on the host
         KC_CUDA(c, cudaMemsetAsync(dmax, 0, 4, c->stream));
-        max_id_kernel<<<std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)c->num_sms * 8)), 256, 0,
-                        c->stream>>>(dids, n, dmax);
+        max_id_kernel<<<(int)std::max<int64_t>(1, std::min<int64_t>((n + 4095) / 4096, (int64_t)c->num_sms * 8)), 256, 0,
+                        c->stream>>>(dids, n, (uintptr_t)dids % 16 == 0, dmax);
         KC_TRY(after_launch(c, "subset id check"));
         unsigned hmax = 0;
         KC_CUDA(c, cudaMemcpyAsync(&hmax, dmax, 4, cudaMemcpyDeviceToHost, c->stream));
@@ -512,20 +511,6 @@ kc_status kc_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, cons
         if ((int64_t)hmax >= c->N)
             return set_err(c, KC_EINVAL, "kc_lower_bounds_subset: id %u outside [0, N)", hmax);
     }
-    int64_t hd[7] = {0, n, 0, (n + LT - 1) / LT, 0, 0, 0};   // seg_off, seg_n, tile_prefix[2], node_start[2]
-    int *ns = reinterpret_cast<int *>(&hd[4]);
-    ns[0] = 0;
-    ns[1] = B;
-    KC_CUDA(c, cudaMemcpyAsync(w, hd, sizeof(hd), cudaMemcpyHostToDevice, c->stream));
-    const int64_t *dd = reinterpret_cast<const int64_t *>(w);
-    ListBatch L;
-    L.pool = dids;
-    L.seg_off = dd;
-    L.seg_n = dd + 1;
-    L.tile_prefix = dd + 2;
-    L.node_start = reinterpret_cast<const int *>(dd + 4);
-    L.B = 1;
-    L.W = hd[3];
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (kernel_ms_out) {
         KC_CUDA(c, cudaEventCreate(&e0));
@@ -535,9 +520,8 @@ kc_status kc_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, cons
         }
         cudaEventRecord(e0, c->stream);
     }
-    kc_status st = launch_seg_lb(c, L, sg.dev(ilo), sg.dev(ihi), B, reinterpret_cast<unsigned long long *>(w + keys_off),
-                                 static_cast<double *>(sg.dev(ilb)), static_cast<double *>(sg.dev(iraw)),
-                                 static_cast<int64_t *>(sg.dev(iarg)));
+    kc_status st = launch_lower_bounds_subset(c, dids, n, sg.dev(ilo), sg.dev(ihi), B, static_cast<double *>(sg.dev(ilb)),
+                                              static_cast<double *>(sg.dev(iraw)), static_cast<int64_t *>(sg.dev(iarg)));
     if (kernel_ms_out) {
         cudaEventRecord(e1, c->stream);
         if (st == KC_OK && cudaEventSynchronize(e1) == cudaSuccess) cudaEventElapsedTime(kernel_ms_out, e0, e1);

@@ -59,6 +59,7 @@ struct kc_ctx {
     kc::DevBuf stage_in;         // staged host inputs
     kc::DevBuf stage_out;        // device-side outputs destined for host
     kc::DevBuf work;             // per-call work arrays
+    kc::DevBuf work2;            // gathered rows of a subset
     kc::DevBuf obj;              // coordinates of the centers being evaluated
     kc::DevBuf exact;            // kc_exact.cu: screen keys and exact maxima, zero between calls
     kc::DevBuf tmax;             // kc_exact.cu: the screen's largest value per tile and node
@@ -197,6 +198,8 @@ kc_status launch_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B, 
                               double *lb_raw, int64_t *argmax);
 kc_status launch_lower_bounds_view(kc_ctx *c, const View &v, const void *lo, const void *hi, int B,
                                    double *lb, double *lb_raw, int64_t *arg, int st_override);
+kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, const void *lo, const void *hi, int B,
+                                     double *lb, double *lb_raw, int64_t *arg);
 kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, const void *hi, int B, double *lb,
                                   double *lb_raw, int64_t *arg, int st_override, int chunk_override);
 kc_status launch_lower_bounds_refine(kc_ctx *c, const View &v, const void *lo, const void *hi, int B,

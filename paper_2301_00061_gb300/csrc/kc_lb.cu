@@ -169,6 +169,29 @@ __global__ void lb_finalize_f64(const double *__restrict__ pval, const uint32_t 
     }
 }
 
+constexpr int64_t kSubsetChunk = (int64_t)1 << 25;
+
+// Rows of the samples named by ids: out[a * ldo + i] = X[a * ld + ids[i]].
+__global__ void __launch_bounds__(256)
+gather_rows_kernel(const float *__restrict__ X, int64_t ld, int D, const uint32_t *__restrict__ ids, int64_t n,
+                   float *__restrict__ out, int64_t ldo)
+{
+    for (int64_t i0 = (int64_t)blockIdx.x * 1024; i0 < n; i0 += (int64_t)gridDim.x * 1024) {
+        uint32_t id[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int64_t i = i0 + j * 256 + threadIdx.x;
+            id[j] = i < n ? ids[i] : 0u;
+        }
+        for (int a = 0; a < D; ++a)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int64_t i = i0 + j * 256 + threadIdx.x;
+                if (i < n) out[(size_t)a * ldo + i] = __ldg(X + (size_t)a * ld + id[j]);
+            }
+    }
+}
+
 // ---------------------------------------------------------------- dispatch
 
 // Launches the float maxima of A.B nodes into A.keys (zeroed by the caller) on
@@ -273,6 +296,56 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
         KC_TRY(launch_exact_max(c, v, lo, hi, B, K, __builtin_huge_val(), lb, lb_raw, arg));
     }
     return KC_OK;
+}
+
+// Float bounds of B nodes over the samples named by ids [n] (device, D <= 8,
+// every id below N): few nodes gather as they stream, batches gather the samples
+// into rows of their own first (at most kSubsetChunk at a time) and prune.
+kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, const void *lo, const void *hi, int B,
+                                     double *lb, double *lb_raw, int64_t *arg)
+{
+    const int D = c->D;
+    if (c->keys.bytes < (size_t)B * 8) {
+        KC_TRY(ensure(c, c->keys, (size_t)B * 8));
+        KC_CUDA(c, cudaMemsetAsync(c->keys.p, 0, c->keys.bytes, c->stream));
+    }
+    PruneArgs A{};
+    A.lo = lo;
+    A.hi = hi;
+    A.B = B;
+    A.K = c->K;
+    A.D = D;
+    A.keys = static_cast<unsigned long long *>(c->keys.p);
+    if (n > 0 && use_stream_f32(B, c->K, D)) {
+        A.X = c->X;
+        A.ld = c->ldx;
+        A.n = n;
+        A.ids = ids;
+        A.vec = (uintptr_t)ids % 16 == 0;
+        KC_CUDA(c, launch_stream_gather_f32(A, c->num_sms, c->stream));
+        ++c->launches;
+    } else if (n > 0) {
+        const int64_t chunk = std::min(n, kSubsetChunk), ld = (chunk + 63) / 64 * 64;
+        KC_TRY(ensure(c, c->work2, (size_t)ld * D * 4));
+        for (int64_t i0 = 0; i0 < n; i0 += chunk) {
+            const int64_t m = std::min(chunk, n - i0);
+            const int grid = (int)std::min<int64_t>((m + 1023) / 1024, (int64_t)c->num_sms * 8);
+            gather_rows_kernel<<<grid, 256, 0, c->stream>>>(static_cast<const float *>(c->X), c->ldx, D, ids + i0, m,
+                                                            static_cast<float *>(c->work2.p), ld);
+            KC_TRY(after_launch(c, "subset gather"));
+            A.X = c->work2.p;
+            A.ld = ld;
+            A.n = m;
+            A.ids = ids + i0;
+            A.vec = 1;
+            KC_CUDA(c, prune_run(prune_pick(prune_table<false, false>(), D, m, c->num_sms, 0), A, false, c->num_sms,
+                                 c->smem_optin > 0 ? c->smem_optin : 48 * 1024, 0, c->stream));
+            ++c->launches;
+        }
+    }
+    lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B, nullptr, deflate_factor(KC_F32, D),
+                                                            underflow_slack(KC_F32, D), lb, lb_raw, arg);
+    return after_launch(c, "lower bound finalize");
 }
 
 kc_status launch_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B, double *lb,

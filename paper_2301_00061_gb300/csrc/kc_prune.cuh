@@ -55,6 +55,7 @@ struct PruneArgs {
     const void *lo, *hi;      // [B][K][D] in the samples' type
     int B, K, D;
     int per;                  // nodes per CTA range (blockIdx.y), a multiple of kPG unless B is smaller
+    const uint32_t *ids;      // NULL, or the names of the samples: keys hold ids[position]
     int vec;                  // rows may be read with 16-byte loads (X 16-byte aligned, ld a multiple of 16 bytes)
     unsigned long long *keys; // [B] (value bits, ~position), zero before the launch
     // screens of an exact maximum (kc_exact.cu): the largest float value of each
@@ -513,6 +514,7 @@ prune_max_kernel(const PruneArgs A)
         if (seed) {
             // the first tile's farthest samples, against every node
             const int64_t cp = (int64_t)(uint32_t)cand[lane];
+            const uint32_t cid = A.ids ? A.ids[cp] : (uint32_t)cp;
             uint64_t xc[1][P];
 #pragma unroll
             for (int p = 0; p < P; ++p)
@@ -524,7 +526,7 @@ prune_max_kernel(const PruneArgs A)
                     box_dists<1, P, PT>(xc, box + ((size_t)b * K + k) * RW, d);
                     best = fminf(best, d[0]);
                 }
-                raise(b, key_max(best, (uint32_t)cp));
+                raise(b, key_max(best, cid));
             }
             seed = false;
         }
@@ -532,7 +534,8 @@ prune_max_kernel(const PruneArgs A)
 #pragma unroll
         for (int j = 0; j < ST; ++j) {
             const int o = off[j] + base[r[j]];
-            spos[o] = (uint32_t)(s0 + j < A.n ? s0 + j : A.n - 1);
+            const int64_t w = s0 + j < A.n ? s0 + j : A.n - 1;
+            spos[o] = A.ids ? A.ids[w] : (uint32_t)w;
             rr[o] = (uint8_t)r[j];
 #pragma unroll
             for (int p = 0; p < P; ++p) stage[(size_t)p * T + o] = x[j][p];
@@ -747,6 +750,8 @@ inline bool use_stream_f32(int B, int K, int D)
     return (D <= 8 && B * K * D <= kStreamTerms) || (B <= 2 && B * K <= kStreamCols);
 }
 cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream);
+// The same over the samples A.ids[0 .. A.n) of the rows A.X (D <= 8).
+cudaError_t launch_stream_gather_f32(const PruneArgs &A, int sms, cudaStream_t stream);
 constexpr int kStreamTile = 128;   // samples of a tmax row of the streaming screen
 
 }  // namespace kc

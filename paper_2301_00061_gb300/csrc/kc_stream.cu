@@ -118,7 +118,7 @@ __device__ __forceinline__ void stream_finish(const PruneArgs &A, int b, unsigne
 // K fixed, the loop over the clusters unrolled; 0: any K, about 8 % slower).
 // MANY (more than two nodes): each warp keeps its nodes' keys in shared memory
 // and reduces over its lanes only when one of them may beat the key.
-template <int DC, int KC, int Q, int CTAS, bool MANY, bool TM>
+template <int DC, int KC, int Q, int CTAS, bool MANY, bool TM, bool GATHER = false>
 __global__ void __launch_bounds__(kThreads, CTAS)
 stream_max_small(const PruneArgs A)
 {
@@ -139,11 +139,34 @@ stream_max_small(const PruneArgs A)
         // quad q of a thread: samples base + (q kThreads + tid) 4 ..
         const int64_t s0 = base + (int64_t)threadIdx.x * 4;
         uint64_t x[Q][DC][2];
+        uint32_t id[GATHER ? ST : 1];
+        if constexpr (GATHER) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
+            for (int q = 0; q < Q; ++q) {
+                const int64_t t0 = s0 + q * kThreads * 4;
+                if (A.vec && t0 + 4 <= A.n) {
+                    const uint4 v = __ldg(reinterpret_cast<const uint4 *>(A.ids + t0));
+                    id[4 * q] = v.x; id[4 * q + 1] = v.y; id[4 * q + 2] = v.z; id[4 * q + 3] = v.w;
+                } else {
 #pragma unroll
-            for (int a = 0; a < DC; ++a)
-                load_quad(X + (size_t)a * A.ld, A.n, A.vec != 0, s0 + q * kThreads * 4, x[q][a]);
+                    for (int j = 0; j < 4; ++j) id[4 * q + j] = __ldg(A.ids + (t0 + j < A.n ? t0 + j : A.n - 1));
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+#pragma unroll
+                for (int a = 0; a < DC; ++a)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+                        x[q][a][h] = pk(__ldg(X + (size_t)a * A.ld + id[4 * q + 2 * h]),
+                                        __ldg(X + (size_t)a * A.ld + id[4 * q + 2 * h + 1]));
+        } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+#pragma unroll
+                for (int a = 0; a < DC; ++a)
+                    load_quad(X + (size_t)a * A.ld, A.n, A.vec != 0, s0 + q * kThreads * 4, x[q][a]);
+        }
         uint64_t xs[Q][DC][2];
 #pragma unroll
         for (int q = 0; q < Q; ++q)
@@ -207,7 +230,8 @@ stream_max_small(const PruneArgs A)
 #pragma unroll
                     for (int j = 0; j < ST; ++j) {
                         const int64_t s = s0 + (j / 4) * kThreads * 4 + j % 4;
-                        const unsigned long long c = may ? key_max(m[j], (uint32_t)(s < A.n ? s : A.n - 1)) : 0ull;
+                        const uint32_t pos = GATHER ? id[GATHER ? j : 0] : (uint32_t)(s < A.n ? s : A.n - 1);
+                        const unsigned long long c = may ? key_max(m[j], pos) : 0ull;
                         key = c > key ? c : key;
                     }
                     key = warp_max_u64(key);
@@ -335,6 +359,19 @@ StreamKernel small_kernel_of(int D, int K, bool many, bool tm)
     default: return small_kernel_k<8>(K, many, tm);
     }
 }
+StreamKernel gather_kernel_of(int D)
+{
+    switch (D) {
+    case 1: return stream_max_small<1, 0, 2, 4, true, false, true>;
+    case 2: return stream_max_small<2, 0, 2, 4, true, false, true>;
+    case 3: return stream_max_small<3, 0, 1, 4, true, false, true>;
+    case 4: return stream_max_small<4, 0, 1, 4, true, false, true>;
+    case 5: return stream_max_small<5, 0, 1, 3, true, false, true>;
+    case 6: return stream_max_small<6, 0, 1, 3, true, false, true>;
+    case 7: return stream_max_small<7, 0, 1, 3, true, false, true>;
+    default: return stream_max_small<8, 0, 1, 3, true, false, true>;
+    }
+}
 template <bool TM>
 StreamKernel wide_kernel_of(int cols)
 {
@@ -353,6 +390,20 @@ cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream)
         fn = small_kernel_of(A.D, A.K, A.B > 2, tm);
         smem += (size_t)kThreads / 32 * A.B * 8;
     }
+    int per_sm = 0;
+    const cudaError_t r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem);
+    if (r != cudaSuccess) return r;
+    const int64_t tiles = (A.n + kThreads * 4 * Q - 1) / (kThreads * 4 * Q);
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)std::max(1, per_sm) * sms));
+    fn<<<grid, kThreads, smem, stream>>>(A);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_stream_gather_f32(const PruneArgs &A, int sms, cudaStream_t stream)
+{
+    const int Q = A.D <= 2 ? 2 : 1;
+    const size_t smem = (size_t)A.B * A.K * A.D * 16 + (size_t)kThreads / 32 * A.B * 8;
+    const StreamKernel fn = gather_kernel_of(A.D);
     int per_sm = 0;
     const cudaError_t r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem);
     if (r != cudaSuccess) return r;
