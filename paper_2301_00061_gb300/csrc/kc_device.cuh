@@ -30,6 +30,14 @@ __device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b)
     return r;
 }
 
+// (a.x + b.x, a.y + b.y), each correctly rounded.
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
 // (a.x*b.x + c.x, a.y*b.y + c.y), each fused (one rounding).
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
 {

@@ -18,13 +18,6 @@ namespace {
 // that meet in one sum, so each lane's value is box_dist_f32's.  The upper
 // difference is taken of the swapped pair, so that the 3-input maximum reads
 // one even and one odd register (220 against 235 us at four nodes).
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
-{
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-
 __device__ __forceinline__ float min3f(float a, float b, float c)
 {
     float r;

@@ -201,50 +201,21 @@ struct WarpKeys {
     unsigned long long *__restrict__ dmax, *__restrict__ dmin;
 };
 
-// u64 words of a warp's key slot: the keys, then a (lo, hi) pair of floats per
-// cluster and attribute (its core)
-__host__ __device__ constexpr int warp_key_words(int K, int D, int ndir) { return 2 * K * D + 2 * K * ndir + K * D; }
+// u64 words of a warp's key slot: the keys, then one (max, -min) pair of floats
+// per cluster and direction, the limits.
+__host__ __device__ constexpr int warp_key_words(int K, int D, int ndir) { return 3 * K * (D + ndir); }
 
-// The core of cluster k: an open box in which no sample can raise a key of the
-// cluster, so that an assigned sample is one test of D intervals instead of
-// D + ndir pairs of compares (an assigned sample took about 200 instructions, and
-// all but one in a thousand lie in the core once the first tiles are in).  The
-// attributes' ranges shrunk about their middles by one factor until every pair
-// direction's extremes lie outside: x_a < H_a and x_b < H_b give
-// fl(x_a + x_b) <= fl(H_a + H_b), which is checked to be below the key.
-__device__ __forceinline__ void core_of(const unsigned long long *sk, int k, int K, int D, int ndir, uint64_t *core)
+// The limits of one direction from its keys (max at slot, min at slot + 1): a
+// value v can raise one of them only if max(v - max, min - v) >= 0, which costs
+// one packed difference and one 3-input maximum a direction; with the keys
+// compared one by one an assigned sample took some 200 instructions.  Other
+// lanes may be raising the keys: limits that lag let a sample through, no more.
+__device__ __forceinline__ uint64_t limits_of(const unsigned long long *slot)
 {
-    using KT = Key<float>;
-    const int lane = threadIdx.x & 31;
-    const unsigned long long *sa = sk + (size_t)k * D * 2, *sd = sk + (size_t)2 * K * D + (size_t)k * ndir * 2;
+    const unsigned long long a = *const_cast<const volatile unsigned long long *>(slot);
+    const unsigned long long b = *const_cast<const volatile unsigned long long *>(slot + 1);
     const float INF = __int_as_float(0x7f800000);
-    bool ok = sa[0] != 0ull;
-    float t = 1.f;
-    auto mid = [&](int a) { return 0.5f * KT::vmax(sa[2 * a]) + 0.5f * KT::vmin(sa[2 * a + 1]); };
-    auto half = [&](int a) { return 0.5f * KT::vmax(sa[2 * a]) - 0.5f * KT::vmin(sa[2 * a + 1]); };
-    int pa = 0, pb = 0;
-    const bool pair = ok && lane < ndir / 2;
-    float smx = 0.f, smn = 0.f, dmx = 0.f, dmn = 0.f;
-    if (pair) {
-        int r = lane;
-        while (r >= D - 1 - pa) r -= D - 1 - pa++;
-        pb = pa + 1 + r;
-        const unsigned long long *q = sd + 4 * lane;   // sum (max, min), difference (max, min)
-        smx = KT::vmax(q[0]), smn = KT::vmin(q[1]), dmx = KT::vmax(q[2]), dmn = KT::vmin(q[3]);
-        const float ms = mid(pa) + mid(pb), md = mid(pa) - mid(pb), w = half(pa) + half(pb);
-        t = 0.999f * fminf(fminf(smx - ms, ms - smn), fminf(dmx - md, md - dmn)) / w;
-        if (!(t > 0.f)) t = 0.f;   // (also 0 / 0)
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) t = fminf(t, __shfl_xor_sync(0xffffffffu, t, o));
-    auto low = [&](int a) { return fmaxf(mid(a) - t * half(a), KT::vmin(sa[2 * a + 1])); };
-    auto high = [&](int a) { return fminf(mid(a) + t * half(a), KT::vmax(sa[2 * a])); };
-    if (pair) {
-        const float la = low(pa), ha = high(pa), lb = low(pb), hb = high(pb);
-        ok = __fadd_rn(ha, hb) < smx && __fadd_rn(la, lb) > smn && __fsub_rn(ha, lb) < dmx && __fsub_rn(la, hb) > dmn;
-    }
-    ok = __all_sync(0xffffffffu, ok) && t > 0.f;
-    if (lane < D) core[k * D + lane] = ok ? pk(low(lane), high(lane)) : pk(INF, -INF);
+    return pk(a ? Key<float>::vmax(a) : -INF, b ? -Key<float>::vmin(b) : -INF);
 }
 
 // Raise the float key at `slot` (max) and `slot + 1` (min) by value v of the
@@ -279,22 +250,22 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
     using KY = typename KT::K;
     constexpr bool F32 = sizeof(T) == 4;
     const int lane = threadIdx.x & 31;
-    uint64_t *core = nullptr;
+    uint64_t *lim = nullptr;   // float data: [K][D + ndir]
     if constexpr (F32) {
-        core = reinterpret_cast<uint64_t *>(dk.sk) + 2 * K * (D + dk.ndir);
+        lim = reinterpret_cast<uint64_t *>(dk.sk) + 2 * K * (D + dk.ndir);
         for (int i = lane; i < K * D; i += 32) {
             const size_t o = (size_t)b * K * D + i;
             dk.sk[2 * i] = *const_cast<const volatile unsigned long long *>(&amax[o]);
             dk.sk[2 * i + 1] = *const_cast<const volatile unsigned long long *>(&amin[o]);
+            lim[i / D * (D + dk.ndir) + i % D] = limits_of(dk.sk + 2 * i);
         }
         unsigned long long *sd = dk.sk + (size_t)2 * K * D;
         for (int i = lane; i < K * dk.ndir; i += 32) {
             const size_t o = (size_t)b * K * dk.ndir + i;
             sd[2 * i] = *const_cast<const volatile unsigned long long *>(&dk.dmax[o]);
             sd[2 * i + 1] = *const_cast<const volatile unsigned long long *>(&dk.dmin[o]);
+            lim[i / dk.ndir * (D + dk.ndir) + D + i % dk.ndir] = limits_of(sd + 2 * i);
         }
-        __syncwarp();
-        for (int k = 0; k < K; ++k) core_of(dk.sk, k, K, D, dk.ndir, core);
         __syncwarp();
     }
     bool raised = false;
@@ -378,31 +349,50 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
                             }
                     }
             } else {
-                bool in = true;
+                uint64_t *lm = lim + k1 * (D + dk.ndir);
+                float over = -1.f;
 #pragma unroll
                 for (int a = 0; a < DM; ++a)
                     if (a < D) {
-                        const float2 c = upk(core[k1 * D + a]);
-                        in = in && x[a] > c.x && x[a] < c.y;
+                        const float2 t = upk(sub2(px[a], lm[a]));
+                        over = max3f(over, t.x, t.y);
                     }
-                if (in) continue;
+                int q = 0;
+#pragma unroll
+                for (int a = 0; a < DM; ++a)
+#pragma unroll
+                    for (int c = a + 1; c < DM; ++c)
+                        if (c < D && q < dk.ndir) {
+                            const float2 t = upk(sub2(add2(px[a], px[c]), lm[D + q]));
+                            const float2 u = upk(sub2(sub2(px[a], px[c]), lm[D + q + 1]));
+                            over = max3f(max3f(over, t.x, t.y), u.x, u.y);
+                            q += 2;
+                        }
+                if (!(over >= 0.f)) continue;
                 unsigned long long *sa = dk.sk + (size_t)k1 * D * 2;
 #pragma unroll
                 for (int a = 0; a < DM; ++a)
-                    if (a < D) raised |= raise_keys(sa + 2 * a, x[a], pos);
-                if (dk.ndir > 0) {
-                    unsigned long long *s = dk.sk + (size_t)2 * K * D + (size_t)k1 * dk.ndir * 2;
-                    int q = 0;
+                    if (a < D && raise_keys(sa + 2 * a, x[a], pos)) {
+                        raised = true;
+                        lm[a] = limits_of(sa + 2 * a);
+                    }
+                unsigned long long *sd = dk.sk + (size_t)2 * K * D + (size_t)k1 * dk.ndir * 2;
+                q = 0;
 #pragma unroll
-                    for (int a = 0; a < DM; ++a)
+                for (int a = 0; a < DM; ++a)
 #pragma unroll
-                        for (int c = a + 1; c < DM; ++c)
-                            if (c < D && q < dk.ndir) {
-                                raised |= raise_keys(s + 2 * q, __fadd_rn(x[a], x[c]), pos);
-                                raised |= raise_keys(s + 2 * q + 2, __fsub_rn(x[a], x[c]), pos);
-                                q += 2;
+                    for (int c = a + 1; c < DM; ++c)
+                        if (c < D && q < dk.ndir) {
+                            if (raise_keys(sd + 2 * q, __fadd_rn(x[a], x[c]), pos)) {
+                                raised = true;
+                                lm[D + q] = limits_of(sd + 2 * q);
                             }
-                }
+                            if (raise_keys(sd + 2 * q + 2, __fsub_rn(x[a], x[c]), pos)) {
+                                raised = true;
+                                lm[D + q + 1] = limits_of(sd + 2 * q + 2);
+                            }
+                            q += 2;
+                        }
             }
         }
     }
@@ -757,13 +747,21 @@ constexpr int kSub = 256;   // samples flagged per warp before processing
 // the warp's running bounding boxes, merged into global memory at the end.
 template <typename T, int KM, int DM>
 struct PBSlot {
-    uint64_t bx[KM][DM];                 // float data: packed (lo, -hi) of the input boxes
-    T ilo[KM][DM], ihi[KM][DM];          // double data: input boxes
+    T ilo[KM][DM], ihi[KM][DM];          // input boxes
     T l[KM][DM], h[KM][DM], mid[KM][DM]; // box-BT boxes and their midpoints
     OrdT<T> smax[KM][DM], smin[KM][DM];  // bbox of S_+ (ordered integers)
     OrdT<T> jmax[KM][DM], jmin[KM][DM];  // bbox of the sample-based assigned samples
-    uint64_t c0[KM][(DM + 1) / 2];       // float data: the representatives' ball (BallTest)
+};
+template <int KM, int DM>
+struct PBSlot<float, KM, DM> {
+    uint64_t bx[KM][DM];                 // (lo, -hi) of the input boxes
+    uint64_t bt[KM][DM];                 // (lo, -hi) of the box-BT boxes
+    uint64_t mid[KM][(DM + 1) / 2];      // their midpoints
+    uint64_t c0[KM][(DM + 1) / 2];       // the representatives' ball (BallTest)
     BallTest one[KM], four[KM];          // against alpha and 4 alpha
+    uint64_t slim[KM][DM];               // (max, -min) of S_+ so far
+    unsigned smax[KM][DM], smin[KM][DM]; // its bbox (ordered integers)
+    unsigned jmax[KM][DM], jmin[KM][DM]; // bbox of the sample-based assigned samples
 };
 
 __device__ __forceinline__ unsigned to_ord(float v) { return ord_f32(v); }
@@ -774,24 +772,24 @@ __device__ __forceinline__ unsigned long long to_ord(double v) { return ord_f64(
 template <typename T, int DM>
 constexpr int rep_words() { return sizeof(T) == 4 ? (DM + 1) / 2 : DM; }
 
-template <typename T, int KM, int DM>
-__device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int jstart, int wstep, const uint32_t *tids,
+// Double data.
+template <int KM, int DM>
+__device__ __forceinline__ void pass_b_node(const double *tx, int tile, int tn, int jstart, int wstep, const uint32_t *tids,
                                             const uint32_t *__restrict__ ids, int64_t base, uint32_t *list,
-                                            PBSlot<T, KM, DM> *ws, uint64_t *wrep, int b, int K, int D, int RM,
-                                            const T *__restrict__ lo_in, const T *__restrict__ hi_in,
-                                            const T *__restrict__ blo, const T *__restrict__ bhi,
-                                            const T *__restrict__ repx, const int *__restrict__ nreps,
-                                            const int *__restrict__ allhave, const float *__restrict__ ball, double alpha,
-                                            const Margins &mg, const int64_t *seed_id, unsigned long long *__restrict__ cnt,
-                                            OrdT<T> *__restrict__ smax, OrdT<T> *__restrict__ smin,
-                                            OrdT<T> *__restrict__ jmax, OrdT<T> *__restrict__ jmin,
-                                            typename Key<T>::K *__restrict__ cand, unsigned *__restrict__ flags)
+                                            PBSlot<double, KM, DM> *ws, uint64_t *wrep, int b, int K, int D, int RM,
+                                            const double *__restrict__ lo_in, const double *__restrict__ hi_in,
+                                            const double *__restrict__ blo, const double *__restrict__ bhi,
+                                            const double *__restrict__ repx, const int *__restrict__ nreps,
+                                            const int *__restrict__ allhave, const float *, double alpha,
+                                            const Margins &, const int64_t *seed_id, unsigned long long *__restrict__ cnt,
+                                            unsigned long long *__restrict__ smax, unsigned long long *__restrict__ smin,
+                                            unsigned long long *__restrict__ jmax, unsigned long long *__restrict__ jmin,
+                                            K128 *__restrict__ cand, unsigned *__restrict__ flags)
 {
+    using T = double;
     using KT = Key<T>;
     using KY = typename KT::K;
     using OT = OrdT<T>;
-    constexpr bool F32 = sizeof(T) == 4;
-    constexpr int DH = (DM + 1) / 2;
     const int lane = threadIdx.x & 31;
     const double four_alpha = 4.0 * alpha;
     // node b: input boxes (center-based status), box-BT boxes, midpoints
@@ -799,13 +797,12 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
         const int k = i / DM, a = i % DM;
         const bool in = k < K && a < D;
         const size_t o = ((size_t)b * K + k) * D + a;
-        if constexpr (F32) ws->bx[k][a] = in ? pk((float)lo_in[o], -(float)hi_in[o]) : pk(0.f, -0.f);
-        else { ws->ilo[k][a] = in ? lo_in[o] : T(0); ws->ihi[k][a] = in ? hi_in[o] : T(0); }
+        ws->ilo[k][a] = in ? lo_in[o] : T(0);
+        ws->ihi[k][a] = in ? hi_in[o] : T(0);
         const T lv = in ? blo[o] : T(0), hv = in ? bhi[o] : T(0);
         ws->l[k][a] = lv;
         ws->h[k][a] = hv;
-        if constexpr (F32) ws->mid[k][a] = (float)(0.5 * ((double)lv + (double)hv));
-        else ws->mid[k][a] = 0.5 * (lv + hv);
+        ws->mid[k][a] = 0.5 * (lv + hv);
         ws->smax[k][a] = (OT)0;
         ws->smin[k][a] = ~(OT)0;
         ws->jmax[k][a] = (OT)0;
@@ -815,18 +812,6 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
 #pragma unroll
     for (int k = 0; k < KM; ++k) nr[k] = k < K ? nreps[(size_t)b * K + k] : 0;
     const bool have = allhave[b] == K;
-    if constexpr (F32) {
-        for (int i = lane; i < KM * DH; i += 32) {
-            const int k = i / DH, p = i % DH;
-            const float *c = ball + ((size_t)b * K + k) * (D + 2);
-            ws->c0[k][p] = pk(k < K && 2 * p < D ? c[2 * p] : 0.f, k < K && 2 * p + 1 < D ? c[2 * p + 1] : 0.f);
-        }
-        if (lane < K) {
-            const float *c = ball + ((size_t)b * K + lane) * (D + 2) + D;
-            ws->one[lane] = ball_test(mg.t_alpha, c[0], c[1], mg.g4);
-            ws->four[lane] = ball_test(mg.t_four, c[0], c[1], mg.g4);
-        }
-    }
     // the node's representatives into the warp's slot wrep [K][RM][words]
     constexpr int RW = rep_words<T, DM>();
     {
@@ -837,14 +822,8 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
             const T *src = rxb + (size_t)k * RM * D;
             for (int i = lane; i < nr[k] * RW; i += 32) {
                 const int r = i / RW, p = i - r * RW;
-                if constexpr (F32) {
-                    const float v0 = 2 * p < D ? (float)src[(size_t)r * D + 2 * p] : 0.f;
-                    const float v1 = 2 * p + 1 < D ? (float)src[(size_t)r * D + 2 * p + 1] : 0.f;
-                    wrep[((size_t)k * RM + r) * RW + p] = pk(v0, v1);
-                } else {
-                    const double v = p < D ? (double)src[(size_t)r * D + p] : 0.0;
-                    wrep[((size_t)k * RM + r) * RW + p] = (uint64_t)__double_as_longlong(v);
-                }
+                const double v = p < D ? src[(size_t)r * D + p] : 0.0;
+                wrep[((size_t)k * RM + r) * RW + p] = (uint64_t)__double_as_longlong(v);
             }
         }
     }
@@ -875,18 +854,7 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
 #pragma unroll
                 for (int k = 0; k < KM; ++k)
                     if (have && k < K) {
-                        bool excl;
-                        if constexpr (F32) {
-                            uint64_t px[DM];
-#pragma unroll
-                            for (int a = 0; a < DM; ++a) px[a] = pk(x[a], -x[a]);
-                            excl = box_dist_f32<DM>(px, ws->bx[k]) > mg.t_alpha;
-                        } else {
-                            excl = box_dist_f64<DM>(reinterpret_cast<const double *>(x),
-                                                    reinterpret_cast<const double *>(ws->ilo[k]),
-                                                    reinterpret_cast<const double *>(ws->ihi[k]), D) > alpha;
-                        }
-                        if (!excl) ++left;
+                        if (!(box_dist_f64<DM>(x, ws->ilo[k], ws->ihi[k], D) > alpha)) ++left;
                     }
                 if (have && left >= 2) {
                     // the seeds count as assigned in every node
@@ -921,11 +889,6 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
             T x[DM];
 #pragma unroll
             for (int a = 0; a < DM; ++a) x[a] = a < D ? tx[(size_t)a * tile + j] : T(0);
-            uint64_t px[DH];
-            if constexpr (F32) {
-#pragma unroll
-                for (int p = 0; p < DH; ++p) px[p] = pk(x[2 * p], 2 * p + 1 < DM ? x[2 * p + 1] : 0.f);
-            }
             // distances to the representatives of the clusters that need them:
             // far4[k] = some representative of k proved farther than 4 alpha
             // (Lemma 2), far1[k] = some proved farther than alpha (ball test).
@@ -933,24 +896,14 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
             // distance (a short last chunk repeats the last representative);
             // far4 implies far1, so a cluster's scan stops at its first far4,
             // or at its first far1 when only the ball test needs it
-            const T th1 = F32 ? (T)mg.t_alpha : (T)alpha, th4 = F32 ? (T)mg.t_four : (T)four_alpha;
+            const T th1 = alpha, th4 = four_alpha;
             bool far4[KM], far1[KM];
 #pragma unroll
             for (int k = 0; k < KM; ++k) {
                 far4[k] = far1[k] = false;
                 const bool need = k < K && ((fl & 1u) || (fl & (2u << k)));
                 if (!need) continue;
-                bool want4 = (fl & 1u) != 0u;
-                if constexpr (F32) {
-                    // the ball decides most samples
-                    const float dc = pt_dist_f32<2 * DH>(px, ws->c0[k]);
-                    const BallTest b1 = ws->one[k], b4 = ws->four[k];
-                    if (dc > b1.far) far1[k] = true;
-                    if (dc > b4.far) far4[k] = true;
-                    want4 = want4 && !far4[k] && !(dc <= b4.near);
-                    const bool want1 = (fl & (2u << k)) && !far1[k] && !(dc <= b1.near);
-                    if (!want1 && !want4) continue;
-                }
+                const bool want4 = (fl & 1u) != 0u;
                 const uint64_t *rk = wrep + (size_t)k * RM * RW;
                 const int nk = nr[k];
                 for (int r0 = 0; r0 < nk; r0 += 4) {
@@ -958,14 +911,9 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
 #pragma unroll
                     for (int u = 0; u < 4; ++u) {
                         const int r = r0 + u < nk ? r0 + u : nk - 1;
-                        if constexpr (F32) d[u] = pt_dist_f32<2 * DH>(px, rk + (size_t)r * RW);
-                        else
-                            d[u] = pt_dist_f64<DM>(reinterpret_cast<const double *>(x),
-                                                   reinterpret_cast<const double *>(rk + (size_t)r * RW), D);
+                        d[u] = pt_dist_f64<DM>(x, reinterpret_cast<const double *>(rk + (size_t)r * RW), D);
                     }
-                    T m;
-                    if constexpr (F32) m = fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3]));
-                    else m = fmax(fmax(d[0], d[1]), fmax(d[2], d[3]));
+                    const T m = fmax(fmax(d[0], d[1]), fmax(d[2], d[3]));
                     if (m > th1) {
                         far1[k] = true;
                         if (m > th4) { far4[k] = true; break; }
@@ -999,17 +947,7 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
                         if (v > ws->smax[k][a]) atomicMax(&ws->smax[k][a], v);
                         if (v < ws->smin[k][a]) atomicMin(&ws->smin[k][a], v);
                     }
-                    T dm;
-                    if constexpr (F32) {
-                        uint64_t pm[DH];
-#pragma unroll
-                        for (int p = 0; p < DH; ++p)
-                            pm[p] = pk(ws->mid[k][2 * p], 2 * p + 1 < DM ? ws->mid[k][2 * p + 1] : 0.f);
-                        dm = pt_dist_f32<2 * DH>(px, pm);
-                    } else {
-                        dm = pt_dist_f64<DM>(reinterpret_cast<const double *>(x),
-                                             reinterpret_cast<const double *>(ws->mid[k]), D);
-                    }
+                    const T dm = pt_dist_f64<DM>(x, ws->mid[k], D);
                     c_cand[k] = kmax<T>(c_cand[k], KT::min_of(dm, pos));
                 }
         }
@@ -1040,6 +978,246 @@ __device__ __forceinline__ void pass_b_node(const T *tx, int tile, int tn, int j
     if (__any_sync(0xffffffffu, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
 }
 
+// Float data: the same decisions.  Tiles hold (x, -x) pairs, so that being outside
+// a box (or beyond the bounding box of S_+ so far) is one packed difference and
+// one 3-input maximum per attribute; the ball around a cluster's
+// representatives decides most samples, and the representatives are staged only
+// when some lane has to scan them.
+template <int KM, int DM>
+__device__ __forceinline__ void pass_b_node(const uint64_t *tx, int tile, int tn, int jstart, int wstep,
+                                            const uint32_t *tids, const uint32_t *__restrict__ ids, int64_t base,
+                                            uint32_t *list, PBSlot<float, KM, DM> *ws, uint64_t *wrep, int b, int K, int D,
+                                            int RM, const float *__restrict__ lo_in, const float *__restrict__ hi_in,
+                                            const float *__restrict__ blo, const float *__restrict__ bhi,
+                                            const float *__restrict__ repx, const int *__restrict__ nreps,
+                                            const int *__restrict__ allhave, const float *__restrict__ ball, double,
+                                            const Margins &mg, const int64_t *seed_id, unsigned long long *__restrict__ cnt,
+                                            unsigned *__restrict__ smax, unsigned *__restrict__ smin,
+                                            unsigned *__restrict__ jmax, unsigned *__restrict__ jmin,
+                                            unsigned long long *__restrict__ cand, unsigned *__restrict__ flags)
+{
+    using KT = Key<float>;
+    constexpr int DH = (DM + 1) / 2, RW = rep_words<float, DM>();
+    constexpr unsigned ALL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const float INF = __int_as_float(0x7f800000);
+    auto mid_of = [&](size_t o) { return (float)(0.5 * ((double)blo[o] + (double)bhi[o])); };
+    // node b: input boxes (center-based status), box-BT boxes, midpoints
+    for (int i = lane; i < KM * DM; i += 32) {
+        const int k = i / DM, a = i % DM;
+        const bool in = k < K && a < D;
+        const size_t o = ((size_t)b * K + k) * D + a;
+        ws->bx[k][a] = in ? pk(lo_in[o], -hi_in[o]) : pk(0.f, -0.f);
+        ws->bt[k][a] = in ? pk(blo[o], -bhi[o]) : pk(0.f, -0.f);
+        ws->slim[k][a] = in ? pk(-INF, -INF) : pk(0.f, -0.f);
+        ws->smax[k][a] = 0u;
+        ws->smin[k][a] = ~0u;
+        ws->jmax[k][a] = 0u;
+        ws->jmin[k][a] = ~0u;
+    }
+    for (int i = lane; i < KM * DH; i += 32) {
+        const int k = i / DH, p = i % DH;
+        const bool i0 = k < K && 2 * p < D, i1 = k < K && 2 * p + 1 < D;
+        const size_t o = ((size_t)b * K + k) * D + 2 * p;
+        const float *c = ball + ((size_t)b * K + k) * (D + 2) + 2 * p;
+        ws->mid[k][p] = pk(i0 ? mid_of(o) : 0.f, i1 ? mid_of(o + 1) : 0.f);
+        ws->c0[k][p] = pk(i0 ? c[0] : 0.f, i1 ? c[1] : 0.f);
+    }
+    if (lane < K) {
+        const float *c = ball + ((size_t)b * K + lane) * (D + 2) + D;
+        ws->one[lane] = ball_test(mg.t_alpha, c[0], c[1], mg.g4);
+        ws->four[lane] = ball_test(mg.t_four, c[0], c[1], mg.g4);
+    }
+    const bool have = allhave[b] == K;
+    bool staged = false;   // the representatives are in wrep [K][RM][RW]
+    unsigned c_cnt[KM];
+    float near_d[KM];      // candidates: the smallest distance to the midpoint, and its sample
+    uint32_t near_p[KM];
+#pragma unroll
+    for (int k = 0; k < KM; ++k) {
+        c_cnt[k] = 0u;
+        near_d[k] = INF;
+        near_p[k] = ~0u;
+    }
+    __syncwarp();
+    bool infeasible = false;
+    for (int r0 = jstart; r0 < tn; r0 += 8 * wstep) {
+        // phase 1: flag the samples that need representative distances
+        int count = 0;
+        for (int g = 0; g < 8; ++g) {
+            const int jb = r0 + g * wstep;
+            if (jb >= tn) break;   // uniform across the warp
+            const int j = jb + lane;
+            uint32_t fl = 0u;
+            if (j < tn) {
+                uint64_t px[DM];
+#pragma unroll
+                for (int a = 0; a < DM; ++a) px[a] = a < D ? tx[(size_t)a * tile + j] : pk(0.f, -0.f);
+                // clusters the center-based rule leaves open (only needed when the
+                // sample-based rule can run: every cluster has representatives)
+                int left = 0;
+#pragma unroll
+                for (int k = 0; k < KM; ++k) {
+                    if (k >= K) continue;
+                    if (have && !(box_dist_f32<DM>(px, ws->bx[k]) > mg.t_alpha)) ++left;
+                    float out = 0.f;
+#pragma unroll
+                    for (int a = 0; a < DM; ++a) {
+                        const float2 t = upk(sub2(ws->bt[k][a], px[a]));
+                        out = max3f(out, t.x, t.y);
+                    }
+                    if (!(out > 0.f)) fl |= 2u << k;
+                }
+                if (left >= 2) {
+                    // the seeds count as assigned in every node
+                    const int64_t id = tids ? (int64_t)tids[j] : (ids ? (int64_t)ids[base + j] : base + j);
+                    bool is_seed = false;
+#pragma unroll
+                    for (int k = 0; k < KM; ++k)
+                        if (seed_id[k] == id) is_seed = true;
+                    if (!is_seed) fl |= 1u;
+                }
+            }
+            const unsigned bal = __ballot_sync(ALL, fl != 0u);
+            if (fl) list[count + __popc(bal & ((1u << lane) - 1u))] = (uint32_t)j | (fl << 16);
+            count += __popc(bal);
+        }
+        __syncwarp();
+        // phase 2: the representatives against the flagged samples
+        for (int e = lane; e - lane < count; e += 32) {
+            const uint32_t ent = e < count ? list[e] : 0u;
+            const int j = (int)(ent & 0xFFFFu);
+            const uint32_t fl = ent >> 16;
+            uint64_t px[DM], xx[DH];
+#pragma unroll
+            for (int a = 0; a < DM; ++a) px[a] = a < D ? tx[(size_t)a * tile + j] : pk(0.f, -0.f);
+#pragma unroll
+            for (int p = 0; p < DH; ++p) xx[p] = pk(upk(px[2 * p]).x, 2 * p + 1 < DM ? upk(px[2 * p + 1 < DM ? 2 * p + 1 : 0]).x : 0.f);
+            // far4: some representative proved farther than 4 alpha (Lemma 2); far1:
+            // than alpha (ball test); far4 implies far1
+            unsigned far4 = 0u, far1 = 0u, want4 = 0u, want1 = 0u;
+#pragma unroll
+            for (int k = 0; k < KM; ++k) {
+                if (k >= K || !((fl & 1u) || (fl & (2u << k)))) continue;
+                const float dc = pt_dist_f32<2 * DH>(xx, ws->c0[k]);
+                const BallTest b1 = ws->one[k], b4 = ws->four[k];
+                if (dc > b1.far) far1 |= 1u << k;
+                else if ((fl & (2u << k)) && !(dc <= b1.near)) want1 |= 1u << k;
+                if (dc > b4.far) far4 |= 1u << k;
+                else if ((fl & 1u) && !(dc <= b4.near)) want4 |= 1u << k;
+            }
+            if (__any_sync(ALL, (want1 | want4) != 0u)) {
+                if (!staged) {
+                    for (int k = 0; k < K; ++k) {
+                        const float *src = repx + ((size_t)b * K + k) * RM * D;
+                        const int nk = nreps[(size_t)b * K + k];
+                        for (int i = lane; i < nk * RW; i += 32) {
+                            const int r = i / RW, p = i - r * RW;
+                            wrep[((size_t)k * RM + r) * RW + p] =
+                                pk(2 * p < D ? src[(size_t)r * D + 2 * p] : 0.f,
+                                   2 * p + 1 < D ? src[(size_t)r * D + 2 * p + 1] : 0.f);
+                        }
+                    }
+                    staged = true;
+                    __syncwarp();
+                }
+                // chunks of 4 decided by their largest distance (a short last chunk
+                // repeats the last representative)
+#pragma unroll
+                for (int k = 0; k < KM; ++k) {
+                    const bool w4 = want4 >> k & 1u;
+                    if (k >= K || !(w4 || (want1 >> k & 1u))) continue;
+                    const uint64_t *rk = wrep + (size_t)k * RM * RW;
+                    const int nk = nreps[(size_t)b * K + k];
+                    for (int q0 = 0; q0 < nk; q0 += 4) {
+                        float d[4];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            d[u] = pt_dist_f32<2 * DH>(xx, rk + (size_t)(q0 + u < nk ? q0 + u : nk - 1) * RW);
+                        const float m = fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3]));
+                        if (m > mg.t_alpha) {
+                            far1 |= 1u << k;
+                            if (m > mg.t_four) { far4 |= 1u << k; break; }
+                            if (!w4) break;
+                        }
+                    }
+                }
+            }
+            // sample-based assignment of an unassigned sample (Algorithm 3, Lemma 2)
+            if (fl & 1u) {
+                const unsigned open = ((1u << K) - 1u) & ~far4;
+                if (open == 0u) infeasible = true;
+                if (open != 0u && (open & (open - 1u)) == 0u) {
+                    const int k1 = __ffs(open) - 1;
+#pragma unroll
+                    for (int a = 0; a < DM; ++a)
+                        if (a < D) {
+                            // a plain read skips the atomics that cannot change the value
+                            const unsigned v = ord_f32(upk(px[a]).x);
+                            if (v > ws->jmax[k1][a]) atomicMax(&ws->jmax[k1][a], v);
+                            if (v < ws->jmin[k1][a]) atomicMin(&ws->jmin[k1][a], v);
+                        }
+                }
+            }
+            // ball-based tightening and centers on samples (Algorithm 4)
+#pragma unroll
+            for (int k = 0; k < KM; ++k) {
+                if (k >= K || !(fl & (2u << k)) || (far1 >> k & 1u)) continue;
+                ++c_cnt[k];
+                float over = 0.f;
+#pragma unroll
+                for (int a = 0; a < DM; ++a) {
+                    const float2 t = upk(sub2(px[a], ws->slim[k][a]));
+                    over = max3f(over, t.x, t.y);
+                }
+                if (over > 0.f) {
+#pragma unroll
+                    for (int a = 0; a < DM; ++a)
+                        if (a < D) {
+                            const float x = upk(px[a]).x;
+                            const unsigned v = ord_f32(x);
+                            const unsigned hi = max(atomicMax(&ws->smax[k][a], v), v);
+                            const unsigned lo = min(atomicMin(&ws->smin[k][a], v), v);
+                            ws->slim[k][a] = pk(unord_f32(hi), -unord_f32(lo));   // (may lag behind other lanes')
+                        }
+                }
+                const float dm = pt_dist_f32<2 * DH>(xx, ws->mid[k]);
+                if (dm <= near_d[k]) {
+                    const uint32_t pos = tids ? tids[j] : (uint32_t)(base + j);
+                    if (dm < near_d[k] || pos < near_p[k]) {
+                        near_d[k] = dm;
+                        near_p[k] = pos;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+    }
+    // reduce and merge
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+        if (k < K) {
+            const unsigned cn = __reduce_add_sync(ALL, c_cnt[k]);
+            const unsigned long long cd = warp_max_u64(c_cnt[k] ? KT::min_of(near_d[k], near_p[k]) : 0ull);
+            const size_t ok_ = (size_t)b * K + k;
+            if (lane == 0 && cn) {
+                atomicAdd(&cnt[ok_], (unsigned long long)cn);
+                atomicMax(&cand[ok_], cd);
+            }
+        }
+    __syncwarp();
+    for (int i = lane; i < K * D; i += 32) {
+        const int k = i / D, a = i % D;
+        const size_t o = ((size_t)b * K + k) * D + a;
+        if (ws->smax[k][a] != 0u) atomicMax(&smax[o], ws->smax[k][a]);
+        if (ws->smin[k][a] != ~0u) atomicMin(&smin[o], ws->smin[k][a]);
+        if (ws->jmax[k][a] != 0u) atomicMax(&jmax[o], ws->jmax[k][a]);
+        if (ws->jmin[k][a] != ~0u) atomicMin(&jmin[o], ws->jmin[k][a]);
+    }
+    __syncwarp();   // the slot is rewritten by the warp's next node
+    if (__any_sync(ALL, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
+}
+
 template <typename T, int KM, int DM>
 __global__ void __launch_bounds__(kThreads, 3)
 visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, int B, int K, int D, int RM,
@@ -1055,7 +1233,8 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
 #pragma unroll
     for (int k = 0; k < KM; ++k) seed_id[k] = (seeds && k < K) ? seeds[k] : -1;
     extern __shared__ __align__(16) unsigned char smem[];
-    T *tx = reinterpret_cast<T *>(smem);                                        // [D][tile]
+    using TT = typename std::conditional<sizeof(T) == 4, uint64_t, double>::type;
+    TT *tx = reinterpret_cast<TT *>(smem);                                      // [D][tile]
     uint32_t *lists = reinterpret_cast<uint32_t *>(tx + (size_t)D * tile);      // [warps][kSub]
     auto *slots = reinterpret_cast<PBSlot<T, KM, DM> *>(lists + NWV * kSub);   // [warps]
     const int warp = threadIdx.x >> 5;
@@ -1068,11 +1247,13 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
         __syncthreads();
         for (int i = threadIdx.x; i < D * tile; i += kThreads) {
             const int a = i / tile, j = i - a * tile;
-            tx[i] = j < tn ? X[(size_t)a * ld + base + j] : T(0);
+            const T v = j < tn ? X[(size_t)a * ld + base + j] : T(0);
+            if constexpr (sizeof(T) == 4) tx[i] = pk(v, -v);
+            else tx[i] = v;
         }
         __syncthreads();
         for (int b = (int)(u % split) * NWV + warp; b < B; b += split * NWV)
-            pass_b_node<T, KM, DM>(tx, tile, tn, 0, 32, nullptr, ids, base, list, slots + warp, wrep, b, K, D, RM,
+            pass_b_node<KM, DM>(tx, tile, tn, 0, 32, nullptr, ids, base, list, slots + warp, wrep, b, K, D, RM,
                                         lo_in, hi_in, blo, bhi, repx, nreps, allhave, ball, alpha, mg, seed_id, cnt, smax,
                                         smin, jmax, jmin, cand, flags);
     }
@@ -1094,7 +1275,8 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, 
 #pragma unroll
     for (int k = 0; k < KM; ++k) seed_id[k] = (seeds && k < K) ? seeds[k] : -1;
     extern __shared__ __align__(16) unsigned char smem[];
-    T *tx = reinterpret_cast<T *>(smem);                                        // [D][tile]
+    using TT = typename std::conditional<sizeof(T) == 4, uint64_t, double>::type;
+    TT *tx = reinterpret_cast<TT *>(smem);                                      // [D][tile]
     uint32_t *lists = reinterpret_cast<uint32_t *>(tx + (size_t)D * tile);      // [warps][kSub]
     auto *slots = reinterpret_cast<PBSlot<T, KM, DM> *>(lists + NWV * kSub);   // [warps]
     uint32_t *tids = reinterpret_cast<uint32_t *>(slots + NWV);                 // [tile]
@@ -1113,14 +1295,16 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, 
         __syncthreads();
         for (int i = threadIdx.x; i < D * tile; i += kThreads) {
             const int a = i / tile, j = i - a * tile;
-            tx[i] = j < tn ? X[(size_t)a * ld + tids[j]] : T(0);
+            const T v = j < tn ? X[(size_t)a * ld + tids[j]] : T(0);
+            if constexpr (sizeof(T) == 4) tx[i] = pk(v, -v);
+            else tx[i] = v;
         }
         __syncthreads();
         const int n0 = L.node_start ? L.node_start[b] : b, n1 = L.node_start ? L.node_start[b + 1] : b + 1;
         const int teams = (n1 - n0) < NWV ? (n1 - n0) : NWV, wpt = NWV / teams, team = warp / wpt;
         if (team < teams)
             for (int nd = n0 + team; nd < n1; nd += teams)
-                pass_b_node<T, KM, DM>(tx, tile, tn, (warp % wpt) * 32, wpt * 32, tids, nullptr, 0, list,
+                pass_b_node<KM, DM>(tx, tile, tn, (warp % wpt) * 32, wpt * 32, tids, nullptr, 0, list,
                                        slots + warp, wrep, nd, K, D, RM, lo_in, hi_in, blo, bhi, repx, nreps, allhave,
                                        ball, alpha, mg, seed_id, cnt, smax, smin, jmax, jmin, cand, flags);
         (void)lane;
@@ -1454,18 +1638,18 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     // pass B
     int tileB, splitB;
     tile_units(c, v.n, B,
-               (int)std::max<int64_t>(256, std::min<int64_t>(2048, (32 * 1024) / (D * (int64_t)sizeof(T))) / 32 * 32),
+               (int)std::max<int64_t>(256, std::min<int64_t>(2048, (32 * 1024) / (D * 8)) / 32 * 32),
                &tileB, &splitB);
     static_assert(kThreads / 32 * kSub * 4 <= 16 * 1024, "pass B lists");
     const size_t slotB = (size_t)NWV * sizeof(PBSlot<T, KM, DM>);
     const size_t repB = (size_t)NWV * KM * RM * rep_words<T, DM>() * 8;   // per-warp representatives
-    const size_t smemB = (size_t)D * tileB * sizeof(T) + (size_t)NWV * kSub * 4 + slotB + repB;
+    const size_t smemB = (size_t)D * tileB * 8 + (size_t)NWV * kSub * 4 + slotB + repB;
     int gB = 1;
     auto kB = visit_b_kernel<T, KM, DM>;
     if (L) {
         if constexpr (sizeof(T) == 4) {
             const int lt = list_tile();
-            const size_t smem = (size_t)D * lt * sizeof(T) + (size_t)NWV * kSub * 4 + slotB + (size_t)lt * 4 + repB;
+            const size_t smem = (size_t)D * lt * 8 + (size_t)NWV * kSub * 4 + slotB + (size_t)lt * 4 + repB;
             auto kBL = visit_b_list_kernel<T, KM, DM>;
             int g = 1;
             KC_TRY(grid_of(c, kBL, smem, std::max<int64_t>(1, L->W), &g));
