@@ -360,18 +360,29 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
         unsigned long long best0 = 0ull, best1 = 0ull;
         float top0 = -1.f, top1 = -1.f;
         uint32_t pos0 = ~0u, pos1 = ~0u;
-        for (int j0 = 0; j0 < tn; j0 += blockDim.x) {
-            const int j = j0 + threadIdx.x;
-            bool keep = false;
-            uint32_t id = 0;
+        // a thread's entries: all their gathers in flight before the first is used
+        constexpr int U = kLT / 256;
+        uint32_t eid[U];
+        float ex[U][DMAX];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = u * 256 + threadIdx.x;
+            eid[u] = j < tn ? ids[j] : 0u;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int a = 0; a < DMAX; ++a)
+                ex[u][a] = (a < D && u * 256 + threadIdx.x < tn) ? X[(size_t)a * ld + eid[u]] : 0.f;
+        unsigned kept = 0u;   // bit u: entry u survives
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int j = u * 256 + threadIdx.x;
+            const uint32_t id = eid[u];
             if (j < tn) {
-                id = ids[j];
                 uint64_t px[DMAX];
 #pragma unroll
-                for (int a = 0; a < DMAX; ++a) {
-                    const float v = a < D ? X[(size_t)a * ld + id] : 0.f;
-                    px[a] = pk(v, -v);
-                }
+                for (int a = 0; a < DMAX; ++a) px[a] = pk(ex[u][a], -ex[u][a]);
                 // lower-bound redundancy: alpha_s(M) < beta (Eq. 13), proved in float
                 float as = __int_as_float(0x7f800000);
                 for (int k = 0; k < K; ++k) {
@@ -423,8 +434,8 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                         if (!excl) redundant = false;
                     }
                 }
-                keep = !redundant;
-                if (keep && ckeys) {
+                if (!redundant) kept |= 1u << u;
+                if (!redundant && ckeys) {
                     // children's bounds over the surviving samples (the closed form
                     // of Section 3.1 in the same float evaluation as seg_lb_f32);
                     // their boxes differ from the node's in cluster ks alone
@@ -437,16 +448,28 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                     if (v1 >= top1 && (v1 > top1 || id < pos1)) { top1 = v1; pos1 = id; }
                 }
             }
-            // one reservation per warp (no block barrier): lane 0 claims the
-            // warp's surviving entries, the others write behind it in lane order
-            const unsigned bal = __ballot_sync(0xffffffffu, keep);
-            if (bal) {
-                unsigned long long base = 0ull;
-                if (lane == 0) base = atomicAdd(&out_n[b], (unsigned long long)__popc(bal));
+        }
+        // one reservation per warp (no block barrier): lane 0 claims the warp's
+        // surviving entries, the others write behind it, each 32 entries as one
+        // run in lane order
+        unsigned bal[U];
+        int all = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            bal[u] = __ballot_sync(0xffffffffu, kept >> u & 1u);
+            all += __popc(bal[u]);
+        }
+        if (all) {
+            unsigned long long base = 0ull;
+            if (lane == 0) base = atomicAdd(&out_n[b], (unsigned long long)all);
+            if (out_pool && out_off[b] >= 0) {
                 base = __shfl_sync(0xffffffffu, base, 0);
-                const int64_t pos = (int64_t)(base + __popc(bal & ((1u << lane) - 1u)));
-                if (keep && out_pool && out_off[b] >= 0 && (!out_cap || pos < out_cap[b]))
-                    out_pool[out_off[b] + pos] = id;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t pos = (int64_t)(base + __popc(bal[u] & ((1u << lane) - 1u)));
+                    if ((kept >> u & 1u) && (!out_cap || pos < out_cap[b])) out_pool[out_off[b] + pos] = eid[u];
+                    base += __popc(bal[u]);
+                }
             }
         }
         if (ckeys) {

@@ -358,11 +358,12 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
                         over = max3f(over, t.x, t.y);
                     }
                 int q = 0;
+                const bool dirs = dk.ndir > 0;   // all pairs where D <= 6
 #pragma unroll
                 for (int a = 0; a < DM; ++a)
 #pragma unroll
                     for (int c = a + 1; c < DM; ++c)
-                        if (c < D && q < dk.ndir) {
+                        if (dirs && c < D && (DM <= 6 || q < dk.ndir)) {
                             const float2 t = upk(sub2(add2(px[a], px[c]), lm[D + q]));
                             const float2 u = upk(sub2(sub2(px[a], px[c]), lm[D + q + 1]));
                             over = max3f(max3f(over, t.x, t.y), u.x, u.y);
@@ -456,7 +457,7 @@ __device__ __forceinline__ void stage_tile_a(const T *__restrict__ X, int64_t ld
     }
 }
 
-template <typename T, int KM, int DM>
+template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads)
 visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, const T *__restrict__ lo,
                const T *__restrict__ hi, int B, int K, int D, double alpha, Margins mg,
@@ -464,6 +465,7 @@ visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
                typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags, int ndir,
                unsigned long long *__restrict__ dmax, unsigned long long *__restrict__ dmin)
 {
+    if constexpr (EX) { K = KM; D = DM; }   // known shapes: the loops unroll without tests
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *tp = reinterpret_cast<uint64_t *>(smem);
     double *td = reinterpret_cast<double *>(smem);
@@ -488,7 +490,7 @@ visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
 
 // List mode: work item w = one tile of a group's sample-id list (see
 // ListBatch); the CTA evaluates every node of the group on the staged tile.
-template <typename T, int KM, int DM>
+template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads, 3)
 visit_a_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile,
                     const T *__restrict__ lo, const T *__restrict__ hi, int K, int D, double alpha, Margins mg,
@@ -496,6 +498,7 @@ visit_a_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile,
                     typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags, int ndir,
                     unsigned long long *__restrict__ dmax, unsigned long long *__restrict__ dmin)
 {
+    if constexpr (EX) { K = KM; D = DM; }   // known shapes: the loops unroll without tests
     extern __shared__ __align__(16) unsigned char smem[];
     uint64_t *tp = reinterpret_cast<uint64_t *>(smem);
     double *td = reinterpret_cast<double *>(smem);
@@ -1218,7 +1221,7 @@ __device__ __forceinline__ void pass_b_node(const uint64_t *tx, int tile, int tn
     if (__any_sync(ALL, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
 }
 
-template <typename T, int KM, int DM>
+template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads, 3)
 visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int split, int B, int K, int D, int RM,
                const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
@@ -1229,6 +1232,7 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
                OrdT<T> *__restrict__ smax, OrdT<T> *__restrict__ smin, OrdT<T> *__restrict__ jmax,
                OrdT<T> *__restrict__ jmin, typename Key<T>::K *__restrict__ cand, unsigned *__restrict__ flags)
 {
+    if constexpr (EX) { K = KM; D = DM; }   // known shapes: the loops unroll without tests
     int64_t seed_id[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k) seed_id[k] = (seeds && k < K) ? seeds[k] : -1;
@@ -1260,7 +1264,7 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
 }
 
 // List mode of pass B (see visit_a_list_kernel).
-template <typename T, int KM, int DM>
+template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads, 3)
 visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, int K,
                     int D, int RM, const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
@@ -1271,6 +1275,7 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, 
                     OrdT<T> *__restrict__ jmax, OrdT<T> *__restrict__ jmin, typename Key<T>::K *__restrict__ cand,
                     unsigned *__restrict__ flags)
 {
+    if constexpr (EX) { K = KM; D = DM; }   // known shapes: the loops unroll without tests
     int64_t seed_id[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k) seed_id[k] = (seeds && k < K) ? seeds[k] : -1;
@@ -1592,13 +1597,15 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const size_t smemA = (size_t)D * tileA * 8 + dkA;
     int gA = 1;
     const int64_t unitsA = (v.n + tileA - 1) / tileA * splitA;
-    auto kA = visit_a_kernel<T, KM, DM>;
+    constexpr bool F32 = sizeof(T) == 4;
+    const bool ex = F32 && K_ == KM && D == DM;
+    auto kA = ex ? visit_a_kernel<T, KM, DM, F32> : visit_a_kernel<T, KM, DM, false>;
     if (L) {
         // list mode (float data): one node per work item, tile = list_tile() gathered ids
         if constexpr (sizeof(T) == 4) {
             const int lt = list_tile();
             const size_t smem = (size_t)D * lt * 8 + (size_t)lt * 4 + dkA;
-            auto kAL = visit_a_list_kernel<T, KM, DM>;
+            auto kAL = ex ? visit_a_list_kernel<T, KM, DM, true> : visit_a_list_kernel<T, KM, DM, false>;
             int g = 1;
             KC_TRY(grid_of(c, kAL, smem, std::max<int64_t>(1, L->W), &g));
             if (L->W > 0) {
@@ -1645,12 +1652,12 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const size_t repB = (size_t)NWV * KM * RM * rep_words<T, DM>() * 8;   // per-warp representatives
     const size_t smemB = (size_t)D * tileB * 8 + (size_t)NWV * kSub * 4 + slotB + repB;
     int gB = 1;
-    auto kB = visit_b_kernel<T, KM, DM>;
+    auto kB = ex ? visit_b_kernel<T, KM, DM, F32> : visit_b_kernel<T, KM, DM, false>;
     if (L) {
         if constexpr (sizeof(T) == 4) {
             const int lt = list_tile();
             const size_t smem = (size_t)D * lt * 8 + (size_t)NWV * kSub * 4 + slotB + (size_t)lt * 4 + repB;
-            auto kBL = visit_b_list_kernel<T, KM, DM>;
+            auto kBL = ex ? visit_b_list_kernel<T, KM, DM, true> : visit_b_list_kernel<T, KM, DM, false>;
             int g = 1;
             KC_TRY(grid_of(c, kBL, smem, std::max<int64_t>(1, L->W), &g));
             if (L->W > 0) {
