@@ -212,4 +212,18 @@ __device__ __forceinline__ BallTest ball_test(float T, float radius, float err, 
     return b;
 }
 
+// The order in which a grid takes the W work items of a list batch of G groups:
+// step i is item spread_item(i, G, W) (none where it is >= W; steps up to
+// spread_steps).  Consecutive steps lie in different groups at about the same
+// place of their lists: what a node's first tiles found (its extreme keys) is
+// known before most of its other tiles start (pass A executed half the
+// instructions).  Items of a group with many nodes cost more, so the CTAs draw
+// the steps from a counter: a fixed stride met the same groups again and again.
+__device__ __forceinline__ int64_t spread_steps(int G, int64_t W) { return G > 0 ? (W + G - 1) / G * G : 0; }
+__device__ __forceinline__ int64_t spread_item(int64_t i, int G, int64_t W)
+{
+    const int64_t rows = (W + G - 1) / G;
+    return i % G * rows + i / G;
+}
+
 }  // namespace kc

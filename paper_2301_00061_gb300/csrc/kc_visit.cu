@@ -492,7 +492,7 @@ visit_a_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
 // ListBatch); the CTA evaluates every node of the group on the staged tile.
 template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads, 3)
-visit_a_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile,
+visit_a_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, unsigned long long *__restrict__ next, int tile,
                     const T *__restrict__ lo, const T *__restrict__ hi, int K, int D, double alpha, Margins mg,
                     typename Key<T>::K *__restrict__ lbkey, typename Key<T>::K *__restrict__ amax,
                     typename Key<T>::K *__restrict__ amin, unsigned *__restrict__ flags, int ndir,
@@ -507,7 +507,14 @@ visit_a_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile,
     // per-warp key slots after the ids (tile is a multiple of 32)
     const WarpKeys dk{ndir, reinterpret_cast<unsigned long long *>(tids + tile) + (size_t)warp * warp_key_words(K, D, ndir),
                       dmax, dmin};
-    for (int64_t w = blockIdx.x; w < L.W; w += gridDim.x) {
+    __shared__ unsigned long long step;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) step = atomicAdd(next, 1ull);
+        __syncthreads();
+        if ((int64_t)step >= spread_steps(L.B, L.W)) break;
+        const int64_t w = spread_item((int64_t)step, L.B, L.W);
+        if (w >= L.W) continue;
         int b;
         int64_t st;
         list_item(L.tile_prefix, L.B, w, tile, &b, &st);
@@ -1012,7 +1019,10 @@ __device__ __forceinline__ void pass_b_node(const uint64_t *tx, int tile, int tn
         const size_t o = ((size_t)b * K + k) * D + a;
         ws->bx[k][a] = in ? pk(lo_in[o], -hi_in[o]) : pk(0.f, -0.f);
         ws->bt[k][a] = in ? pk(blo[o], -bhi[o]) : pk(0.f, -0.f);
-        ws->slim[k][a] = in ? pk(-INF, -INF) : pk(0.f, -0.f);
+        // (from what other warps have found so far)
+        const unsigned gmx = in ? *const_cast<const volatile unsigned *>(&smax[o]) : 0u;
+        const unsigned gmn = in ? *const_cast<const volatile unsigned *>(&smin[o]) : ~0u;
+        ws->slim[k][a] = in ? pk(gmx != 0u ? unord_f32(gmx) : -INF, gmn != ~0u ? -unord_f32(gmn) : -INF) : pk(0.f, -0.f);
         ws->smax[k][a] = 0u;
         ws->smin[k][a] = ~0u;
         ws->jmax[k][a] = 0u;
@@ -1039,7 +1049,8 @@ __device__ __forceinline__ void pass_b_node(const uint64_t *tx, int tile, int tn
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
         c_cnt[k] = 0u;
-        near_d[k] = INF;
+        const unsigned long long c = k < K ? *const_cast<const volatile unsigned long long *>(&cand[(size_t)b * K + k]) : 0ull;
+        near_d[k] = KT::is_none(c) ? INF : KT::vmin(c);
         near_p[k] = ~0u;
     }
     __syncwarp();
@@ -1201,12 +1212,10 @@ __device__ __forceinline__ void pass_b_node(const uint64_t *tx, int tile, int tn
     for (int k = 0; k < KM; ++k)
         if (k < K) {
             const unsigned cn = __reduce_add_sync(ALL, c_cnt[k]);
-            const unsigned long long cd = warp_max_u64(c_cnt[k] ? KT::min_of(near_d[k], near_p[k]) : 0ull);
+            const unsigned long long cd = warp_max_u64(near_p[k] != ~0u ? KT::min_of(near_d[k], near_p[k]) : 0ull);
             const size_t ok_ = (size_t)b * K + k;
-            if (lane == 0 && cn) {
-                atomicAdd(&cnt[ok_], (unsigned long long)cn);
-                atomicMax(&cand[ok_], cd);
-            }
+            if (lane == 0 && cn) atomicAdd(&cnt[ok_], (unsigned long long)cn);
+            if (lane == 0 && cd) atomicMax(&cand[ok_], cd);
         }
     __syncwarp();
     for (int i = lane; i < K * D; i += 32) {
@@ -1266,7 +1275,7 @@ visit_b_kernel(const T *__restrict__ X, int64_t ld, int64_t n, int tile, int spl
 // List mode of pass B (see visit_a_list_kernel).
 template <typename T, int KM, int DM, bool EX>
 __global__ void __launch_bounds__(kThreads, 3)
-visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, int K,
+visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, unsigned long long *__restrict__ next, int tile, int K,
                     int D, int RM, const T *__restrict__ lo_in, const T *__restrict__ hi_in, const T *__restrict__ blo,
                     const T *__restrict__ bhi, const T *__restrict__ repx, const int *__restrict__ nreps,
                     const int *__restrict__ allhave, const float *__restrict__ ball, double alpha, Margins mg,
@@ -1289,7 +1298,14 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, int tile, 
     uint32_t *list = lists + warp * kSub;
     // [warps][KM][RM][words] after the ids (tile is a multiple of 32)
     uint64_t *wrep = reinterpret_cast<uint64_t *>(tids + tile) + (size_t)warp * KM * RM * rep_words<T, DM>();
-    for (int64_t w = blockIdx.x; w < L.W; w += gridDim.x) {
+    __shared__ unsigned long long step;
+    for (;;) {
+        __syncthreads();
+        if (threadIdx.x == 0) step = atomicAdd(next, 1ull);
+        __syncthreads();
+        if ((int64_t)step >= spread_steps(L.B, L.W)) break;
+        const int64_t w = spread_item((int64_t)step, L.B, L.W);
+        if (w >= L.W) continue;
         int b;
         int64_t st;
         list_item(L.tile_prefix, L.B, w, tile, &b, &st);
@@ -1564,7 +1580,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     const size_t o_smin = take(KD * sizeof(OrdT<T>)), o_jmax = take(KD * sizeof(OrdT<T>));
     const size_t o_jmin = take(KD * sizeof(OrdT<T>)), o_cand = take(BK * sizeof(KY));
     const size_t o_dmax = take(BK * ndir * 8), o_dmin = take(BK * ndir * 8);
-    const size_t o_ball = take(sizeof(T) == 4 ? BK * (D + 2) * 4 : 0);
+    const size_t o_ball = take(sizeof(T) == 4 ? BK * (D + 2) * 4 : 0), o_next = take(16);
     KC_TRY(ensure(c, vs->buf, off));
     char *w = static_cast<char *>(vs->buf.p);
     KY *lbkey = reinterpret_cast<KY *>(w + o_lbkey), *amax = reinterpret_cast<KY *>(w + o_amax);
@@ -1577,6 +1593,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
     int *nreps = reinterpret_cast<int *>(w + o_nreps), *have = reinterpret_cast<int *>(w + o_have);
     T *repx = reinterpret_cast<T *>(w + o_repx);
     float *ball = reinterpret_cast<float *>(w + o_ball);
+    unsigned long long *next = reinterpret_cast<unsigned long long *>(w + o_next);   // list mode: work counters
     unsigned long long *cnt = reinterpret_cast<unsigned long long *>(w + o_cnt);
     OrdT<T> *smax = reinterpret_cast<OrdT<T> *>(w + o_smax), *smin = reinterpret_cast<OrdT<T> *>(w + o_smin);
     OrdT<T> *jmax = reinterpret_cast<OrdT<T> *>(w + o_jmax), *jmin = reinterpret_cast<OrdT<T> *>(w + o_jmin);
@@ -1609,7 +1626,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
             int g = 1;
             KC_TRY(grid_of(c, kAL, smem, std::max<int64_t>(1, L->W), &g));
             if (L->W > 0) {
-                kAL<<<g, kThreads, smem, c->stream>>>(static_cast<const T *>(c->X), c->ldx, *L, lt, lo, hi, K_, D,
+                kAL<<<g, kThreads, smem, c->stream>>>(static_cast<const T *>(c->X), c->ldx, *L, next, lt, lo, hi, K_, D,
                                                       alpha, mg, lbkey, amax, amin, flags, ndir, dmax, dmin);
                 KC_TRY(after_launch(c, "tighten pass A (lists)"));
             }
@@ -1661,7 +1678,7 @@ kc_status tighten_impl(kc_ctx *c, const View &v, const void *lo_, const void *hi
             int g = 1;
             KC_TRY(grid_of(c, kBL, smem, std::max<int64_t>(1, L->W), &g));
             if (L->W > 0) {
-                kBL<<<g, kThreads, smem, c->stream>>>(static_cast<const T *>(c->X), c->ldx, *L, lt, K_, D, RM, lo, hi,
+                kBL<<<g, kThreads, smem, c->stream>>>(static_cast<const T *>(c->X), c->ldx, *L, next + 1, lt, K_, D, RM, lo, hi,
                                                       blo, bhi, repx, nreps, have, ball, alpha, mg, seeds, cnt, smax, smin,
                                                       jmax, jmin, cand, flags);
                 KC_TRY(after_launch(c, "tighten pass B (lists)"));
