@@ -1490,7 +1490,7 @@ __global__ void gather_reps_kernel(int M, int K, int D, int R, const int64_t *__
 template <typename F>
 kc_status grid_of(kc_ctx *c, F fn, size_t smem, int64_t work, int *grid)
 {
-    if (smem > 48 * 1024)
+    if (smem > 46 * 1024)   // (48 KiB with a kernel's static shared memory)
         KC_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = 0;
     KC_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem));
