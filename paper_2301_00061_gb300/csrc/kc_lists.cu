@@ -311,6 +311,11 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
     __shared__ int snr[kMaxK];
     __shared__ BallTest sball[kMaxK];              // the representatives' balls against alpha
     __shared__ uint64_t sc0[kMaxK * DMAX / 2];
+    // entries of each warp that the balls leave open: entry | clusters << 8, their
+    // coordinates, and which of them survive
+    __shared__ uint32_t sopen[8][kLT / 8];
+    __shared__ uint64_t sx[8][kLT / 8][DMAX / 2];
+    __shared__ unsigned skept[8][kLT / 256];
     // the node's representatives as packed coordinate pairs [K][RM][DMAX / 2]
     extern __shared__ uint64_t srep[];
     constexpr int H = DMAX / 2;
@@ -375,11 +380,13 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
             for (int a = 0; a < DMAX; ++a)
                 ex[u][a] = (a < D && u * 256 + threadIdx.x < tn) ? X[(size_t)a * ld + eid[u]] : 0.f;
         unsigned kept = 0u;   // bit u: entry u survives
+        int open = 0;         // entries of the warp in sopen
+        const int warp = threadIdx.x >> 5;
+        if (lane < U) skept[warp][lane] = 0u;
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int j = u * 256 + threadIdx.x;
-            const uint32_t id = eid[u];
-            if (j < tn) {
+            unsigned scan = 0u;   // clusters whose representatives must be scanned
+            if (u * 256 + threadIdx.x < tn) {
                 uint64_t px[DMAX];
 #pragma unroll
                 for (int a = 0; a < DMAX; ++a) px[a] = pk(ex[u][a], -ex[u][a]);
@@ -398,13 +405,13 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                     const float2 s2 = upk(acc);
                     as = fminf(as, s2.x + s2.y);
                 }
-                bool redundant = __fadd_ru(__fmul_ru(as, infl), slack) < bth;
+                bool keep = !(__fadd_ru(__fmul_ru(as, infl), slack) < bth);
                 // the upper-bound test only matters for lower-bound redundant samples
-                if (redundant) {
-                    uint64_t pxx[DMAX / 2];
+                if (!keep) {
+                    uint64_t pxx[H];
 #pragma unroll
-                    for (int p = 0; p < DMAX / 2; ++p) pxx[p] = pk(upk(px[2 * p]).x, upk(px[2 * p + 1]).x);
-                    for (int k = 0; k < K && redundant; ++k) {
+                    for (int p = 0; p < H; ++p) pxx[p] = pk(ex[u][2 * p], ex[u][2 * p + 1]);
+                    for (int k = 0; k < K && !keep; ++k) {
                         // outside the box: some lo - x or x - hi is positive
                         float out = 0.f;
 #pragma unroll
@@ -413,41 +420,69 @@ seg_filter_f32(const float *__restrict__ X, int64_t ld, ListBatch L, const float
                             out = max3f(out, t.x, t.y);
                         }
                         if (out > 0.f) continue;
-                        int nr = snr[k];
-                        bool excl = false;
-                        const uint64_t *ck = srep + (size_t)k * RM * (DMAX / 2);
-                        if (nr > 0) {
-                            // the ball decides most samples
-                            const float dc = pair_dist<DMAX / 2>(pxx, sc0 + k * (DMAX / 2));
-                            excl = dc > sball[k].far;
-                            if (dc <= sball[k].near) nr = 0;
-                        }
-                        // chunks of 4 representatives decided by their largest distance
-                        // (a short last chunk repeats the last representative)
-                        for (int r0 = 0; r0 < nr && !excl; r0 += 4) {
-                            float d[4];
+                        // no representatives, or none farther than alpha: it stays
+                        const float dc = snr[k] > 0 ? pair_dist<H>(pxx, sc0 + k * H) : 0.f;
+                        if (snr[k] == 0 || dc <= sball[k].near) keep = true;
+                        else if (!(dc > sball[k].far)) scan |= 1u << k;
+                    }
+                    if (keep) scan = 0u;
+                    if (scan) {
 #pragma unroll
-                            for (int u = 0; u < 4; ++u)
-                                d[u] = pair_dist<DMAX / 2>(pxx, ck + (size_t)(r0 + u < nr ? r0 + u : nr - 1) * (DMAX / 2));
-                            if (fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])) > t_alpha) excl = true;
-                        }
-                        if (!excl) redundant = false;
+                        for (int p = 0; p < H; ++p) sx[warp][u * 32 + lane][p] = pxx[p];
                     }
                 }
-                if (!redundant) kept |= 1u << u;
-                if (!redundant && ckeys) {
-                    // children's bounds over the surviving samples (the closed form
-                    // of Section 3.1 in the same float evaluation as seg_lb_f32);
-                    // their boxes differ from the node's in cluster ks alone
-                    float other = __int_as_float(0x7f800000);
-                    for (int k = 0; k < K; ++k)
-                        if (k != ks) other = fminf(other, box_dist_f32<DMAX>(px, sbox + k * DMAX));
-                    const float v0 = fminf(other, box_dist_f32<DMAX>(px, skid));
-                    const float v1 = fminf(other, box_dist_f32<DMAX>(px, skid + DMAX));
-                    if (v0 >= top0 && (v0 > top0 || id < pos0)) { top0 = v0; pos0 = id; }
-                    if (v1 >= top1 && (v1 > top1 || id < pos1)) { top1 = v1; pos1 = id; }
-                }
+                if (keep) kept |= 1u << u;
             }
+            const unsigned bal = __ballot_sync(0xffffffffu, scan != 0u);
+            if (scan) sopen[warp][open + __popc(bal & ((1u << lane) - 1u))] = (uint32_t)(u * 32 + lane) | (scan << 8);
+            open += __popc(bal);
+        }
+        __syncwarp();
+        // the open entries, one to a lane (with each lane scanning for its own
+        // entry in place, 14 of 32 lanes were active): an entry survives when some
+        // cluster has no representative farther than alpha
+        for (int e = lane; e < open; e += 32) {
+            const uint32_t w = sopen[warp][e];
+            const int at = (int)(w & 0xFFu);
+            uint64_t pxx[H];
+#pragma unroll
+            for (int p = 0; p < H; ++p) pxx[p] = sx[warp][at][p];
+            bool keep = false;
+            for (unsigned m = w >> 8; m && !keep; m &= m - 1) {
+                const int k = __ffs(m) - 1, nr = snr[k];
+                const uint64_t *ck = srep + (size_t)k * RM * H;
+                // chunks of 4 representatives decided by their largest distance
+                // (a short last chunk repeats the last representative)
+                bool excl = false;
+                for (int r0 = 0; r0 < nr && !excl; r0 += 4) {
+                    float d[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) d[u] = pair_dist<H>(pxx, ck + (size_t)(r0 + u < nr ? r0 + u : nr - 1) * H);
+                    excl = fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3])) > t_alpha;
+                }
+                keep = !excl;
+            }
+            if (keep) atomicOr(&skept[warp][at >> 5], 1u << (at & 31));
+        }
+        __syncwarp();
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (skept[warp][u] >> lane & 1u) kept |= 1u << u;
+            if (!ckeys || !(kept >> u & 1u)) continue;
+            // children's bounds over the surviving samples (the closed form of
+            // Section 3.1 in the same float evaluation as seg_lb_f32); their boxes
+            // differ from the node's in cluster ks alone
+            const uint32_t id = eid[u];
+            uint64_t px[DMAX];
+#pragma unroll
+            for (int a = 0; a < DMAX; ++a) px[a] = pk(ex[u][a], -ex[u][a]);
+            float other = __int_as_float(0x7f800000);
+            for (int k = 0; k < K; ++k)
+                if (k != ks) other = fminf(other, box_dist_f32<DMAX>(px, sbox + k * DMAX));
+            const float v0 = fminf(other, box_dist_f32<DMAX>(px, skid));
+            const float v1 = fminf(other, box_dist_f32<DMAX>(px, skid + DMAX));
+            if (v0 >= top0 && (v0 > top0 || id < pos0)) { top0 = v0; pos0 = id; }
+            if (v1 >= top1 && (v1 > top1 || id < pos1)) { top1 = v1; pos1 = id; }
         }
         // one reservation per warp (no block barrier): lane 0 claims the warp's
         // surviving entries, the others write behind it, each 32 entries as one
@@ -655,7 +690,7 @@ kc_status launch_seg_filter(kc_ctx *c, const ListBatch &L, const void *lo, const
     const int dm = c->D <= 2 ? 2 : c->D <= 4 ? 4 : 8;   // attributes the kernels are compiled for
     const size_t srep = nreps ? (size_t)c->K * RM * (dm / 2) * 8 : 0;
     const auto fn = dm == 2 ? seg_filter_f32<2> : dm == 4 ? seg_filter_f32<4> : seg_filter_f32<8>;
-    if (srep > 48 * 1024)
+    if (srep > 8 * 1024)   // (48 KiB with the static 38 KiB at D = 8)
         KC_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)srep));
     fn<<<gr, 256, srep, c->stream>>>(static_cast<const float *>(c->X), c->ldx, L,
                                                  static_cast<const float *>(lo), static_cast<const float *>(hi), c->K,
