@@ -226,7 +226,7 @@ kc_status kc_fft_multi(kc_ctx *ctx, const int64_t *starts, int32_t S, int64_t *c
  *   lb_out, lb_raw_out, argmax_out  as in kc_lower_bounds (the argmax is a
  *              sample index, smallest on ties).
  *   kernel_ms_out  host float or NULL: the device time of the bound launch
- *              (key reset, the gather-and-bound kernel and its finalize),
+ *              (the gather-and-bound kernels and their finalize),
  *              measured with CUDA events on the context's stream; the call
  *              then waits for it.
  * Float data with D <= 8 only (KC_EINVAL otherwise).
