@@ -160,6 +160,25 @@ __device__ __forceinline__ void list_item(const int64_t *__restrict__ tile_prefi
     *start_out = (int64_t)(w - tile_prefix[lo]) * tile;
 }
 
+// Certified bound from the value of an evaluation in T: deflated by its error
+// bound, rounded down.  Data so far apart that squares leave T's range evaluate to
+// infinity; with unbounded exponents they would evaluate to no less than T's
+// largest finite value, so that value takes its place.
+template <typename T>
+__device__ __forceinline__ double certified_lb(double raw, double defl, double slack)
+{
+    const double top = sizeof(T) == 4 ? 3.4028234663852886e38 : 1.7976931348623157e308;
+    return fmax(0.0, __dsub_rd(__dmul_rd(fmin(raw, top), defl), slack));
+}
+
+// A float screen's largest value m proves that the exact maximum is >= cut (gam:
+// the relative error bound; an infinite cut is never reached, and an overflowed m
+// proves no more than the largest finite value).
+__device__ __forceinline__ bool screen_proves(float m, double gam, double cut)
+{
+    return __ddiv_rd(fmin((double)m, 3.4028234663852886e38), 1.0 + gam) >= cut;
+}
+
 // ---- 128-bit keys (ordered value, ~position): double values with positions
 
 __device__ __forceinline__ ulonglong2 cas128(ulonglong2 *p, ulonglong2 c, ulonglong2 v)

@@ -80,7 +80,7 @@ struct HitArgs {
 // Float data (double data have no cut: gam < 0): the screen proves value >= cut.
 __device__ __forceinline__ bool node_cut(float m, double gam, double cut)
 {
-    return gam >= 0.0 && __ddiv_rd((double)m, 1.0 + gam) >= cut;
+    return gam >= 0.0 && screen_proves(m, gam, cut);
 }
 
 // A CTA looks over 256 (node, tile) entries at a time: does the tile hold a
@@ -230,7 +230,7 @@ __global__ void exact_finalize_kernel(unsigned long long *__restrict__ keys, ulo
     const bool none = k.x == 0ull;
     const double v = none ? 0.0 : unord_f64(k.x);
     if (val) val[b] = v;
-    if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(v, defl), slack));
+    if (lb) lb[b] = certified_lb<double>(v, defl, slack);   // (only double data ask for it)
     if (arg) {
         const int64_t p = none ? -1 : (int64_t)(0xFFFFFFFFull - k.y);
         arg[b] = (p < 0 || !ids) ? p : (int64_t)ids[p];

@@ -132,7 +132,7 @@ __global__ void lb_finalize_f32(unsigned long long *__restrict__ keys, int B, co
     keys[b] = 0ull;
     const double raw = m ? (double)key_val(m) : 0.0;
     if (lb_raw) lb_raw[b] = raw;
-    if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(raw, defl), slack));
+    if (lb) lb[b] = certified_lb<float>(raw, defl, slack);
     if (arg) {
         const int64_t pos = m ? (int64_t)key_pos(m) : -1;
         arg[b] = (pos < 0 || !ids) ? pos : (int64_t)ids[pos];
@@ -366,7 +366,7 @@ kc_status launch_lower_bounds_refine(kc_ctx *c, const View &v, const void *lo, c
     const double gam = gamma_n(f32_roundings(D), kU32) + 2 * gamma_n(f64_roundings(D), kU64) + 1e-15;
     std::vector<float> thr(B);
     for (int b = 0; b < B; ++b) {
-        double t = raw_host[b] / (1.0 + gam) * (1.0 - gam) * (1.0 - 1e-6) - 1e-37;
+        double t = std::min(raw_host[b], 3.4028234663852886e38) / (1.0 + gam) * (1.0 - gam) * (1.0 - 1e-6) - 1e-37;
         float f = (float)t;
         if ((double)f > t) f = nextafterf(f, -1.f);
         thr[b] = t > 0 ? f : -1.f;

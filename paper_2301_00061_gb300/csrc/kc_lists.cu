@@ -534,7 +534,7 @@ __global__ void keys_finalize(const unsigned long long *__restrict__ keys, int B
     const unsigned long long m = keys[b];
     const double r = m ? (double)key_val(m) : 0.0;
     if (raw) raw[b] = r;
-    if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(r, defl), slack));
+    if (lb) lb[b] = certified_lb<float>(r, defl, slack);
     if (arg) arg[b] = m ? (int64_t)key_pos(m) : -1;
 }
 
@@ -553,9 +553,9 @@ __global__ void screen_threshold(const unsigned long long *__restrict__ keys, in
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= B) return;
-    const double raw = keys[b] ? (double)key_val(keys[b]) : 0.0;
-    const double low = __ddiv_rd(raw, 1.0 + gam);
-    if (low >= alpha_cut) { thr[b] = __int_as_float(0x7f800000); return; }
+    const float raw = keys[b] ? key_val(keys[b]) : 0.f;
+    const double low = __ddiv_rd((double)fminf(raw, 3.4028235e38f), 1.0 + gam);
+    if (screen_proves(raw, gam, alpha_cut)) { thr[b] = __int_as_float(0x7f800000); return; }
     const double t = __dmul_rd(__dmul_rd(low, 1.0 - gam), 1.0 - 1e-6) - 1e-37;
     thr[b] = t > 0.0 ? __double2float_rd(t) : -1.0f;
 }
@@ -603,7 +603,7 @@ kc_status launch_seg_refine(kc_ctx *c, const ListBatch &L, const void *lo, const
     const double gam = gamma_n(f32_roundings(c->D), kU32) + 2 * gamma_n(f64_roundings(c->D), kU64) + 1e-15;
     std::vector<float> thr(B);
     for (int b = 0; b < B; ++b) {
-        const double t = raw_host[b] / (1.0 + gam) * (1.0 - gam) * (1.0 - 1e-6) - 1e-37;
+        const double t = std::min(raw_host[b], 3.4028234663852886e38) / (1.0 + gam) * (1.0 - gam) * (1.0 - 1e-6) - 1e-37;
         float f = (float)t;
         if ((double)f > t) f = nextafterf(f, -1.f);
         thr[b] = t > 0 ? f : -1.f;

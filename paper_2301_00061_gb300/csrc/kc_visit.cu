@@ -594,7 +594,7 @@ finalize_a_kernel(int B, int K, int D, const T *__restrict__ lo, const T *__rest
         const bool none = KT::is_none(key);
         const double raw = none ? 0.0 : (double)KT::vmax(key);
         if (lb_raw) lb_raw[b] = raw;
-        if (lb) lb[b] = fmax(0.0, __dsub_rd(__dmul_rd(raw, f.defl), f.slack));
+        if (lb) lb[b] = certified_lb<T>(raw, f.defl, f.slack);
         if (lbarg) {
             const int64_t p = none ? -1 : (int64_t)KT::pos(key);
             lbarg[b] = (p < 0 || !f.ids) ? p : (int64_t)f.ids[p];
