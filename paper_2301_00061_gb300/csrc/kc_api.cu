@@ -93,10 +93,12 @@ bool is_device_ptr(const void *p)
 }
 
 // The device address of the `bytes` at p when they are all within one allocation of
-// pinned host memory that kernels can read, else NULL (pageable memory, a range that
-// is only partly registered).
-static const void *pinned_device_ptr(const void *p, size_t bytes)
+// pinned host memory that kernels can read as elements of esize bytes, else NULL
+// (pageable memory, a range that is only partly registered, an address that is no
+// multiple of esize).
+static const void *pinned_device_ptr(const void *p, size_t bytes, size_t esize)
 {
+    if (reinterpret_cast<uintptr_t>(p) % esize != 0) return nullptr;
     cudaPointerAttributes a;
     void *f = nullptr;
     cudaDriverEntryPointQueryResult found;
@@ -209,7 +211,7 @@ kc_status kc_create(const void *X, int64_t N, int32_t D, int32_t K, kc_dtype dt,
             e = cudaMemset2DAsync(static_cast<char *>(c->X) + N * c->esize, c->ldx * c->esize, 0,
                                   (c->ldx - N) * c->esize, D, c->stream);
         if (e != cudaSuccess) st = set_err(c, KC_ECUDA, "kc_create: upload failed: %s", cudaGetErrorString(e));
-    } else if (const void *mapped = pinned_device_ptr(X, src_bytes)) {
+    } else if (const void *mapped = pinned_device_ptr(X, src_bytes, c->esize)) {
         // pinned host rows: the transpose reads them where they are, one pass at
         // the link's rate (a copy and a transpose per chunk take turns: 2.93 ms
         // for a dataset of 320 MB with its root box and first incumbent, so 2.49);
