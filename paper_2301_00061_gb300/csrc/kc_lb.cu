@@ -463,8 +463,8 @@ namespace {
 constexpr int kNoAllocMaxNodes = 4096;    // nodes per call
 constexpr int kNoAllocMaxDevices = 64;
 
-// The best key of each node of a call, zero between calls: 32 KiB, held by every
-// GPU that loads the library until the process exits.
+// The best key of each node of a call: 32 KiB, held by every GPU that loads the
+// library until the process exits.
 static __device__ __align__(256) unsigned long long g_noalloc_keys[kNoAllocMaxNodes];
 
 std::atomic<void *> g_noalloc_ptr[kNoAllocMaxDevices];
@@ -525,6 +525,9 @@ extern "C" kc_status kc_lower_bounds_noalloc(const float *X, int64_t N, int64_t 
     A.K = K;
     A.D = D;
     A.keys = static_cast<unsigned long long *>(scratch);
+    // the keys start from zero whatever an earlier call left (one whose last launch
+    // failed): this array has no context that would end with the error
+    if (cudaMemsetAsync(scratch, 0, (size_t)B * 8, st) != cudaSuccess) return KC_ECUDA;
     if (N > 0 && launch_max_f32(A, sms, (size_t)optin, 0, 0, st) != cudaSuccess) return KC_ECUDA;
     lb_finalize_f32<<<(B + 127) / 128, 128, 0, st>>>(A.keys, B, nullptr, defl, slack, lb_out, lb_raw_out, argmax_out);
     if (cudaGetLastError() != cudaSuccess) return KC_ECUDA;
