@@ -52,18 +52,31 @@ __device__ __forceinline__ void warp_raise128(ulonglong2 *p, double v, uint32_t 
     if ((threadIdx.x & 31) == 0 && v >= 0.0) raise128(p, v, pos);
 }
 
-// Exact value of sample s: min over clusters, attribute order.
+// Exact value of sample s: min over clusters, attribute order.  Few samples come here,
+// so the loads of four attributes are in flight together.
 template <typename T>
 __device__ double exact_value(const T *__restrict__ X, int64_t ld, int64_t s, const T *__restrict__ lo,
                               const T *__restrict__ hi, int K, int D)
 {
+    constexpr int AH = 4;
     double e = __longlong_as_double(0x7ff0000000000000ll);
     for (int k = 0; k < K; ++k) {
         double acc = 0.0;
-        for (int a = 0; a < D; ++a) {
-            const double x = (double)X[(size_t)a * ld + s];
-            const double d = __dsub_rn(x, mid3d((double)lo[k * D + a], x, (double)hi[k * D + a]));
-            acc = __dadd_rn(acc, __dmul_rn(d, d));
+        for (int a0 = 0; a0 < D; a0 += AH) {
+            T x[AH], l[AH], h[AH];
+#pragma unroll
+            for (int i = 0; i < AH; ++i) {
+                const int a = a0 + i < D ? a0 + i : D - 1;
+                x[i] = X[(size_t)a * ld + s];
+                l[i] = lo[k * D + a];
+                h[i] = hi[k * D + a];
+            }
+#pragma unroll
+            for (int i = 0; i < AH; ++i) {
+                if (a0 + i >= D) break;
+                const double d = __dsub_rn((double)x[i], mid3d((double)l[i], (double)x[i], (double)h[i]));
+                acc = __dadd_rn(acc, __dmul_rn(d, d));
+            }
         }
         if (acc < e) e = acc;
     }
@@ -73,6 +86,7 @@ __device__ double exact_value(const T *__restrict__ X, int64_t ld, int64_t s, co
 struct HitArgs {
     PruneArgs A;
     int T;                 // samples of a tmax row
+    int run;               // consecutive (node, tile) entries that a CTA looks over, a power of two <= 8
     double gam, cut;       // nodes whose float value proves an exact value >= cut are skipped
     ulonglong2 *best;      // [B] exact maxima, zero before the screen
 };
@@ -83,98 +97,173 @@ __device__ __forceinline__ bool node_cut(float m, double gam, double cut)
     return gam >= 0.0 && screen_proves(m, gam, cut);
 }
 
+constexpr int kHitCtas = 4;      // CTAs per SM: the grid is resident at once
+constexpr int kHitTile = 2048;   // most samples of a tmax row (of any kernel that fills tmax)
+
 // A CTA looks over 256 (node, tile) entries at a time: does the tile hold a
 // sample that may attain the node's maximum?  All its threads then go through
-// each such tile, four samples a thread at a time: in float, and those that
-// reach the floor in double.  (The tiles of one sample far from everything are
-// hits of every node; entries are ordered by node, so they meet different CTAs:
-// with one warp to a hit and 32 nodes to a warp this took 375 us of 450.)
+// each such tile in float, four samples a thread at a time, and list those that
+// reach the floor; the listed ones are evaluated in double, one to a thread.
+// Entries are dealt out in runs of at most eight, because the tiles of one sample
+// far from everything are hits of every node, and all tiles of a node are hits
+// where many samples attain its maximum: with 256 consecutive entries to a CTA, 16
+// nodes of bound 0 over 1e5 samples (784 entries, all hits) kept four CTAs
+// busy for 4.2 ms (now 0.05 ms a call; 64 double nodes of bound 0 over 1e6 samples 12.3,
+// now 1.1 ms; 64 float center sets whose maximum 1e6 samples attain often 3.2, now 1.0).
+//
+// A node whose largest float value is within the margin of 0 keeps every sample
+// (floor 0), but a sample inside a box has the exact value 0: it cannot beat the
+// others, and among equal zeros the first sample wins, so that one alone is evaluated
+// with those outside every box.  Being inside is decided on the ordered bits of the
+// values (double comparisons would run at the rate of the double arithmetic that
+// this saves).
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kHitCtas)
 exact_hits_kernel(const HitArgs H)
 {
     constexpr bool F64 = sizeof(T) == 8;
-    constexpr int U = 4;
+    // float data: a hit is bound by load latency, so four attributes are in flight (16
+    // sets at N = 2e5, D = 29: 160 us a call, one attribute at a time 184); double
+    // data: by the double arithmetic of the conversions
+    constexpr int U = 4, AH = F64 ? 1 : 4;
+    constexpr unsigned ALL = 0xffffffffu;
+    using Ord = typename std::conditional<F64, uint64_t, uint32_t>::type;
     __shared__ int64_t hits[256];
     __shared__ float floors[256];
-    __shared__ int count;
+    __shared__ uint16_t list[kHitTile];   // samples of a hit that need the double value
+    __shared__ int count, listed;
+    // its node's boxes: float values, or (floor 0) ordered bits in the type's size
+    extern __shared__ __align__(16) unsigned char boxes[];
     const PruneArgs &A = H.A;
-    const int tid = threadIdx.x, K = A.K, D = A.D;
+    const int tid = threadIdx.x, lane = tid & 31, K = A.K, D = A.D, KD = K * D, run = H.run;
+    float *flo = reinterpret_cast<float *>(boxes), *fhi = flo + KD;
+    Ord *olo = reinterpret_cast<Ord *>(boxes), *ohi = olo + KD;
+    auto ord = [](T v) {
+        if constexpr (F64) return ord_f64(v);
+        else return ord_f32(v);
+    };
     const T *X = static_cast<const T *>(A.X);
     const int64_t total = A.rows * A.B;
-    for (int64_t i0 = (int64_t)blockIdx.x * 256; i0 < total; i0 += (int64_t)gridDim.x * 256) {
+    for (int64_t i0 = (int64_t)blockIdx.x * run; i0 < total; i0 += (int64_t)gridDim.x * 256) {
         if (tid == 0) count = 0;
         __syncthreads();
-        const int64_t i = i0 + tid;
+        const int64_t i = i0 + (int64_t)(tid / run) * gridDim.x * run + tid % run;
         if (i < total) {
             const float m = key_val(A.keys[i / A.rows]), t = screen_floor(m, A.c1, A.eps);
             if (A.tmax[i] >= t && !node_cut(m, H.gam, H.cut)) {
                 const int o = atomicAdd(&count, 1);
                 hits[o] = i;
-                floors[o] = t;
+                floors[o] = t > 0.f ? t : -1.f;   // -1: every sample outside the boxes
             }
         }
         __syncthreads();
-        for (int o = 0; o < count; ++o) {
+        const int found = count;
+        for (int o = 0; o < found; ++o) {
             const int64_t q = hits[o];
             const float tq = floors[o];
             const int b = (int)(q / A.rows);
             const int64_t s0 = q % A.rows * H.T, s1 = s0 + H.T < A.n ? s0 + H.T : A.n;
-            const T *lo = static_cast<const T *>(A.lo) + (size_t)b * K * D;
-            const T *hi = static_cast<const T *>(A.hi) + (size_t)b * K * D;
-            double v = -1.0;
-            uint32_t pos = 0xFFFFFFFFu;
-            for (int64_t s = s0 + tid; s < s1; s += 256 * U) {
-                float near[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) near[u] = __int_as_float(0x7f800000);
-                for (int k = 0; k < K; ++k) {
-                    // two chains over even and odd attributes, as the screen's
-                    float acc[2][U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) acc[0][u] = acc[1][u] = 0.f;
-                    for (int a = 0; a < D; ++a) {
-                        float l, h, c[U];
-                        if constexpr (F64) {
-                            const double f = A.off[a];
-                            l = __double2float_ru(__dsub_ru(lo[k * D + a], f));
-                            h = __double2float_rd(__dsub_rd(hi[k * D + a], f));
+            const T *lo = static_cast<const T *>(A.lo) + (size_t)b * KD;
+            const T *hi = static_cast<const T *>(A.hi) + (size_t)b * KD;
+            if (tid == 0) listed = 0;
+            for (int e = tid; e < KD; e += 256) {
+                if (tq < 0.f) {
+                    olo[e] = ord(lo[e]);
+                    ohi[e] = ord(hi[e]);
+                } else if constexpr (F64) {
+                    const double f = A.off[e % D];
+                    flo[e] = __double2float_ru(__dsub_ru(lo[e], f));
+                    fhi[e] = __double2float_rd(__dsub_rd(hi[e], f));
+                } else {
+                    flo[e] = lo[e];
+                    fhi[e] = hi[e];
+                }
+            }
+            __syncthreads();
+            for (int64_t s = s0 + tid; s - lane < s1; s += 256 * U) {   // (whole warps stay together)
+                const int64_t left = s1 - (s - lane);
+                const int nu = left > 256 * (U - 1) ? U : (int)((left + 255) / 256);   // of the U samples
+                unsigned may = 0u;   // bit u: sample s + 256 u needs the double value
+                if (tq < 0.f) {
+                    unsigned in = 0u;
+                    for (int k = 0; k < K && !__all_sync(ALL, in == (1u << nu) - 1u); ++k) {
+                        unsigned inside = (1u << nu) - 1u;
+                        for (int a = 0; a < D; ++a) {
+                            const Ord l = olo[k * D + a], h = ohi[k * D + a];
 #pragma unroll
                             for (int u = 0; u < U; ++u) {
+                                if (u >= nu) break;
                                 const int64_t w = s + u * 256;
-                                c[u] = __double2float_rn(X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)] - f);
-                            }
-                        } else {
-                            l = lo[k * D + a];
-                            h = hi[k * D + a];
-#pragma unroll
-                            for (int u = 0; u < U; ++u) {
-                                const int64_t w = s + u * 256;
-                                c[u] = X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)];
+                                const Ord x = ord(X[(size_t)a * A.ld + (w < s1 ? w : s1 - 1)]);
+                                if (x < l || x > h) inside &= ~(1u << u);
                             }
                         }
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            const float m = max3f(l - c[u], c[u] - h, 0.f);
-                            if (a & 1) acc[1][u] = fmaf(m, m, acc[1][u]);
-                            else acc[0][u] = fmaf(m, m, acc[0][u]);
-                        }
+                        in |= inside;
                     }
+                    may = ~in;
+                    if (s == 0) may |= 1u;
+                } else {
+                    unsigned reach = (1u << nu) - 1u;   // no distance below the floor so far
+                    for (int k = 0; k < K && __any_sync(ALL, reach); ++k) {
+                        // two chains over even and odd attributes, as the screen's
+                        float acc[2][U];
 #pragma unroll
-                    for (int u = 0; u < U; ++u) near[u] = fminf(near[u], acc[0][u] + acc[1][u]);
+                        for (int u = 0; u < U; ++u) acc[0][u] = acc[1][u] = 0.f;
+                        for (int a0 = 0; a0 < D; a0 += AH) {
+                            T x[AH][U];
+#pragma unroll
+                            for (int i = 0; i < AH; ++i)
+#pragma unroll
+                                for (int u = 0; u < U; ++u) {
+                                    if (F64 && u >= nu) break;
+                                    const int64_t w = s + u * 256;
+                                    x[i][u] = X[(size_t)(a0 + i < D ? a0 + i : D - 1) * A.ld + (w < s1 ? w : s1 - 1)];
+                                }
+#pragma unroll
+                            for (int i = 0; i < AH; ++i) {
+                                if (a0 + i >= D) break;
+                                const float l = flo[k * D + a0 + i], h = fhi[k * D + a0 + i];
+#pragma unroll
+                                for (int u = 0; u < U; ++u) {
+                                    if (F64 && u >= nu) break;
+                                    float c;
+                                    if constexpr (F64) c = __double2float_rn(x[i][u] - A.off[a0 + i]);
+                                    else c = x[i][u];
+                                    const float m = max3f(l - c, c - h, 0.f);
+                                    if ((a0 + i) & 1) acc[1][u] = fmaf(m, m, acc[1][u]);
+                                    else acc[0][u] = fmaf(m, m, acc[0][u]);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (!(acc[0][u] + acc[1][u] >= tq)) reach &= ~(1u << u);
+                    }
+                    may = reach;
                 }
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int64_t w = s + u * 256;
-                    if (w < s1 && near[u] >= tq) {
-                        const double e = exact_value<T>(X, A.ld, w, lo, hi, K, D);
-                        if (e > v) { v = e; pos = (uint32_t)w; }   // (w increases)
-                    }
+                    const bool on = w < s1 && (may >> u & 1u);
+                    const unsigned bal = __ballot_sync(ALL, on);
+                    if (!bal) continue;
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(&listed, __popc(bal));
+                    at = __shfl_sync(ALL, at, 0) + __popc(bal & ((1u << lane) - 1u));
+                    if (on) list[at] = (uint16_t)(w - s0);
                 }
             }
-            if (__any_sync(0xffffffffu, v >= 0.0)) warp_raise128(&H.best[b], v, pos);
+            __syncthreads();
+            double v = -1.0;
+            uint32_t pos = 0xFFFFFFFFu;
+            for (int j = tid; j < listed; j += 256) {
+                const int64_t w = s0 + list[j];
+                const double e = exact_value<T>(X, A.ld, w, lo, hi, K, D);
+                if (e > v || (e == v && (uint32_t)w < pos)) { v = e; pos = (uint32_t)w; }
+            }
+            if (__any_sync(ALL, v >= 0.0)) warp_raise128(&H.best[b], v, pos);
+            __syncthreads();
         }
-        __syncthreads();
     }
 }
 
@@ -325,9 +414,16 @@ kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *
             H.gam = f64 ? -1.0 : gam;
             H.cut = cut;
             H.best = best;
-            const int grid = (int)std::min<int64_t>((rows * B + 255) / 256, (int64_t)c->num_sms * 8);
-            if (f64) exact_hits_kernel<double><<<grid, 256, 0, c->stream>>>(H);
-            else exact_hits_kernel<float><<<grid, 256, 0, c->stream>>>(H);
+            if (H.T > kHitTile) return set_err(c, KC_EINTERNAL, "screen tile of %d samples", H.T);
+            // short runs where there are few entries, so that they reach every SM; runs of
+            // eight (one sector of tmax) where there are enough
+            const int64_t most = (int64_t)c->num_sms * kHitCtas;
+            H.run = 8;
+            while (H.run > 1 && rows * B / H.run < 2 * most) H.run /= 2;
+            const int grid = (int)std::min<int64_t>((rows * B + H.run - 1) / H.run, most);
+            const auto fn = f64 ? exact_hits_kernel<double> : exact_hits_kernel<float>;
+            const size_t smem = (size_t)2 * K * D * es;   // (at most 32 KiB, and 8 static)
+            fn<<<grid, 256, smem, c->stream>>>(H);
             KC_TRY(after_launch(c, "exact maximum of the screened samples"));
         }
     }
