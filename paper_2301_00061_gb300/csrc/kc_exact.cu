@@ -402,7 +402,7 @@ kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *
             A.cut = cf < 3e38 ? (float)cf : __builtin_huge_valf();
             const PruneEntry *e = f64 ? prune_pick(prune_table<true, true>(), D, v.n, c->num_sms, 0)
                                       : prune_pick(prune_table<false, true>(), D, v.n, c->num_sms, 0);
-            const bool stream = !f64 && use_stream_f32(B, K, D);
+            const bool stream = !f64 && use_stream_f32(B, K, D, v.n);
             H.T = stream ? kStreamTile : e->T;
             const int64_t rows = (v.n + H.T - 1) / H.T;
             KC_TRY(ensure(c, c->tmax, (size_t)rows * B * 4));

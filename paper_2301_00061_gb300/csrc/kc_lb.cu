@@ -120,13 +120,19 @@ lb_refine_f32(const float *__restrict__ X, int64_t ld, int64_t n, const float *_
     }
 }
 
+constexpr int kMaxLeft = 256;   // flags of the pruning kernel's CTAs (an SM each) and one for all
+
 // Keys (value bits, ~position) -> certified bound, value and sample per node.
-// The keys go back to zero, as the next launch wants them.
-__global__ void lb_finalize_f32(unsigned long long *__restrict__ keys, int B, const uint32_t *__restrict__ ids,
+// The keys (and the pruning kernel's flags) go back to zero, as the next launch
+// wants them.
+__global__ void lb_finalize_f32(unsigned long long *__restrict__ keys, int *__restrict__ left, int B,
+                                const uint32_t *__restrict__ ids,
                                 double defl, double slack, double *__restrict__ lb, double *__restrict__ lb_raw,
                                 int64_t *__restrict__ arg)
 {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    if (left && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < kMaxLeft; i += blockDim.x) left[i] = 0;
     if (b >= B) return;
     const unsigned long long m = keys[b];
     keys[b] = 0ull;
@@ -194,15 +200,39 @@ gather_rows_kernel(const float *__restrict__ X, int64_t ld, int D, const uint32_
 
 // ---------------------------------------------------------------- dispatch
 
-// Launches the float maxima of A.B nodes into A.keys (zeroed by the caller) on
-// `stream`; st (samples per thread: 4 or 2, where both exist) and chunk (nodes
+// Launches the float maxima of A.B nodes into A.keys (zeroed by the caller, as
+// A.left) on `stream`: full evaluation, or the pruning kernel and full evaluation
+// of what it leaves.  st (samples per thread: 4 or 2, where both exist) and chunk (nodes
 // per CTA) of 0 are chosen here.
-cudaError_t launch_max_f32(PruneArgs A, int sms, size_t smem_cap, int st, int chunk, cudaStream_t stream)
+cudaError_t launch_max_f32(PruneArgs A, int sms, size_t smem_cap, int st, int chunk, cudaStream_t stream,
+                           int64_t *launches = nullptr)
 {
+    if (launches) ++*launches;
     A.vec = (uintptr_t)A.X % 16 == 0 && A.ld % 4 == 0;
-    if (use_stream_f32(A.B, A.K, A.D)) return launch_stream_f32(A, sms, stream);
-    return prune_run(prune_pick(prune_table<false, false>(), A.D, A.n, sms, st), A, false, sms, smem_cap, chunk, stream);
+    int *const left = A.left;
+    A.left = nullptr;
+    if (use_stream_f32(A.B, A.K, A.D, A.n)) return launch_stream_f32(A, sms, stream);
+    const PruneEntry *e = prune_pick(prune_table<false, false>(), A.D, A.n, sms, st);
+    A.T = e->T;
+    A.gx = (int)std::min<int64_t>((A.n + e->T - 1) / e->T, sms);
+    if (may_leave(A.B, A.D, (A.n + e->T - 1) / e->T <= sms) && A.gx < kMaxLeft) A.left = left;
+    const cudaError_t r = prune_run(e, A, false, sms, smem_cap, chunk, stream);
+    if (r != cudaSuccess || !A.left) return r;
+    if (launches) ++*launches;
+    return launch_stream_f32(A, sms, stream);
 }
+
+// The context's flags and keys of B nodes, all zero between calls.
+kc_status ensure_keys(kc_ctx *c, int B)
+{
+    const size_t need = kMaxLeft * 4 + (size_t)B * 8;
+    if (c->keys.bytes >= need) return KC_OK;
+    KC_TRY(ensure(c, c->keys, need));
+    KC_CUDA(c, cudaMemsetAsync(c->keys.p, 0, c->keys.bytes, c->stream));
+    return KC_OK;
+}
+int *flags_of(const kc_ctx *c) { return static_cast<int *>(c->keys.p); }
+unsigned long long *keys_of(const kc_ctx *c) { return reinterpret_cast<unsigned long long *>(flags_of(c) + kMaxLeft); }
 
 template <typename F>
 kc_status prep_kernel(kc_ctx *c, F fn, size_t smem, int *grid, int64_t tiles)
@@ -226,10 +256,17 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
     const auto bytes = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32, tm).end; };
     int per = A.B;
     if (chunk > 0 && chunk < per) per = chunk;
-    if (tiles < sms) {
-        // few tiles: spread the nodes over the SMs as well, whole groups to a CTA
-        const int64_t want = std::max<int64_t>(1, sms / tiles);
-        per = (int)std::min<int64_t>(per, ((A.B + want - 1) / want + kPG - 1) / kPG * kPG);
+    if (tiles < 4 * (int64_t)sms) {
+        // few tiles: node ranges (whole groups) so that the last round of CTAs leaves
+        // little idle; a range repeats the sort of its tile, about 16 nodes' worth (1e5
+        // samples, D = 8, K = 5, 256 nodes: 280 us in one range, 212 in three)
+        int64_t best = INT64_MAX;
+        const int most = per;
+        for (int64_t r = 1; r <= 4 * (int64_t)sms / tiles + 1 && r <= (A.B + kPG - 1) / kPG; ++r) {
+            const int64_t nodes = std::min<int64_t>(most, ((A.B + r - 1) / r + kPG - 1) / kPG * kPG);
+            const int64_t ranges = (A.B + nodes - 1) / nodes, cost = (tiles * ranges + sms - 1) / sms * (16 + nodes);
+            if (cost < best) { best = cost; per = (int)nodes; }
+        }
     }
     while (per > 1 && bytes(per) > smem_cap) per = per > 2 * kPG ? (per - 1) / kPG * kPG : per - 1;
     A.per = per;
@@ -239,9 +276,17 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
         const cudaError_t r = cudaFuncSetAttribute(e->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (r != cudaSuccess) return r;
     }
+    // 512 threads at 128 registers fill an SM; of the smaller CTAs several fit (D = 128,
+    // 3e5 samples, 8 nodes: 480 us with one, 286 with two)
+    int per_sm = 1;
+    if (e->NT < 512) {
+        const cudaError_t r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, e->fn, e->NT, smem);
+        if (r != cudaSuccess) return r;
+        per_sm = std::max(1, per_sm);
+    }
     // at most 65535 node ranges to a launch
     const int B = A.B, step = (int)std::min<int64_t>((int64_t)per * 65535, B);
-    const size_t box = (size_t)A.K * A.D * (A.off ? 8 : 4);
+    const size_t box = (size_t)A.K * A.D * (tm && A.off ? 8 : 4);
     if (tm && step < B) return cudaErrorInvalidConfiguration;   // (screens come in batches far smaller)
     for (int b0 = 0; b0 < B; b0 += step) {
         PruneArgs C = A;
@@ -249,7 +294,7 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
         C.lo = static_cast<const char *>(A.lo) + b0 * box;
         C.hi = static_cast<const char *>(A.hi) + b0 * box;
         C.keys = A.keys + b0;
-        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, sms)), (unsigned)((C.B + per - 1) / per));
+        const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms * per_sm)), (unsigned)((C.B + per - 1) / per));
         e->fn<<<grid, e->NT, smem, stream>>>(C);
         const cudaError_t r = cudaGetLastError();
         if (r != cudaSuccess) return r;
@@ -271,10 +316,7 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
     const double defl = deflate_factor(c->dt, D), slack = underflow_slack(c->dt, D);
     const size_t smem_cap = c->smem_optin > 0 ? c->smem_optin : 48 * 1024;
     if (c->dt == KC_F32) {
-        if (c->keys.bytes < (size_t)B * 8) {
-            KC_TRY(ensure(c, c->keys, (size_t)B * 8));
-            KC_CUDA(c, cudaMemsetAsync(c->keys.p, 0, c->keys.bytes, c->stream));
-        }
+        KC_TRY(ensure_keys(c, B));
         PruneArgs A{};
         A.X = v.X;
         A.ld = v.ld;
@@ -284,13 +326,14 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
         A.B = B;
         A.K = K;
         A.D = D;
-        A.keys = static_cast<unsigned long long *>(c->keys.p);
+        A.keys = keys_of(c);
+        A.left = flags_of(c);
         if (v.n > 0) {
             KC_CUDA(c, launch_max_f32(A, c->num_sms, smem_cap, st_override > 0 ? st_override : c->lb_st,
-                                      chunk_override > 0 ? chunk_override : c->lb_chunk, c->stream));
-            ++c->launches;
+                                      chunk_override > 0 ? chunk_override : c->lb_chunk, c->stream,
+                                      &c->launches));
         }
-        lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B, v.ids, defl, slack, lb, lb_raw, arg);
+        lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B > 2 && D <= 8 ? A.left : nullptr, B, v.ids, defl, slack, lb, lb_raw, arg);
         KC_TRY(after_launch(c, "lower bound finalize"));
     } else {
         KC_TRY(launch_exact_max(c, v, lo, hi, B, K, __builtin_huge_val(), lb, lb_raw, arg));
@@ -305,18 +348,15 @@ kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, 
                                      double *lb, double *lb_raw, int64_t *arg)
 {
     const int D = c->D;
-    if (c->keys.bytes < (size_t)B * 8) {
-        KC_TRY(ensure(c, c->keys, (size_t)B * 8));
-        KC_CUDA(c, cudaMemsetAsync(c->keys.p, 0, c->keys.bytes, c->stream));
-    }
+    KC_TRY(ensure_keys(c, B));
     PruneArgs A{};
     A.lo = lo;
     A.hi = hi;
     A.B = B;
     A.K = c->K;
     A.D = D;
-    A.keys = static_cast<unsigned long long *>(c->keys.p);
-    if (n > 0 && use_stream_f32(B, c->K, D)) {
+    A.keys = keys_of(c);
+    if (n > 0 && use_stream_f32(B, c->K, D, INT64_MAX)) {
         A.X = c->X;
         A.ld = c->ldx;
         A.n = n;
@@ -343,7 +383,7 @@ kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, 
             ++c->launches;
         }
     }
-    lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, B, nullptr, deflate_factor(KC_F32, D),
+    lb_finalize_f32<<<(B + 127) / 128, 128, 0, c->stream>>>(A.keys, nullptr, B, nullptr, deflate_factor(KC_F32, D),
                                                             underflow_slack(KC_F32, D), lb, lb_raw, arg);
     return after_launch(c, "lower bound finalize");
 }
@@ -465,7 +505,7 @@ constexpr int kNoAllocMaxDevices = 64;
 
 // The best key of each node of a call: 32 KiB, held by every GPU that loads the
 // library until the process exits.
-static __device__ __align__(256) unsigned long long g_noalloc_keys[kNoAllocMaxNodes];
+static __device__ __align__(256) unsigned long long g_noalloc_keys[kNoAllocMaxNodes + kMaxLeft / 2];   // (and the flags)
 
 std::atomic<void *> g_noalloc_ptr[kNoAllocMaxDevices];
 
@@ -525,11 +565,12 @@ extern "C" kc_status kc_lower_bounds_noalloc(const float *X, int64_t N, int64_t 
     A.K = K;
     A.D = D;
     A.keys = static_cast<unsigned long long *>(scratch);
+    A.left = reinterpret_cast<int *>(A.keys + B);
     // the keys start from zero whatever an earlier call left (one whose last launch
     // failed): this array has no context that would end with the error
-    if (cudaMemsetAsync(scratch, 0, (size_t)B * 8, st) != cudaSuccess) return KC_ECUDA;
+    if (cudaMemsetAsync(scratch, 0, (size_t)B * 8 + kMaxLeft * 4, st) != cudaSuccess) return KC_ECUDA;
     if (N > 0 && launch_max_f32(A, sms, (size_t)optin, 0, 0, st) != cudaSuccess) return KC_ECUDA;
-    lb_finalize_f32<<<(B + 127) / 128, 128, 0, st>>>(A.keys, B, nullptr, defl, slack, lb_out, lb_raw_out, argmax_out);
+    lb_finalize_f32<<<(B + 127) / 128, 128, 0, st>>>(A.keys, nullptr, B, nullptr, defl, slack, lb_out, lb_raw_out, argmax_out);
     if (cudaGetLastError() != cudaSuccess) return KC_ECUDA;
     return KC_OK;
 }

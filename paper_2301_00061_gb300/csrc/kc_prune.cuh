@@ -14,11 +14,14 @@
 //     involved (difference, maximum, fused multiply-add, sum) is monotone;
 //   node: the distance to the node's own box of that cluster.
 // A warp goes on to the remaining clusters only when some lane passes.  The
-// tests are strict (a value equal to the best is evaluated), so the maximum and
-// the smallest position attaining it are those of the full evaluation, bit for
-// bit; inputs without structure cost a few percent more than evaluating
-// everything (one test per 8 nodes), and 1 / K of it when only the group tests
-// fail.
+// tests dismiss only what cannot win (a value equal to the best is evaluated
+// unless the best one's position lies before the tile), so the maximum and the
+// smallest position attaining it are those of the full evaluation, bit for bit.
+// Where the group tests dismiss nothing, the node tests cost one cluster's
+// evaluation more; at few attributes such batches are left to the streaming kernel
+// after the first group tests (may_leave).  Nodes of bound 0 (each sample in some
+// box): 256 nodes at N = 1e7, D = 8, K = 5 take 8.9 ms, 17.4 when ties passed every
+// test, 12.4 evaluated in full; at N = 1e6, D = 2, K = 4 0.44 ms, 1.19 and 0.43.
 //
 // For the one cluster to be the right one for a whole warp, a CTA sorts each
 // tile of samples by the nearest of K reference points (the box centers of the
@@ -54,7 +57,7 @@ struct PruneArgs {
     int64_t ld, n;
     const void *lo, *hi;      // [B][K][D] in the samples' type
     int B, K, D;
-    int per;                  // nodes per CTA range (blockIdx.y), a multiple of kPG unless B is smaller
+    int per;                  // nodes per CTA range (blockIdx.y)
     const uint32_t *ids;      // NULL, or the names of the samples: keys hold ids[position]
     int vec;                  // rows may be read with 16-byte loads (X 16-byte aligned, ld a multiple of 16 bytes)
     unsigned long long *keys; // [B] (value bits, ~position), zero before the launch
@@ -62,9 +65,16 @@ struct PruneArgs {
     // node in each tile, of all samples that may attain the exact maximum
     float *tmax;              // [B][rows], a row a tile
     int64_t rows;
-    float c1, eps;            // such a sample's float value reaches screen_floor(best, c1, eps)
-    float cut;                // nodes proved to reach this float value are done
-    const double *off;        // [D] double data: subtracted before the conversion to float
+    // screens: a sample that may attain the maximum has a float value that reaches
+    // screen_floor(best, c1, eps); off [D] is subtracted from double data before the
+    // conversion to float.  Bounds: left, NULL or [gx + 1] zeros, says which of the
+    // pruning kernel's gx CTAs (by blockIdx.x) left their samples, tiles of T, to the
+    // streaming kernel, and at [gx] whether any did.  (One struct of the size it
+    // had: with 16 bytes more the streaming kernel took 150 us for 146.)
+    union { float c1; int gx; };
+    union { float eps; int T; };
+    float cut;                // screens: nodes proved to reach this float value are done
+    union { const double *off; int *left; };
 };
 
 // Below this float value a sample cannot attain a maximum whose largest float
@@ -414,13 +424,26 @@ prune_max_kernel(const PruneArgs A)
     __syncthreads();
     for (int i = tid; i < ns * K; i += NT) fs[i] = first_of(sbox + (size_t)(i / K) * KR, i % K);
 
+    uint32_t first = 0u;   // the tile's first position
+    // What a sample of this tile has to reach where the best key is m.  An equal value
+    // wins only at a smaller position: where m's lies before the tile, the next
+    // float above is wanted.  (Nodes of bound 0, and values that many samples attain:
+    // every sample passed every test.)
+    auto thr_of = [&](unsigned long long m) {
+        const float v = floor_of(key_val(m));
+        if constexpr (!TM)
+            if (!A.ids && m != 0ull && key_pos(m) <= first && v < __int_as_float(0x7f800000))
+                return __uint_as_float(__float_as_uint(v) + 1u);
+        return v;
+    };
+
     // raise node b's best value by a warp whose lanes hold keys (0: none)
     auto raise = [&](int b, unsigned long long k) {
         k = warp_max_u64(k);
         if (TM && lane == 0) atomicMax(&tmx[b], (unsigned)(k >> 32));
         if (lane == 0 && k > key[b]) {
             atomicMax(const_cast<unsigned long long *>(&key[b]), k);
-            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(floor_of(key_val(k))));
+            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(thr_of(k)));
         }
         __syncwarp();
     };
@@ -437,7 +460,31 @@ prune_max_kernel(const PruneArgs A)
         if (TM) atomicMax(&tmx[b], __float_as_uint(v));
         if (k > key[b]) {
             atomicMax(const_cast<unsigned long long *>(&key[b]), k);
-            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(floor_of(v)));
+            atomicMax(reinterpret_cast<int *>(const_cast<float *>(&thr[b])), __float_as_int(thr_of(k)));
+        }
+    };
+    // node b, all its clusters, over a strip's samples y (its slots from q0)
+    auto finish = [&](const uint64_t (&y)[ST][P], int q0, int b) {
+        float v[ST];
+        box_dists<ST, P, PT>(y, box + b * KR, v);
+        for (int k = 1; k < K; ++k) {
+            float e[ST];
+            box_dists<ST, P, PT>(y, box + b * KR + k * RW, e);
+#pragma unroll
+            for (int j = 0; j < ST; ++j) v[j] = fminf(v[j], e[j]);
+        }
+        if (!__any_sync(ALL, max_of<ST>(v) >= thr[b])) return;
+        if constexpr (TM) {   // (the position of a screen's key is not used)
+            raise(b, ((unsigned long long)__reduce_max_sync(ALL, __float_as_uint(max_of<ST>(v))) << 32) | 1ull);
+        } else {
+            const unsigned long long cur = key[b];
+            unsigned long long top = 0ull;
+#pragma unroll
+            for (int j = 0; j < ST; ++j) {
+                const unsigned long long q = key_max(v[j], spos[q0 + j * 32 + lane]);
+                top = q > top ? q : top;
+            }
+            if (__any_sync(ALL, top > cur)) raise(b, top > cur ? top : 0ull);
         }
     };
 
@@ -448,6 +495,7 @@ prune_max_kernel(const PruneArgs A)
     bool seed = true;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
         const int64_t s0 = tile * T + (int64_t)tid * ST;
+        first = (uint32_t)(tile * T);
         if (tid < kMaxK) hist[tid] = 0;
         if (tid >= kMaxK && tid < kMaxK + 3) qn[tid - kMaxK] = 0;
         // nearest reference of each sample, and the sample farthest from its reference
@@ -493,7 +541,7 @@ prune_max_kernel(const PruneArgs A)
             unsigned long long m = seed ? 0ull : key[b];
             m = g > m ? g : m;
             key[b] = m;
-            thr[b] = floor_of(key_val(m));
+            thr[b] = thr_of(m);
         }
         // slots of the samples, sorted by reference
         int off[ST];
@@ -512,8 +560,9 @@ prune_max_kernel(const PruneArgs A)
             base[tid] = s;
         }
         if (seed) {
-            // the first tile's farthest samples, against every node
-            const int64_t cp = (int64_t)(uint32_t)cand[lane];
+            // the first tile's farthest samples, against every node (and its first
+            // sample: where no value is larger, none of the tile can win a tie)
+            const int64_t cp = lane == 0 ? tile * T : (int64_t)(uint32_t)cand[lane];
             const uint32_t cid = A.ids ? A.ids[cp] : (uint32_t)cp;
             uint64_t xc[1][P];
 #pragma unroll
@@ -587,8 +636,17 @@ prune_max_kernel(const PruneArgs A)
         const bool more = tile + gridDim.x < tiles;
         if (AHEAD && more) load(s0 + (int64_t)gridDim.x * T, x);
         __syncthreads();
-        const int items = qn[0], pairs = min(qn[1], CAP);
-        for (int it = warp; it < items; it += NWP) {
+        // Where the group tests dismiss little (boxes that differ in every cluster: all
+        // items), tests cost more than they save at few attributes; the streaming kernel
+        // takes this CTA's samples.  (Inputs are one or the other: 0 to 5 % of the
+        // items on nested boxes, all of them on open nodes of a branch and bound.)
+        if (!TM && P <= 4 && A.left && tile == blockIdx.x && 2 * qn[0] > NWP * ng) {
+            if (tid == 0) A.left[blockIdx.x] = A.left[gridDim.x] = 1;
+            return;
+        }
+        const int items = qn[0], pairs = min(qn[1], CAP), units = items + (pairs + 31) / 32;
+        // (strip, group) items: the node tests
+        auto take_item = [&](int it) {
             const uint32_t w = queue[it];
             const int g = (int)(w >> 16), q0 = (int)(w & 0xFFFFu) * 32 * ST, bg = g * kPG, nn = min(kPG, nb - bg);
             uint64_t y[ST][P];
@@ -610,36 +668,19 @@ prune_max_kernel(const PruneArgs A)
                 m |= mi << (i * ST);
             }
             const int c = (int)__reduce_add_sync(ALL, (unsigned)__popc(m));
-            if (c == 0) continue;
+            if (c == 0) return;
             if (c <= CAP / 8 && push_pairs<ST * kPG>(m, c, &qn[2], qc, CAP, [&](int e) {
                     return ((uint32_t)(bg + e / ST) << 16) | (uint32_t)(q0 + (e % ST) * 32 + lane);
                 }))
-                continue;
+                return;
             // many: every cluster of the nodes that have any
             for (int i = 0; i < nn; ++i) {
-                const int b = bg + i;
                 if (!__any_sync(ALL, (m >> (i * ST) & ((1u << ST) - 1u)) != 0u)) continue;
-                float v[ST];
-                box_dists<ST, P, PT>(y, box + b * KR, v);
-                for (int k = 1; k < K; ++k) {
-                    float e[ST];
-                    box_dists<ST, P, PT>(y, box + b * KR + k * RW, e);
-#pragma unroll
-                    for (int j = 0; j < ST; ++j) v[j] = fminf(v[j], e[j]);
-                }
-                const unsigned long long cur = key[b];
-                unsigned long long top = 0ull;
-#pragma unroll
-                for (int j = 0; j < ST; ++j) {
-                    const unsigned long long q = key_max(v[j], spos[q0 + j * 32 + lane]);
-                    top = q > top ? q : top;
-                }
-                if constexpr (TM) raise(b, top);
-                else if (__any_sync(ALL, top > cur)) raise(b, top > cur ? top : 0ull);
+                finish(y, q0, bg + i);
             }
-        }
+        };
         // (group, sample) pairs, one to a lane
-        for (int it = warp * 32; it < pairs; it += NT) {
+        auto take_pairs = [&](int it) {
             const uint32_t w = it + lane < pairs ? qb[it + lane] : ~0u;
             const bool on = w != ~0u;
             const int bg = on ? (int)(w >> 16) * kPG : 0, slot = (int)(w & 0xFFFFu) & (T - 1);
@@ -655,10 +696,9 @@ prune_max_kernel(const PruneArgs A)
                 if (on && bg + i < nb && d[0] >= thr[b]) m |= 1u << i;
             }
             const int c = (int)__reduce_add_sync(ALL, (unsigned)__popc(m));
-            if (c == 0) continue;
-            if (push_pairs<kPG>(m, c, &qn[2], qc, CAP,
-                                [&](int e) { return ((uint32_t)(bg + e) << 16) | (uint32_t)slot; }))
-                continue;
+            if (c == 0 || push_pairs<kPG>(m, c, &qn[2], qc, CAP,
+                                          [&](int e) { return ((uint32_t)(bg + e) << 16) | (uint32_t)slot; }))
+                return;
             for (; m; m &= m - 1) {
                 const int b = bg + __ffs(m) - 1;
                 float v = INF;
@@ -669,24 +709,38 @@ prune_max_kernel(const PruneArgs A)
                 }
                 lift(b, v, spos[slot]);
             }
-        }
-        __syncthreads();
-        // (node, sample) pairs: the minimum over the clusters
-        const int last = min(qn[2], CAP);
-        for (int it = tid; it < last; it += NT) {
-            const uint32_t w = qc[it];
-            if (w == ~0u) continue;
-            const int b = (int)(w >> 16), slot = (int)(w & 0xFFFFu);
-            uint64_t y[1][P];
-#pragma unroll
-            for (int p = 0; p < P; ++p) y[0][p] = stage[(size_t)p * T + slot];
-            float v = INF;
-            for (int k = 0; k < K; ++k) {
-                float d[1];
-                box_dists<1, P, PT>(y, box + b * KR + k * RW, d);
-                v = fminf(v, d[0]);
+        };
+        // The warps take units in turn until none is left or the queue of (node, sample)
+        // pairs fills up, work that queue off one pair to a lane, and go on.  (Pairs that did
+        // not fit were evaluated in place by single lanes, where many samples survive
+        // the group tests.)
+        for (int u = warp;;) {
+            for (; u < units && (u < items || *const_cast<volatile int *>(&qn[2]) < CAP / 2); u += NWP) {
+                if (u < items) take_item(u);
+                else take_pairs((u - items) * 32);
             }
-            lift(b, v, spos[slot]);
+            const bool done = __syncthreads_and(u >= units) != 0;
+            const int last = min(qn[2], CAP);
+            // (node, sample) pairs: the minimum over the clusters
+            for (int it = tid; it < last; it += NT) {
+                const uint32_t w = qc[it];
+                if (w == ~0u) continue;
+                const int b = (int)(w >> 16), slot = (int)(w & 0xFFFFu);
+                uint64_t y[1][P];
+#pragma unroll
+                for (int p = 0; p < P; ++p) y[0][p] = stage[(size_t)p * T + slot];
+                float v = INF;
+                for (int k = 0; k < K; ++k) {
+                    float d[1];
+                    box_dists<1, P, PT>(y, box + b * KR + k * RW, d);
+                    v = fminf(v, d[0]);
+                }
+                lift(b, v, spos[slot]);
+            }
+            if (done) break;
+            __syncthreads();
+            if (tid == 0) qn[2] = 0;
+            __syncthreads();
         }
         if (!AHEAD && more) load(s0 + (int64_t)gridDim.x * T, x);
         __syncthreads();
@@ -744,14 +798,31 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
 // against pruning, us, at 320 MB of samples: D = 8, K = 5, 4 nodes 216 / 283, 8
 // nodes 427 / 386; D = 4, K = 3, 8 nodes 265 / 384, 16 nodes 508 / 515, 32 nodes
 // 1086 / 760; D = 2, K = 4 (160 MB), 16 nodes 363 / 508, 32 nodes 808 / 678.
+// With n <= kStreamSmall terms in all it is taken for any batch at D <= 8: the chip is
+// not filled long enough for the sort to pay (1e5 samples, D = 4, K = 3, 64 nodes: 22 us
+// against 49 without structure, 20 with nested boxes; 3e8 terms, 256 nodes: 65 against
+// 117 and 39).
 constexpr int kStreamTerms = 208, kStreamCols = 16;
-inline bool use_stream_f32(int B, int K, int D)
+constexpr double kStreamSmall = 1e8;
+inline bool use_stream_f32(int B, int K, int D, int64_t n)
 {
-    return (D <= 8 && B * K * D <= kStreamTerms) || (B <= 2 && B * K <= kStreamCols);
+    return (D <= 8 && ((int64_t)B * K * D <= kStreamTerms || ((double)n * B * K * D <= kStreamSmall && B < 65536))) ||
+           (B <= 2 && B * K <= kStreamCols);
 }
-cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream);
+// Batches whose unstructured form the pruning kernel leaves to the streaming one
+// (PruneArgs::left): at few attributes full evaluation is cheaper than tests that
+// dismiss nothing (open nodes of a branch and bound over 1e6 samples, pruned / full /
+// pruned until the first group tests and then full, us: D = 2, K = 3, 64 nodes 224 /
+// 98 / 115; D = 4 220 / 140 / 152); at D = 5 to 8 up to 32 nodes (D = 8, K = 5, 16
+// nodes 120 / 93 / 107; 64 nodes 244 / 333) or where a CTA has one tile (1e5 samples,
+// 64 nodes 72 / 48).
+inline bool may_leave(int B, int D, bool one_tile)
+{
+    return B > 2 && B < 65536 && (D <= 4 || (D <= 8 && (B <= 32 || one_tile)));
+}
+cudaError_t launch_stream_f32(PruneArgs A, int sms, cudaStream_t stream);
 // The same over the samples A.ids[0 .. A.n) of the rows A.X (D <= 8).
-cudaError_t launch_stream_gather_f32(const PruneArgs &A, int sms, cudaStream_t stream);
+cudaError_t launch_stream_gather_f32(PruneArgs A, int sms, cudaStream_t stream);
 constexpr int kStreamTile = 128;   // samples of a tmax row of the streaming screen
 
 }  // namespace kc

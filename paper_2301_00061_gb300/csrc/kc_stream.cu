@@ -95,6 +95,19 @@ __device__ __forceinline__ void stream_boxes(const PruneArgs &A, ulonglong2 *box
         box[i] = make_ulonglong2(pk(lo[i], lo[i]), pk(hi[i], hi[i]));
 }
 
+// The arguments of node range blockIdx.y.
+__device__ __forceinline__ PruneArgs node_range(PruneArgs A)
+{
+    const int b0 = blockIdx.y * A.per;
+    const size_t o = (size_t)b0 * A.K * A.D;
+    A.lo = static_cast<const float *>(A.lo) + o;
+    A.hi = static_cast<const float *>(A.hi) + o;
+    A.B = min(A.per, A.B - b0);
+    A.keys += b0;
+    if (A.tmax) A.tmax += b0 * A.rows;
+    return A;
+}
+
 __device__ __forceinline__ void stream_finish(const PruneArgs &A, int b, unsigned long long k, unsigned long long *red)
 {
     k = warp_max_u64(k);
@@ -111,10 +124,13 @@ __device__ __forceinline__ void stream_finish(const PruneArgs &A, int b, unsigne
 // K fixed, the loop over the clusters unrolled; 0: any K, about 8 % slower).
 // MANY (more than two nodes): each warp keeps its nodes' keys in shared memory
 // and reduces over its lanes only when one of them may beat the key.
+// A CTA takes a range of the nodes (blockIdx.y) where there may be more than two.
 template <int DC, int KC, int Q, int CTAS, bool MANY, bool TM, bool GATHER = false>
 __global__ void __launch_bounds__(kThreads, CTAS)
-stream_max_small(const PruneArgs A)
+stream_max_small(const PruneArgs all)
 {
+    const PruneArgs A = MANY || TM ? node_range(all) : all;
+    if (MANY && !GATHER && A.left && A.left[A.gx] == 0) return;
     constexpr int ST = 4 * Q, NWP = kThreads / 32;
     extern __shared__ __align__(16) unsigned char smem[];
     ulonglong2 *box = reinterpret_cast<ulonglong2 *>(smem);   // [B * K][DC]
@@ -129,6 +145,12 @@ stream_max_small(const PruneArgs A)
     const int K = KC ? KC : A.K;
     StreamBest best0, best1;
     for (int64_t base = (int64_t)blockIdx.x * (kThreads * ST); base < A.n; base += (int64_t)gridDim.x * (kThreads * ST)) {
+        if (MANY && !GATHER && A.left) {
+            // only what the pruning kernel left: its tiles of A.T, dealt to A.gx CTAs
+            bool some = false;
+            for (int64_t t = base / A.T; t <= (base + kThreads * ST - 1) / A.T; ++t) some |= A.left[t % A.gx] != 0;
+            if (!some) continue;
+        }
         // quad q of a thread: samples base + (q kThreads + tid) 4 ..
         const int64_t s0 = base + (int64_t)threadIdx.x * 4;
         uint64_t x[Q][DC][2];
@@ -373,27 +395,40 @@ StreamKernel wide_kernel_of(int cols)
 
 }  // namespace
 
-cudaError_t launch_stream_f32(const PruneArgs &A, int sms, cudaStream_t stream)
+cudaError_t launch_stream_f32(PruneArgs A, int sms, cudaStream_t stream)
 {
     const bool tm = A.tmax != nullptr;
-    const int cols = A.B * A.K, Q = A.D <= 4 && !tm ? 2 : 1;
-    size_t smem = (size_t)cols * A.D * 16;   // at most 32 KB for both forms
-    StreamKernel fn = tm ? wide_kernel_of<true>(cols) : wide_kernel_of<false>(cols);
-    if (A.D <= 8) {
-        fn = small_kernel_of(A.D, A.K, A.B > 2, tm);
-        smem += (size_t)kThreads / 32 * A.B * 8;
+    const int Q = A.D <= 4 && !tm ? 2 : 1;
+    const int64_t tiles = (A.n + kThreads * 4 * Q - 1) / (kThreads * 4 * Q);
+    const size_t node = (size_t)A.K * A.D * 16 + (A.D <= 8 ? kThreads / 32 * 8 : 0);
+    // node ranges so that the last round of CTAs leaves little idle (three CTAs an SM
+    // are resident; loading a tile again costs about two nodes' evaluation)
+    int per = A.B;
+    if (A.D <= 8 && A.B > 2) {
+        const int64_t slots = 3 * (int64_t)sms;
+        int64_t best = INT64_MAX;
+        for (int64_t r = 1; r <= A.B && (r - 1) * tiles < 8 * slots; ++r) {
+            const int64_t nodes = (A.B + r - 1) / r, cost = (tiles * r + slots - 1) / slots * (2 + nodes);
+            if (cost < best) { best = cost; per = (int)nodes; }
+        }
     }
+    per = (int)std::min<int64_t>(per, 46 * 1024 / node);   // (a launch's limit without opting in)
+    A.per = per;
+    const size_t smem = per * node;
+    const StreamKernel fn = A.D <= 8 ? small_kernel_of(A.D, A.K, A.B > 2, tm)
+                          : tm ? wide_kernel_of<true>(A.B * A.K) : wide_kernel_of<false>(A.B * A.K);
     int per_sm = 0;
     const cudaError_t r = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem);
     if (r != cudaSuccess) return r;
-    const int64_t tiles = (A.n + kThreads * 4 * Q - 1) / (kThreads * 4 * Q);
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)std::max(1, per_sm) * sms));
+    const dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)std::max(1, per_sm) * sms)),
+                    (unsigned)((A.B + per - 1) / per));
     fn<<<grid, kThreads, smem, stream>>>(A);
     return cudaGetLastError();
 }
 
-cudaError_t launch_stream_gather_f32(const PruneArgs &A, int sms, cudaStream_t stream)
+cudaError_t launch_stream_gather_f32(PruneArgs A, int sms, cudaStream_t stream)
 {
+    A.per = A.B;
     const int Q = A.D <= 2 ? 2 : 1;
     const size_t smem = (size_t)A.B * A.K * A.D * 16 + (size_t)kThreads / 32 * A.B * 8;
     const StreamKernel fn = gather_kernel_of(A.D);
