@@ -343,6 +343,23 @@ static double exact_screen_gamma(int D)
 
 namespace {
 
+// The screen of B nodes over n samples: the streaming kernel or e.
+struct ScreenPlan {
+    bool stream;
+    const PruneEntry *e;
+    int T;   // samples of a tmax row
+};
+ScreenPlan screen_plan(const kc_ctx *c, int64_t n, int B, int K)
+{
+    const bool f64 = c->dt == KC_F64;
+    ScreenPlan p;
+    p.e = f64 ? prune_pick(prune_table<true, true>(), c->D, n, c->num_sms, 0)
+              : prune_pick(prune_table<false, true>(), c->D, n, c->num_sms, 0);
+    p.stream = !f64 && use_stream_f32(B, K, c->D, n);
+    p.T = p.stream ? kStreamTile : p.e->T;
+    return p;
+}
+
 kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *hi, int B, int K, double cut, double *lb,
                           double *val, int64_t *arg)
 {
@@ -400,16 +417,14 @@ kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *
             }
             const double cf = cut * (1.0 + gam) * (1.0 + 1e-6);   // a float value this large proves the cut
             A.cut = cf < 3e38 ? (float)cf : __builtin_huge_valf();
-            const PruneEntry *e = f64 ? prune_pick(prune_table<true, true>(), D, v.n, c->num_sms, 0)
-                                      : prune_pick(prune_table<false, true>(), D, v.n, c->num_sms, 0);
-            const bool stream = !f64 && use_stream_f32(B, K, D, v.n);
-            H.T = stream ? kStreamTile : e->T;
+            const ScreenPlan plan = screen_plan(c, v.n, B, K);
+            H.T = plan.T;
             const int64_t rows = (v.n + H.T - 1) / H.T;
             KC_TRY(ensure(c, c->tmax, (size_t)rows * B * 4));
             A.tmax = static_cast<float *>(c->tmax.p);
             A.rows = rows;
-            if (stream) KC_CUDA(c, launch_stream_f32(A, c->num_sms, c->stream));
-            else KC_CUDA(c, prune_run(e, A, true, c->num_sms, c->smem_optin > 0 ? c->smem_optin : 48 * 1024, 0, c->stream));
+            if (plan.stream) KC_CUDA(c, launch_stream_f32(A, c->num_sms, c->stream));
+            else KC_CUDA(c, prune_run(plan.e, A, true, c->num_sms, c->smem_optin > 0 ? c->smem_optin : 48 * 1024, 0, c->stream));
             ++c->launches;
             H.gam = f64 ? -1.0 : gam;
             H.cut = cut;
@@ -440,10 +455,15 @@ kc_status exact_max_chunk(kc_ctx *c, const View &v, const void *lo, const void *
 kc_status launch_exact_max(kc_ctx *c, const View &v, const void *lo, const void *hi, int B, int K, double cut, double *lb,
                            double *val, int64_t *arg)
 {
-    // batches whose tile maxima (one float per node and 512 samples or so) stay
-    // within 256 MiB
-    const int64_t rows = v.n / 512 + 1;
-    const int step = (int)std::max<int64_t>(16, std::min<int64_t>(B, ((int64_t)64 << 20) / rows / 8 * 8));
+    // batches whose tile maxima (one float per node and tile of the kernel that runs)
+    // stay within 256 MiB; at most 65528 nodes, so that a launch's node ranges never
+    // exceed its grid.  (N < 2^32 and tiles of at least 128 samples: at least one node.)
+    const auto most = [&](int tile) {
+        const int64_t s = ((int64_t)64 << 20) / ((v.n + tile - 1) / tile + 1);
+        return (int)std::min<int64_t>({B, 65528, s >= 8 ? s / 8 * 8 : std::max<int64_t>(1, s)});
+    };
+    int step = most(screen_plan(c, v.n, B, K).T);
+    if (step < B) step = std::min(step, most(screen_plan(c, v.n, step, K).T));   // (fewer nodes may be streamed)
     const size_t box = (size_t)K * c->D * c->esize;
     for (int b0 = 0; b0 < B; b0 += step)
         KC_TRY(exact_max_chunk(c, v, static_cast<const char *>(lo) + b0 * box, static_cast<const char *>(hi) + b0 * box,

@@ -254,7 +254,7 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
 {
     const int64_t tiles = (A.n + e->T - 1) / e->T;
     const auto bytes = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32, tm).end; };
-    int per = A.B;
+    int per = std::min(A.B, 1 << 16);
     if (chunk > 0 && chunk < per) per = chunk;
     if (tiles < 4 * (int64_t)sms) {
         // few tiles: node ranges (whole groups) so that the last round of CTAs leaves
@@ -268,7 +268,15 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
             if (cost < best) { best = cost; per = (int)nodes; }
         }
     }
-    while (per > 1 && bytes(per) > smem_cap) per = per > 2 * kPG ? (per - 1) / kPG * kPG : per - 1;
+    if (bytes(per) > smem_cap) {
+        // as many nodes as fit, whole groups where there is more than one
+        int fits = 0;   // (bytes(fits) <= smem_cap < bytes(per))
+        while (per - fits > 1) {
+            const int mid = fits + (per - fits) / 2;
+            (bytes(mid) > smem_cap ? per : fits) = mid;
+        }
+        per = std::max(1, fits > kPG ? fits / kPG * kPG : fits);
+    }
     A.per = per;
     const size_t smem = bytes(per);
     if (smem > smem_cap) return cudaErrorInvalidConfiguration;
@@ -287,7 +295,7 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
     // at most 65535 node ranges to a launch
     const int B = A.B, step = (int)std::min<int64_t>((int64_t)per * 65535, B);
     const size_t box = (size_t)A.K * A.D * (tm && A.off ? 8 : 4);
-    if (tm && step < B) return cudaErrorInvalidConfiguration;   // (screens come in batches far smaller)
+    if (tm && step < B) return cudaErrorInvalidConfiguration;   // (screens come in smaller batches)
     for (int b0 = 0; b0 < B; b0 += step) {
         PruneArgs C = A;
         C.B = std::min(step, B - b0);
