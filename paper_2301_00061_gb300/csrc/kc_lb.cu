@@ -256,13 +256,14 @@ cudaError_t prune_run(const PruneEntry *e, PruneArgs A, bool tm, int sms, size_t
     const auto bytes = [&](int nb) { return PruneLayout(nb, A.K, e->P, e->T, e->NT / 32, tm).end; };
     int per = std::min(A.B, 1 << 16);
     if (chunk > 0 && chunk < per) per = chunk;
-    if (tiles < 4 * (int64_t)sms) {
+    if (tiles < sms) {
         // few tiles: node ranges (whole groups) so that the last round of CTAs leaves
         // little idle; a range repeats the sort of its tile, about 16 nodes' worth (1e5
-        // samples, D = 8, K = 5, 256 nodes: 280 us in one range, 212 in three)
+        // samples, D = 8, K = 5, 256 nodes: 280 us in one range, 212 in three; with more tiles than SMs
+        // a second range cost up to 16 %)
         int64_t best = INT64_MAX;
         const int most = per;
-        for (int64_t r = 1; r <= 4 * (int64_t)sms / tiles + 1 && r <= (A.B + kPG - 1) / kPG; ++r) {
+        for (int64_t r = 1; r <= 4 * (int64_t)sms / tiles && r <= (A.B + kPG - 1) / kPG; ++r) {
             const int64_t nodes = std::min<int64_t>(most, ((A.B + r - 1) / r + kPG - 1) / kPG * kPG);
             const int64_t ranges = (A.B + nodes - 1) / nodes, cost = (tiles * ranges + sms - 1) / sms * (16 + nodes);
             if (cost < best) { best = cost; per = (int)nodes; }
