@@ -175,7 +175,7 @@ __global__ void lb_finalize_f64(const double *__restrict__ pval, const uint32_t 
     }
 }
 
-constexpr int64_t kSubsetChunk = (int64_t)1 << 25;
+constexpr int64_t kSubsetBytes = (int64_t)128 << 20;   // of gathered rows at a time
 
 // Rows of the samples named by ids: out[a * ldo + i] = X[a * ld + ids[i]].
 __global__ void __launch_bounds__(256)
@@ -352,7 +352,8 @@ kc_status launch_lower_bounds_cfg(kc_ctx *c, const View &v, const void *lo, cons
 
 // Float bounds of B nodes over the samples named by ids [n] (device, D <= 8,
 // every id below N): few nodes gather as they stream, batches gather the samples
-// into rows of their own first (at most kSubsetChunk at a time) and prune.
+// into rows of their own first (at most kSubsetBytes at a time, less where the device
+// has no room for that) and prune.
 kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, const void *lo, const void *hi, int B,
                                      double *lb, double *lb_raw, int64_t *arg)
 {
@@ -374,8 +375,15 @@ kc_status launch_lower_bounds_subset(kc_ctx *c, const uint32_t *ids, int64_t n, 
         KC_CUDA(c, launch_stream_gather_f32(A, c->num_sms, c->stream));
         ++c->launches;
     } else if (n > 0) {
-        const int64_t chunk = std::min(n, kSubsetChunk), ld = (chunk + 63) / 64 * 64;
-        KC_TRY(ensure(c, c->work2, (size_t)ld * D * 4));
+        int64_t chunk = std::min<int64_t>(n, kSubsetBytes / (4 * D) / 64 * 64), ld = 0;
+        const std::string err = c->err;
+        for (;; chunk = (chunk + 1) / 2) {
+            ld = (chunk + 63) / 64 * 64;
+            const kc_status st = ensure(c, c->work2, (size_t)ld * D * 4);
+            if (st == KC_OK) break;
+            if (st != KC_ENOMEM || chunk <= 4096) return st;
+        }
+        c->err = err;
         for (int64_t i0 = 0; i0 < n; i0 += chunk) {
             const int64_t m = std::min(chunk, n - i0);
             const int grid = (int)std::min<int64_t>((m + 1023) / 1024, (int64_t)c->num_sms * 8);
