@@ -152,10 +152,12 @@ kc_status kc_lower_bounds_noalloc(const float *X, int64_t N, int64_t ld, int32_t
  * kc_autotune -- picks the launch shape of the float lower-bound kernel
  * (samples per thread, nodes per CTA: occupancy against extra passes over
  * the samples) by timing each candidate with CUDA events on the given batch
- * of B nodes (lo, hi as in kc_lower_bounds), and keeps the fastest for later
+ * of B nodes (lo, hi as in kc_lower_bounds), and keeps one that is faster than
+ * the choice by size (by more than 3 %, the noise of equal launches) for later
  * kc_lower_bounds calls on this context.  Outputs (host, each may be NULL):
  * the chosen samples per thread, nodes per launch, and its time per batch in
- * ms.  Double data: nothing to tune (outputs 0).  A scheduling choice; the
+ * ms.  Nothing to tune: double data (outputs 0), and batches so small that
+ * every term is evaluated (the time; the other outputs 0).  A scheduling choice; the
  * paper has no counterpart (the bound itself is Section 3.1's).
  */
 kc_status kc_autotune(kc_ctx *ctx, const void *lo, const void *hi, int32_t B, int32_t *samples_per_thread_out,

@@ -462,9 +462,10 @@ kc_status launch_lower_bounds_refine(kc_ctx *c, const View &v, const void *lo, c
     return KC_OK;
 }
 
-// Times the float lower-bound kernel's launch shapes on the given node batch
-// (samples per thread x nodes per CTA: occupancy against extra sample passes)
-// and keeps the fastest in the context.  Untimed work for the caller.
+// Times the launch shapes of the pruning kernel on the given node batch (samples
+// per thread, where both exist, x nodes per CTA, whole groups) against the choice by
+// size, and keeps one that is faster by more than timing noise in the context.
+// Untimed work for the caller.
 kc_status autotune_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B, double *lb_scratch, int *st_out,
                                 int *chunk_out, float *ms_out)
 {
@@ -472,37 +473,55 @@ kc_status autotune_lower_bounds(kc_ctx *c, const void *lo, const void *hi, int B
     *chunk_out = 0;
     if (c->dt != KC_F32 || B <= 0) return KC_OK;
     const View v = full_view(c);
-    const int chunks[4] = {B, (B + 1) / 2, (B + 2) / 3, (B + 3) / 4};
-    const int sts[2] = {4, 2};
+    const int D = c->D;
+    const auto groups = [](int nodes) { return (nodes + kPG - 1) / kPG * kPG; };
+    struct Shape {
+        int st, chunk;
+    };
+    std::vector<Shape> shapes{{0, 0}};   // by size
+    const bool fixed = use_stream_f32(B, c->K, D, v.n);   // evaluated in full: nothing to choose
+    if (!fixed)
+        for (int st : {4, 2}) {
+            if (D > 8 && st == 2) break;   // one kernel
+            for (int part = 1; part <= 4; ++part) {
+                const int chunk = part == 1 ? B : groups((B + part - 1) / part);
+                if (part == 1 || (chunk < B && chunk != shapes.back().chunk)) shapes.push_back({st, chunk});
+            }
+        }
     cudaEvent_t e0, e1;
     KC_CUDA(c, cudaEventCreate(&e0));
-    KC_CUDA(c, cudaEventCreate(&e1));
-    float best = 3.4e38f;
-    int bst = 4, bch = 0;
+    if (cudaEventCreate(&e1) != cudaSuccess) {
+        cudaEventDestroy(e0);
+        return set_err(c, KC_ECUDA, "autotune: cudaEventCreate failed");
+    }
+    c->lb_st = c->lb_chunk = 0;
+    float best = 0.f, limit = 0.f;
+    Shape pick = shapes[0];
     kc_status st = KC_OK;
-    for (int si = 0; si < 2 && st == KC_OK; ++si)
-        for (int ci = 0; ci < 4 && st == KC_OK; ++ci) {
-            const int ch = chunks[ci];
-            if (ci > 0 && ch == chunks[ci - 1]) continue;
-            st = launch_lower_bounds_cfg(c, v, lo, hi, B, lb_scratch, nullptr, nullptr, sts[si], ch);
-            if (st != KC_OK) break;
-            cudaEventRecord(e0, c->stream);
-            for (int r = 0; r < 3 && st == KC_OK; ++r)
-                st = launch_lower_bounds_cfg(c, v, lo, hi, B, lb_scratch, nullptr, nullptr, sts[si], ch);
-            cudaEventRecord(e1, c->stream);
-            if (cudaEventSynchronize(e1) != cudaSuccess) { st = set_err(c, KC_ECUDA, "autotune: event sync failed"); break; }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, e0, e1);
-            ms /= 3.f;
-            if (ms < best) { best = ms; bst = sts[si]; bch = ch; }
-        }
+    for (const Shape &s : shapes) {
+        st = launch_lower_bounds_cfg(c, v, lo, hi, B, lb_scratch, nullptr, nullptr, s.st, s.chunk);
+        cudaEventRecord(e0, c->stream);
+        for (int r = 0; r < 3 && st == KC_OK; ++r)
+            st = launch_lower_bounds_cfg(c, v, lo, hi, B, lb_scratch, nullptr, nullptr, s.st, s.chunk);
+        cudaEventRecord(e1, c->stream);
+        if (st == KC_OK && cudaEventSynchronize(e1) != cudaSuccess) st = set_err(c, KC_ECUDA, "autotune: event sync failed");
+        if (st != KC_OK) break;
+        float ms = 0.f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= 3.f;
+        // (equal launches differ by less)
+        if (&s == &shapes[0]) limit = 0.97f * (best = ms);
+        else if (ms < limit && ms < best) { best = ms; pick = s; }
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != KC_OK) return st;
-    c->lb_st = bst;
-    c->lb_chunk = bch;
-    *st_out = bst;
-    *chunk_out = bch;
+    c->lb_st = D <= 8 ? pick.st : 0;
+    c->lb_chunk = pick.chunk;
+    if (!fixed) {
+        *st_out = prune_pick(prune_table<false, false>(), D, v.n, c->num_sms, pick.st)->ST;
+        *chunk_out = pick.chunk > 0 ? pick.chunk : B;
+    }
     *ms_out = best;
     return KC_OK;
 }
