@@ -327,10 +327,9 @@ __global__ void exact_finalize_kernel(unsigned long long *__restrict__ keys, ulo
 }
 
 // Up to this many node x sample x cluster x attribute terms double data are
-// evaluated directly.  Bounds, direct against screened, us: 0.1e6 terms 19 / 123,
-// 1.9e6 43 / 358, 2.9e6 (D = 12) 61 / 173, 3.8e6 71 / 195, 19e6 305 / 74 (small sets
-// leave much of the screen within its band, in one CTA's tile).
-constexpr double kDirectTerms = 6e6;
+// evaluated directly.  Bounds, direct against screened, us: 0.1e6 terms 20 / 31, 1.9e6
+// 36 / 37, 2.9e6 (D = 12) 61 / 65, 3.8e6 64 / 37, 7.7e6 117 / 41, 19e6 267 / 41.
+constexpr double kDirectTerms = 3e6;
 
 using DirectFn = void (*)(const double *, int64_t, int64_t, const double *, const double *, int, int, int, int, ulonglong2 *);
 
