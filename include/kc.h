@@ -18,7 +18,9 @@
  *
  * Pointers.  Every array argument may be host memory (pageable or pinned) or
  * device memory of the context's GPU; the library checks which with
- * cudaPointerGetAttributes and stages host arrays through its own buffers.
+ * cudaPointerGetAttributes and stages host arrays through its own buffers
+ * (kc_create reads row-major rows in pinned memory where they are, when their
+ * address is a multiple of the element size).
  * Calls are ordered on the context's stream.  A call whose outputs are all in
  * device memory returns without waiting for the GPU; a call with any output in
  * host memory returns after the results are written.
@@ -134,8 +136,8 @@ kc_status kc_lower_bounds(kc_ctx *ctx, const void *lo, const void *hi, int32_t B
  * call returns KC_ECUDA at once, launches nothing and leaves that error in
  * place for its owner.
  * Scratch is one fixed array in the library (the best value of each of 4096
- * nodes, 32 KiB, kept by every GPU that loads the library until the process
- * exits); B may be at most 4096 (larger B returns KC_EINVAL).  The first call on
+ * nodes and 256 flags, 33 KiB, kept by every GPU that loads the library until the
+ * process exits; each call clears what it uses); B may be at most 4096 (larger B returns KC_EINVAL).  The first call on
  * a device looks up the array's device address with that device current and
  * keeps it for the process; make that first call before any stream capture, and do not call
  * the entry point on a device after cudaDeviceReset (the kept address would

@@ -539,8 +539,8 @@ namespace {
 constexpr int kNoAllocMaxNodes = 4096;    // nodes per call
 constexpr int kNoAllocMaxDevices = 64;
 
-// The best key of each node of a call: 32 KiB, held by every GPU that loads the
-// library until the process exits.
+// The best key of each node of a call and the flags: 33 KiB, held by every GPU
+// that loads the library until the process exits.
 static __device__ __align__(256) unsigned long long g_noalloc_keys[kNoAllocMaxNodes + kMaxLeft / 2];   // (and the flags)
 
 std::atomic<void *> g_noalloc_ptr[kNoAllocMaxDevices];

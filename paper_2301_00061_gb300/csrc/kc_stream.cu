@@ -121,7 +121,9 @@ __device__ __forceinline__ void stream_finish(const PruneArgs &A, int b, unsigne
 }
 
 // D = DC <= 8 attributes: 4 Q samples in registers, two clusters at a time (KC:
-// K fixed, the loop over the clusters unrolled; 0: any K, about 8 % slower).
+// K fixed, the loop over the clusters unrolled; 0: any K, about 8 % slower).  K = 3, 4
+// and 5 are the cluster counts of the package's workloads; another one would be 24
+// kernels more to compile, and a gather's latency hides the loop (no fixed K there).
 // MANY (more than two nodes): each warp keeps its nodes' keys in shared memory
 // and reduces over its lanes only when one of them may beat the key.
 // A CTA takes a range of the nodes (blockIdx.y) where there may be more than two.

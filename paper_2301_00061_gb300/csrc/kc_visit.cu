@@ -46,7 +46,7 @@ struct Key<float> {
     __device__ static float vmax(const K &k) { return unord_f32((uint32_t)(k >> 32)); }
     __device__ static float vmin(const K &k) { return unord_f32(~(uint32_t)(k >> 32)); }
     __device__ static uint32_t pos(const K &k) { return 0xFFFFFFFFu - (uint32_t)k; }
-    __device__ static void atomic_max(K *p, const K &v, unsigned *) { atomicMax(p, v); }
+    __device__ static void atomic_max(K *p, const K &v) { atomicMax(p, v); }
 };
 
 struct __align__(16) K128 {
@@ -69,7 +69,7 @@ struct Key<double> {
     __device__ static double vmin(const K &k) { return unord_f64(~k.hi); }
     __device__ static uint32_t pos(const K &k) { return (uint32_t)(0xFFFFFFFFull - k.lo); }
     // 128-bit compare-and-swap; a key read as equal or larger costs one exchange
-    __device__ static void atomic_max(K *p, const K &v, unsigned *)
+    __device__ static void atomic_max(K *p, const K &v)
     {
         raise_key128(reinterpret_cast<ulonglong2 *>(p), v.hi, v.lo);
     }
@@ -402,7 +402,7 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
         if (top >= 0.f) acc_lb = KT::max_of(top, top_pos);
     }
     acc_lb = warp_kmax<T>(acc_lb);
-    if (lane == 0 && !KT::is_none(acc_lb)) KT::atomic_max(&lbkey[b], acc_lb, &flags[b]);
+    if (lane == 0 && !KT::is_none(acc_lb)) KT::atomic_max(&lbkey[b], acc_lb);
     if constexpr (!F32) {
         // one key to a lane: their exchanges overlap
         KY own = KT::none();
@@ -420,7 +420,7 @@ __device__ __forceinline__ void pass_a_node(const uint64_t *tp, const double *td
                     i += 2;
                 }
         static_assert(2 * KM * DM <= 32 || F32, "one key to a lane");
-        if (at && !KT::is_none(own)) KT::atomic_max(at, own, &flags[b]);
+        if (at && !KT::is_none(own)) KT::atomic_max(at, own);
     }
     if (__any_sync(0xffffffffu, infeasible) && lane == 0) atomicOr(&flags[b], 1u);
     if constexpr (F32) {
@@ -774,7 +774,6 @@ struct PBSlot<float, KM, DM> {
     unsigned jmax[KM][DM], jmin[KM][DM]; // bbox of the sample-based assigned samples
 };
 
-__device__ __forceinline__ unsigned to_ord(float v) { return ord_f32(v); }
 __device__ __forceinline__ unsigned long long to_ord(double v) { return ord_f64(v); }
 
 // Words of one staged representative: float data packs coordinate pairs
@@ -973,7 +972,7 @@ __device__ __forceinline__ void pass_b_node(const double *tx, int tile, int tn, 
             const KY cd = warp_kmax<T>(c_cand[k]);
             const size_t ok_ = (size_t)b * K + k;
             if (lane == 0 && cn) atomicAdd(&cnt[ok_], cn);
-            if (lane == 0 && !KT::is_none(cd)) KT::atomic_max(&cand[ok_], cd, &flags[b]);
+            if (lane == 0 && !KT::is_none(cd)) KT::atomic_max(&cand[ok_], cd);
         }
     __syncwarp();
     for (int i = lane; i < K * D; i += 32) {
@@ -1294,7 +1293,7 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, unsigned l
     uint32_t *lists = reinterpret_cast<uint32_t *>(tx + (size_t)D * tile);      // [warps][kSub]
     auto *slots = reinterpret_cast<PBSlot<T, KM, DM> *>(lists + NWV * kSub);   // [warps]
     uint32_t *tids = reinterpret_cast<uint32_t *>(slots + NWV);                 // [tile]
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int warp = threadIdx.x >> 5;
     uint32_t *list = lists + warp * kSub;
     // [warps][KM][RM][words] after the ids (tile is a multiple of 32)
     uint64_t *wrep = reinterpret_cast<uint64_t *>(tids + tile) + (size_t)warp * KM * RM * rep_words<T, DM>();
@@ -1328,7 +1327,6 @@ visit_b_list_kernel(const T *__restrict__ X, int64_t ld, ListBatch L, unsigned l
                 pass_b_node<KM, DM>(tx, tile, tn, (warp % wpt) * 32, wpt * 32, tids, nullptr, 0, list,
                                        slots + warp, wrep, nd, K, D, RM, lo_in, hi_in, blo, bhi, repx, nreps, allhave,
                                        ball, alpha, mg, seed_id, cnt, smax, smin, jmax, jmin, cand, flags);
-        (void)lane;
     }
 }
 

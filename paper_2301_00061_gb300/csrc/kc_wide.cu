@@ -672,7 +672,7 @@ static int wide_split(const kc_ctx *c, int64_t tiles, int B)
 }
 
 // Pass A and pass B of the wide path on the context's stream; the caller
-// (tighten_common in kc_visit.cu) owns the workspace and the finalize kernels.
+// (tighten_wide in kc_visit.cu) owns the workspace and the finalize kernels.
 kc_status launch_wide_a(kc_ctx *c, const View &v, const ListBatch *L, const float *lo, const float *hi, int B,
                         const Margins &mg, unsigned long long *lbkey, unsigned long long *amax,
                         unsigned long long *amin, unsigned *flags, int ndir, unsigned long long *dmax,
